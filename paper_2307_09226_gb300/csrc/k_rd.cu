@@ -12,130 +12,263 @@
 // v = -d_s lambda / (2 T_slow L).  With the static-clutter option the d = 0 column is
 // left out of the search (a zero-Doppler notch).
 //
-// Three kernels, all deterministic:
-//   fft_rows   - eight (frame, channel, n) rows per CTA: radix-2 FFT over l in shared memory;
-//   fft_cols   - one CTA per (frame, 16 Doppler columns): per channel, radix-2 FFT over
-//                n of the 16 columns, |X|^2 added into a shared-memory tile in channel order;
+// Three kernels, all deterministic, each instantiated for its FFT length:
+//   fft_rows   - FFT over l of the (channel, n) rows;
+//   fft_cols   - one CTA per (frame, 8 Doppler columns): FFT over n, channel by channel,
+//                |X|^2 summed over the channels in registers;
 //   rd_argmax  - one CTA per frame: the largest power (first index on ties) -> velocity.
 // FFT lengths are powers of two up to 1024 (N_s) and 1024 (L).
-#include <vector>
+//
+// The work is bound by memory (the cube is read once, its row transform written and read
+// once), so a transform touches shared memory only between passes: every thread holds 16
+// values and takes radix-16 (or shorter, last) butterflies in registers, Stockham order,
+// two passes up to 256 points.  On 64 cubes of V = 12, N_s = 256, L = 128 (201 MB):
+// radix-2 stages in shared memory with a sine and cosine per butterfly took 638 us (rows),
+// 521 us (columns) and 70 us (maximum), 1.20 ms a call; these kernels take 0.124 ms a call.
+#include <algorithm>
 
+#include "fft_regs.h"
 #include "rsim_ctx.h"
 #include "rsim_internal.h"
 
 namespace rsim {
 namespace {
 
-constexpr int kColBlock = 16;
+constexpr int kRdCols = 8;          // Doppler columns per CTA: a 64-byte run of every row
+constexpr int kRdThreads = 256;     // row kernel, and the column kernel of many frames
+constexpr int kRdThreadsMax = 512;  // column kernel when few frames leave SMs idle
+constexpr int kRdByValue = 64;      // cube pointers passed in the kernel's arguments
 
-__device__ __forceinline__ unsigned bitrev(unsigned x, int bits) { return __brev(x) >> (32 - bits); }
+// FFT of N = 2^k points, 2 <= N <= 1024: a thread holds PER values and T threads share a
+// sequence.  Pass 1 has radix PER; the second radix R2 and the third R3 (1: no such pass).
+template <int N>
+struct FftShape {
+  static constexpr int PER = N < 16 ? N : 16;
+  static constexpr int T = N / PER;
+  static constexpr int R2 = N <= 16 ? 1 : (N <= 256 ? N / 16 : 16);
+  static constexpr int R3 = N <= 256 ? 1 : N / 256;
+  static constexpr int RL = R3 > 1 ? R3 : (R2 > 1 ? R2 : PER);  // radix of the last pass
+  static constexpr int kTw2 = R2 > 1 ? 16 * R2 : 0, kTw3 = R3 > 1 ? 256 * R3 : 0;  // twiddles
+  // Shared-memory pitch of a sequence (element i sits at i + i / 16, so that the stride-16
+  // stores of pass 1 fall on distinct banks).  A half-warp's 16 accesses of 8 bytes reach
+  // 16 / T sequences of T threads in the row kernel and two neighbouring threads of 8
+  // sequences in the column kernel: the pitch is T, or 2, modulo 16.
+  static constexpr int pitch(int want) { return N + N / 16 + ((want - (N + N / 16)) % 16 + 16) % 16; }
+  static constexpr int kRowPitch = pitch(T < 16 ? T : 0);
+  static constexpr int kColPitch = pitch(2);
+  // Index in the transform of the i-th value a thread holds after the last pass.
+  __device__ static __forceinline__ int pos(int i, int t) { return t + (i / RL) * T + (i % RL) * (N / RL); }
+};
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+// Twiddles exp(+j 2 pi j k / (R ns)) of passes 2 (ns = 16) and 3 (ns = 256) at tw[j ns + k],
+// computed by the block.
+template <int N>
+__device__ void make_twiddles(float2* tw) {
+  using S = FftShape<N>;
+  for (int e = threadIdx.x; e < S::kTw2 + S::kTw3; e += blockDim.x) {
+    const bool third = e >= S::kTw2;
+    const int r = third ? e - S::kTw2 : e, ns = third ? 256 : 16, size = third ? S::kTw3 : S::kTw2;
+    float sn, cs;
+    sincospif((float)(2 * (r / ns) * (r % ns)) / (float)size, &sn, &cs);  // size is a power of two: exact
+    tw[e] = make_float2(cs, sn);
+  }
 }
 
-// exp(-j 2 pi k / len) for 0 <= k < len / 2
-__device__ __forceinline__ float2 twiddle(int k, int len) {
-  float s, c;
-  sincospif(-2.0f * (float)k / (float)len, &s, &c);
-  return make_float2(c, s);
-}
-
-// In-place radix-2 decimation-in-time butterflies over `count` independent sequences of
-// length n held in shared memory, element i of sequence j at x[i * istride + j * jstride],
-// already in bit-reversed order.  All threads of the block take part.
-__device__ void fft_stages(float2* x, int n, int count, int istride, int jstride) {
-  const int half_total = (n / 2) * count;
-  for (int len = 2; len <= n; len <<= 1) {
-    const int h = len >> 1;
-    __syncthreads();
-    for (int t = threadIdx.x; t < half_total; t += blockDim.x) {
-      const int j = t % count, b = t / count;
-      const int grp = b / h, k = b % h;
-      const int i0 = grp * len + k, i1 = i0 + h;
-      const float2 w = twiddle(k, len);
-      float2* p0 = x + i0 * istride + j * jstride;
-      float2* p1 = x + i1 * istride + j * jstride;
-      const float2 u = *p0, v = cmul(*p1, w);
-      *p0 = make_float2(u.x + v.x, u.y + v.y);
-      *p1 = make_float2(u.x - v.x, u.y - v.y);
+// One pass of radix R after `ns` points have been combined, from and to the sequence's
+// shared-memory buffer x; the results stay in `a` (sub-butterfly by sub-butterfly) when
+// `last`.  Sync orders the sequence's threads.
+template <int N, int R, class Sync>
+__device__ __forceinline__ void rd_pass(float2 (&a)[FftShape<N>::PER], float2* x, int t, int ns, const float2* tw,
+                                        bool last, Sync sync) {
+  using S = FftShape<N>;
+  constexpr int G = S::PER / R;
+#pragma unroll
+  for (int gi = 0; gi < G; ++gi) {
+    const int b = t + gi * S::T, k = b & (ns - 1);
+    float2 v[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int i = b + j * (N / R);
+      v[j] = x[i + (i >> 4)];
+      if (j > 0) v[j] = cmul(v[j], tw[j * ns + k]);
+    }
+    dft_inv<R>(v);
+#pragma unroll
+    for (int j = 0; j < R; ++j) a[gi * R + j] = v[j];
+  }
+  if (last) return;
+  sync();  // every read of x is done
+#pragma unroll
+  for (int gi = 0; gi < G; ++gi) {
+    const int b = t + gi * S::T, k = b & (ns - 1), o = (b - k) * R + k;
+#pragma unroll
+    for (int m = 0; m < R; ++m) {
+      const int i = o + m * ns;
+      x[i + (i >> 4)] = a[gi * R + m];
     }
   }
+  sync();
+}
+
+// Inverse-sign DFT of the sequence whose elements t + j T (j < PER) are in `a`; value i of
+// the result is element pos(i, t).  (With the components of every input swapped, the
+// result is the forward DFT with its components swapped.)
+template <int N, class Sync>
+__device__ __forceinline__ void rd_fft(float2 (&a)[FftShape<N>::PER], float2* x, int t, const float2* tw, Sync sync) {
+  using S = FftShape<N>;
+  dft_inv<S::PER>(a);
+  if constexpr (S::R2 > 1) {
+    sync();  // the buffer's previous readers are done
+#pragma unroll
+    for (int m = 0; m < S::PER; ++m) x[17 * t + m] = a[m];  // element 16 t + m
+    sync();
+    rd_pass<N, S::R2>(a, x, t, 16, tw, S::R3 == 1, sync);
+    if constexpr (S::R3 > 1) rd_pass<N, S::R3>(a, x, t, 256, tw + S::kTw2, true, sync);
+  }
+}
+
+struct CubePtrs {
+  const float2* p[kRdByValue];
+};
+
+// Rows: FFT over l of every (channel, n) row of frame blockIdx.y, components swapped (the
+// column pass only needs |X|).  The cube is read once, so its lines are marked streaming
+// and leave L2 to the row transforms.
+template <int L>
+__global__ void __launch_bounds__(kRdThreads, 3)
+fft_rows(const __grid_constant__ CubePtrs byval, const float2* const* __restrict__ cubes, float2* __restrict__ tmp,
+         int F, int rows) {
+  using S = FftShape<L>;
+  constexpr int kSeq = kRdThreads / S::T;  // rows per pass of the block
+  extern __shared__ float2 rd_smem[];
+  float2* tw = rd_smem;
+  make_twiddles<L>(tw);
   __syncthreads();
+  const int t = threadIdx.x % S::T, s = threadIdx.x / S::T;
+  float2* x = rd_smem + S::kTw2 + S::kTw3 + s * S::kRowPitch;
+  auto sync = [] {
+    if (S::T <= 32)
+      __syncwarp();
+    else
+      __syncthreads();
+  };
+  for (int f = blockIdx.y; f < F; f += gridDim.y) {
+    const float2* cube = cubes ? cubes[f] : byval.p[f];
+    float2* out = tmp + (int64_t)f * rows * L;
+    for (int64_t r0 = (int64_t)blockIdx.x * kSeq; r0 < rows; r0 += (int64_t)gridDim.x * kSeq) {
+      const int64_t row = r0 + s;
+      const bool live = row < rows;
+      float2 a[S::PER];
+#pragma unroll
+      for (int j = 0; j < S::PER; ++j) {
+        const float2 c = live ? __ldcs(cube + row * L + t + j * S::T) : make_float2(0.f, 0.f);
+        a[j] = make_float2(c.y, c.x);
+      }
+      rd_fft<L>(a, x, t, tw, sync);
+      if (live) {
+#pragma unroll
+        for (int i = 0; i < S::PER; ++i) out[row * L + S::pos(i, t)] = a[i];
+      }
+    }
+  }
 }
 
-// Rows: FFT over l of every (frame, channel, n) row; 8 rows per CTA.
-__global__ void fft_rows(const float2* const* __restrict__ cubes, float2* __restrict__ tmp, int F,
-                         int V, int Ns, int L, int lbits) {
-  extern __shared__ float2 srow[];
-  const int rows_per = 8;
-  const int64_t rows_total = (int64_t)F * V * Ns;
-  const int64_t r0 = (int64_t)blockIdx.x * rows_per;
-  for (int e = threadIdx.x; e < rows_per * L; e += blockDim.x) {
-    const int rr = e / L, l = e % L;
-    const int64_t row = r0 + rr;
-    float2 val = make_float2(0.f, 0.f);
-    if (row < rows_total) {
-      const int64_t f = row / ((int64_t)V * Ns), within = row % ((int64_t)V * Ns);
-      val = cubes[f][within * L + l];
-    }
-    srow[rr * L + bitrev((unsigned)l, lbits)] = val;
-  }
-  fft_stages(srow, L, rows_per, 1, L);
-  for (int e = threadIdx.x; e < rows_per * L; e += blockDim.x) {
-    const int rr = e / L, l = e % L;
-    const int64_t row = r0 + rr;
-    if (row < rows_total) tmp[row * L + l] = srow[rr * L + l];
-  }
-}
-
-// Columns: per frame and block of 16 Doppler bins, FFT over n for every channel and add
-// |X|^2 over the channels in order.
-__global__ void fft_cols(const float2* __restrict__ tmp, float* __restrict__ power, int V, int Ns,
-                         int L, int nbits) {
-  extern __shared__ float2 scol[];  // [Ns][kColBlock] complex, then [Ns][kColBlock] power
-  float* pw = reinterpret_cast<float*>(scol + (size_t)Ns * kColBlock);
-  const int f = blockIdx.y;
-  const int d0 = blockIdx.x * kColBlock;
-  for (int e = threadIdx.x; e < Ns * kColBlock; e += blockDim.x) pw[e] = 0.f;
-  for (int v = 0; v < V; ++v) {
-    const float2* src = tmp + (((int64_t)f * V + v) * Ns) * L;
-    __syncthreads();
-    for (int e = threadIdx.x; e < Ns * kColBlock; e += blockDim.x) {
-      const int n = e / kColBlock, j = e % kColBlock;
-      const int d = d0 + j;
-      const float2 val = (d < L) ? src[(int64_t)n * L + d] : make_float2(0.f, 0.f);
-      scol[bitrev((unsigned)n, nbits) * kColBlock + j] = val;
-    }
-    fft_stages(scol, Ns, kColBlock, kColBlock, 1);
-    for (int e = threadIdx.x; e < Ns * kColBlock; e += blockDim.x) {
-      const float2 x = scol[e];
-      pw[e] += x.x * x.x + x.y * x.y;
-    }
-  }
+// Columns: the threads of a CTA form groups of T x 8, each taking every (number of
+// groups)-th channel's 8 columns; a group sums |X|^2 over its channels in registers and the
+// groups' sums are added in group order.  Frames run from the last to the first: the rows
+// written last are the ones still in L2.
+template <int Ns>
+__global__ void __launch_bounds__(kRdThreadsMax)
+fft_cols(const float2* __restrict__ tmp, float* __restrict__ power, int F, int V, int L) {
+  using S = FftShape<Ns>;
+  constexpr int kGroup = S::T * kRdCols;
+  extern __shared__ float2 rd_smem[];
+  float2* tw = rd_smem;
+  make_twiddles<Ns>(tw);
+  wait_prior_grid();
   __syncthreads();
-  for (int e = threadIdx.x; e < Ns * kColBlock; e += blockDim.x) {
-    const int k = e / kColBlock, j = e % kColBlock;
-    const int d = d0 + j;
-    if (d < L) power[((int64_t)f * Ns + k) * L + d] = pw[e];
+  const int c = threadIdx.x % kRdCols, t = (threadIdx.x / kRdCols) % S::T;
+  const int g = threadIdx.x / kGroup, groups = blockDim.x / kGroup;
+  float2* bufs = rd_smem + S::kTw2 + S::kTw3;
+  float2* x = bufs + (g * kRdCols + c) * S::kColPitch;
+  float* red = reinterpret_cast<float*>(bufs);  // [group][PER][T x 8], over the transform buffers
+  auto sync = [g] {
+    if (kGroup <= 32)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroup) : "memory");
+  };
+  const int d = blockIdx.x * kRdCols + c;
+  for (int f = F - 1 - (int)blockIdx.y; f >= 0; f -= gridDim.y) {
+    float pw[S::PER];
+#pragma unroll
+    for (int i = 0; i < S::PER; ++i) pw[i] = 0.f;
+    // every group runs the same number of rounds: for short transforms groups share a warp
+    for (int v0 = 0; v0 < V; v0 += groups) {
+      const int v = v0 + g;
+      const bool live = v < V && d < L;
+      const float2* src = tmp + ((int64_t)f * V + v) * Ns * L + d;
+      float2 a[S::PER];
+#pragma unroll
+      for (int j = 0; j < S::PER; ++j)
+        a[j] = live ? src[(int64_t)(t + j * S::T) * L] : make_float2(0.f, 0.f);
+      rd_fft<Ns>(a, x, t, tw, sync);
+#pragma unroll
+      for (int i = 0; i < S::PER; ++i) pw[i] += a[i].x * a[i].x + a[i].y * a[i].y;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < S::PER; ++i) red[(g * S::PER + i) * kGroup + threadIdx.x % kGroup] = pw[i];
+    __syncthreads();
+    // the block size is a multiple of 8, so an output's column is this thread's own
+    for (int o = threadIdx.x; o < S::PER * kGroup; o += blockDim.x) {
+      float sum = red[o];
+      for (int h = 1; h < groups; ++h) sum += red[h * S::PER * kGroup + o];
+      const int i = o / kGroup, to = (o % kGroup) / kRdCols;
+      if (d < L) power[((int64_t)f * Ns + S::pos(i, to)) * L + d] = sum;
+    }
+    __syncthreads();  // the next frame's transforms overwrite the sums
   }
 }
 
-// Largest power of one frame (first flat index on ties), optionally without d = 0.
-__global__ void rd_argmax(const float* __restrict__ power, int Ns, int L, int skip_static,
-                          double v_per_bin, float* __restrict__ v_est, int32_t* __restrict__ peak) {
-  const int f = blockIdx.x;
-  const float* p = power + (int64_t)f * Ns * L;
+// Largest power of one frame (first flat index on ties), optionally without d = 0.  Four
+// 16-byte loads in flight per thread where the map is 16-byte aligned.
+constexpr int kArgThreads = 1024;
+__global__ void __launch_bounds__(kArgThreads)
+rd_argmax(const float* __restrict__ power, int Ns, int L, int skip_static, double v_per_bin,
+          float* __restrict__ v_est, int32_t* __restrict__ peak) {
+  wait_prior_grid();
+  const int f = blockIdx.x, n = Ns * L;
+  const float* p = power + (int64_t)f * n;
   float best = -1.f;
   int bi = 0x7fffffff;
-  for (int i = threadIdx.x; i < Ns * L; i += blockDim.x) {
-    const int d = i % L;
-    if (skip_static && d == 0) continue;
-    const float x = p[i];
-    if (x > best || (x == best && i < bi)) {
+  // within a thread the indices rise, so a strict comparison keeps the first of equals
+  auto take = [&](float x, int i) {
+    if (x > best && !(skip_static && (i & (L - 1)) == 0)) {
       best = x;
       bi = i;
     }
+  };
+  if (n % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+    const float4* p4 = reinterpret_cast<const float4*>(p);
+    for (int i0 = threadIdx.x; i0 < n / 4; i0 += 4 * kArgThreads) {
+      float4 q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * kArgThreads;
+        q[u] = i < n / 4 ? p4[i] : make_float4(-1.f, -1.f, -1.f, -1.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = 4 * (i0 + u * kArgThreads);
+        take(q[u].x, i);
+        take(q[u].y, i + 1);
+        take(q[u].z, i + 2);
+        take(q[u].w, i + 3);
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < n; i += kArgThreads) take(p[i], i);
   }
   __shared__ float sb[32];
   __shared__ int si[32];
@@ -154,7 +287,7 @@ __global__ void rd_argmax(const float* __restrict__ power, int Ns, int L, int sk
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int k = 1; k < (int)(blockDim.x >> 5); ++k)
+    for (int k = 1; k < kArgThreads / 32; ++k)
       if (sb[k] > best || (sb[k] == best && si[k] < bi)) {
         best = sb[k];
         bi = si[k];
@@ -169,35 +302,86 @@ __global__ void rd_argmax(const float* __restrict__ power, int Ns, int L, int sk
   }
 }
 
-int ilog2(int x) {
-  int b = 0;
-  while ((1 << b) < x) ++b;
-  return b;
+using RowFn = void (*)(CubePtrs, const float2* const*, float2*, int, int);
+using ColFn = void (*)(const float2*, float*, int, int, int);
+struct RowKernel {
+  RowFn fn;
+  int rows, smem;  // rows per pass of a block
+};
+struct ColKernel {
+  ColFn fn;
+  int group, fixed, per_group;  // threads of a group; shared memory: twiddles, then per group
+};
+
+template <int N>
+RowKernel row_kernel() {
+  using S = FftShape<N>;
+  const int seq = kRdThreads / S::T;
+  return {fft_rows<N>, seq, 8 * (S::kTw2 + S::kTw3 + (S::R2 > 1 ? seq * S::kRowPitch : 0))};
 }
+template <int N>
+ColKernel col_kernel() {
+  using S = FftShape<N>;
+  const int buf = S::R2 > 1 ? 8 * kRdCols * S::kColPitch : 0, sums = 4 * S::PER * S::T * kRdCols;
+  return {fft_cols<N>, S::T * kRdCols, 8 * (S::kTw2 + S::kTw3), std::max(buf, sums)};
+}
+
+template <class R, template <int> class Pick>
+R by_length(int n) {
+  switch (n) {
+    case 2: return Pick<2>::get();
+    case 4: return Pick<4>::get();
+    case 8: return Pick<8>::get();
+    case 16: return Pick<16>::get();
+    case 32: return Pick<32>::get();
+    case 64: return Pick<64>::get();
+    case 128: return Pick<128>::get();
+    case 256: return Pick<256>::get();
+    case 512: return Pick<512>::get();
+    default: return Pick<1024>::get();
+  }
+}
+template <int N>
+struct PickRow {
+  static RowKernel get() { return row_kernel<N>(); }
+};
+template <int N>
+struct PickCol {
+  static ColKernel get() { return col_kernel<N>(); }
+};
 
 }  // namespace
 
-cudaError_t launch_range_doppler(const float2* const* cubes_dev, float2* tmp, float* power, int F,
-                                 int V, int Ns, int L, int skip_static, double v_per_bin, float* v_est,
-                                 int32_t* peak, cudaStream_t st) {
-  const int lbits = ilog2(L), nbits = ilog2(Ns);
-  const int64_t rows = (int64_t)F * V * Ns;
-  const int64_t row_blocks = (rows + 7) / 8;
-  if (row_blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-  const int rsmem = 8 * L * (int)sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(fft_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, rsmem);
+cudaError_t launch_range_doppler(const float2* const* cubes, const float2* const* cubes_dev, float2* tmp, float* power,
+                                 int F, int V, int Ns, int L, int skip_static, double v_per_bin, float* v_est,
+                                 int32_t* peak, int num_sms, cudaStream_t st) {
+  const RowKernel rk = by_length<RowKernel, PickRow>(L);
+  const ColKernel ck = by_length<ColKernel, PickCol>(Ns);
+  CubePtrs byval = {};
+  if (!cubes_dev)
+    for (int f = 0; f < F; ++f) byval.p[f] = cubes[f];
+  const int fy = std::min(F, 65535);
+  // rows: about four waves of blocks at three per SM, so that a block makes its twiddles
+  // once for several passes; at least one block per frame
+  const int64_t rows = (int64_t)V * Ns;
+  const int64_t passes = (rows + rk.rows - 1) / rk.rows;
+  const int64_t bx = std::min<int64_t>(passes, std::max<int64_t>(1, (12ll * num_sms + fy - 1) / fy));
+  cudaError_t e = cudaFuncSetAttribute(rk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, rk.smem);
   if (e != cudaSuccess) return e;
-  fft_rows<<<(unsigned)row_blocks, 256, rsmem, st>>>(cubes_dev, tmp, F, V, Ns, L, lbits);
+  rk.fn<<<dim3((unsigned)bx, fy), kRdThreads, rk.smem, st>>>(byval, cubes_dev, tmp, F, (int)rows);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int smem = Ns * kColBlock * (int)(sizeof(float2) + sizeof(float));
-  e = cudaFuncSetAttribute(fft_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // columns: 256 threads where the frames fill the SMs twice over, else 512 (more channels
+  // of a frame at a time)
+  const int cx = (L + kRdCols - 1) / kRdCols;
+  const int threads = std::max(ck.group, (int64_t)cx * F >= 2ll * num_sms ? kRdThreads : kRdThreadsMax);
+  const int smem = ck.fixed + (threads / ck.group) * ck.per_group;
+  e = cudaFuncSetAttribute(ck.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  fft_cols<<<dim3((L + kColBlock - 1) / kColBlock, F), 256, smem, st>>>(tmp, power, V, Ns, L, nbits);
-  e = cudaGetLastError();
+  e = launch_dependent(ck.fn, dim3(cx, fy), dim3(threads), (size_t)smem, st, (const float2*)tmp, power, F, V, L);
   if (e != cudaSuccess) return e;
-  rd_argmax<<<F, 256, 0, st>>>(power, Ns, L, skip_static, v_per_bin, v_est, peak);
-  return cudaGetLastError();
+  return launch_dependent(rd_argmax, dim3(F), dim3(kArgThreads), 0, st, (const float*)power, Ns, L, skip_static,
+                          v_per_bin, v_est, peak);
 }
 
 }  // namespace rsim
@@ -225,12 +409,17 @@ extern "C" rsim_status rsim_range_doppler(rsim_ctx* ctx, const rsim_radar_params
   s = ensure_workspace(ctx, ptr_bytes + tmp_bytes, st);
   if (s != RSIM_OK) return s;
   char* ws = (char*)ctx->ws;
-  cudaError_t e = cudaMemcpyAsync(ws, cubes, sizeof(void*) * (size_t)F, cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return cuda_fail(e, "upload of the cube table");
+  cudaError_t e = cudaSuccess;
+  const bool table = F > kRdByValue;  // few pointers go in the kernel's arguments
+  if (table) {
+    e = cudaMemcpyAsync(ws, cubes, sizeof(void*) * (size_t)F, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return cuda_fail(e, "upload of the cube table");
+  }
   const double t_slow = params->t_slow > 0 ? params->t_slow : params->M * params->t_b;
   const double v_per_bin = params->lambda / (2.0 * t_slow * k.L);
-  e = launch_range_doppler((const float2* const*)ws, (float2*)(ws + ptr_bytes), power, F, k.V, k.Ns, k.L,
-                           (options & RSIM_RD_SKIP_STATIC) ? 1 : 0, v_per_bin, v_est, peak, st);
+  e = launch_range_doppler((const float2* const*)cubes, table ? (const float2* const*)ws : nullptr,
+                           (float2*)(ws + ptr_bytes), power, F, k.V, k.Ns, k.L,
+                           (options & RSIM_RD_SKIP_STATIC) ? 1 : 0, v_per_bin, v_est, peak, ctx->num_sms, st);
   if (e != cudaSuccess) return cuda_fail(e, "range-Doppler kernels");
   return RSIM_OK;
 }

@@ -288,9 +288,11 @@ cudaError_t launch_umma(const Consts& k, const FrameIO* frames, int F, int split
                         int64_t max_p, int fast_terms_dtype, unsigned* status, int* unit_counter,
                         cudaStream_t st, cudaEvent_t mid = nullptr);
 
-cudaError_t launch_range_doppler(const float2* const* cubes_dev, float2* tmp, float* power, int F,
-                                 int V, int Ns, int L, int skip_static, double v_per_bin, float* v_est,
-                                 int32_t* peak, cudaStream_t st);
+// cubes: HOST array of the F cube pointers; cubes_dev: the same on the device, or NULL to pass
+// them by value (F <= 64).
+cudaError_t launch_range_doppler(const float2* const* cubes, const float2* const* cubes_dev, float2* tmp, float* power,
+                                 int F, int V, int Ns, int L, int skip_static, double v_per_bin, float* v_est,
+                                 int32_t* peak, int num_sms, cudaStream_t st);
 
 // Plan rules shared by single-frame and batch paths (they depend on the shape only).
 // tile_n: the plan's tile (tensor tiers: column tile NT; FP32: n per CTA tile).

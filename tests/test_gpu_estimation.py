@@ -98,3 +98,33 @@ def test_non_power_of_two_is_unsupported(env):
     with pytest.raises(_abi.RsimError) as e:
         _rd(env, radar, [cube])
     assert e.value.status == _abi.ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("Ns,L", [(2, 2), (4, 16), (8, 4), (16, 8), (32, 1024), (64, 64), (128, 512), (1024, 32)])
+@pytest.mark.parametrize("V,F", [(1, 1), (3, 5), (13, 3), (2, 70)])
+def test_every_transform_length(env, Ns, L, V, F):
+    """Each FFT length as rows and as columns, with channel counts that do not fill the
+    column groups, few frames and more than the 64 whose pointers go by value, and a map that
+    is only 4-byte aligned.  FP32 FFT error: about u log2(N_s L) per value (u = 6e-8, at most
+    15 stages here), twice that in |X|^2: below 2e-6 normwise; the bar is 3e-6."""
+    torch, _abi, device, ctx = env
+    radar = Radar(M=V, N=1, Ns=Ns, L=L)
+    g = torch.Generator(device="cpu").manual_seed(Ns * 1000 + L + V)
+    cubes = [torch.randn((V, Ns, L), dtype=torch.complex64, generator=g).cuda() for _ in range(F)]
+    buf = torch.full((F * Ns * L + 1,), float("nan"), dtype=torch.float32, device="cuda")
+    power = buf[1:]
+    v = torch.empty(F, dtype=torch.float32, device="cuda")
+    peak = torch.empty((F, 2), dtype=torch.int32, device="cuda")
+    for skip in (False, True):
+        _abi.rsim_range_doppler(ctx.h, radar, cubes, power, v, peak, skip_static=skip)
+        torch.cuda.synchronize()
+        pw = power.cpu().numpy().reshape(F, Ns, L)
+        for f in sorted({0, F // 2, F - 1}):
+            ref = oracle.range_doppler_power(cubes[f].cpu().numpy())
+            assert np.linalg.norm(pw[f] - ref) / np.linalg.norm(ref) < 3e-6
+        # the peak is the first largest value of the map itself
+        m = pw.copy()
+        if skip:
+            m[:, :, 0] = -1.0
+        first = m.reshape(F, -1).argmax(1)
+        assert np.array_equal(peak.cpu().numpy(), np.stack([first // L, first % L], axis=1))
