@@ -394,7 +394,8 @@ def run_gpu(args):
 
     if rank == 0:
         peaks, kind = _peaks()
-        roof = _roofline(tier, prof.contract_ms - prof.operand_ms, prof.calls, samples, peaks, kind)
+        # the FP32 tier runs three products on the tensor cores, like the split tiers
+        roof = _roofline("split_fp16" if tier == "fp32" else tier, prof.contract_ms - prof.operand_ms, prof.calls, samples, peaks, kind)
         traffic = _load_traffic(tier)
         if traffic is not None:
             roof["traffic"] = traffic
@@ -456,15 +457,21 @@ def run_gpu(args):
     return 0
 
 
-KERNEL_SOURCES = {"fp32": "k_direct.cu", "split_fp16": "k_umma.cu", "split_bf16": "k_umma.cu",
-                  "bf16": "k_umma.cu", "fp16": "k_umma.cu"}
+# the operand builder's file and, for the tiers on pairs of CTAs, the contraction's
+KERNEL_SOURCES = {"fp32": "k_umma.cu k_umma_pair.cu", "split_fp16": "k_umma.cu k_umma_pair.cu",
+                  "split_bf16": "k_umma.cu k_umma_pair.cu", "bf16": "k_umma.cu", "fp16": "k_umma.cu"}
 
 
 def kernel_source_hash(tier):
     import hashlib
-    p = os.path.join(ROOT, "paper_2307_09226_gb300", "csrc", KERNEL_SOURCES[tier])
-    with open(p, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:12]
+    csrc = os.path.join(ROOT, "paper_2307_09226_gb300", "csrc")
+    h = hashlib.sha256()
+    for name in KERNEL_SOURCES[tier].split():
+        p = os.path.join(csrc, name)
+        if os.path.exists(p):
+            with open(p, "rb") as f:
+                h.update(f.read())
+    return h.hexdigest()[:12]
 
 
 def _load_traffic(tier):

@@ -72,7 +72,11 @@ typedef enum {
 
 /* Arithmetic tier of the contraction over pixels. */
 typedef enum {
-  RSIM_TIER_FP32 = 0,       /* FP32 direct sum on CUDA cores */
+  RSIM_TIER_FP32 = 0,       /* FP32 accuracy (relative error below 1e-6 where measured).  From 128
+                               pixels on, tcgen05 with FP16 hi+lo operands (3 products) and FP32 sums
+                               of at most two 32-pixel chunks each; else, and wherever a plan of its
+                               own is pinned or tuned for the shape or the workspace bound holds no
+                               more, the FP32 direct sum on CUDA cores */
   RSIM_TIER_BF16 = 1,       /* tcgen05 tensor cores, BF16 operands, FP32 accumulate */
   RSIM_TIER_SPLIT_BF16 = 2, /* tcgen05, BF16 hi+lo operands (3 products), FP32 accumulate */
   RSIM_TIER_SPLIT_FP16 = 3, /* tcgen05, FP16 hi+lo operands (3 products), FP32 accumulate */
@@ -210,7 +214,8 @@ rsim_status rsim_synth_batch(rsim_ctx* ctx, const rsim_radar_params* params,
  * anything is launched.  Calls no cudaMalloc, cudaFree or other allocating routine.
  * Inputs and output are as in rsim_synth (device pointers owned by the caller); the
  * plan is the library's default rule for the shape, so the result equals rsim_synth
- * of a context that has no tuned plan for it.
+ * of a context that has no tuned plan for it.  (A frame of the FP32 tier whose scratch on
+ * the tensor cores exceeds 64 MiB runs on the CUDA cores: the same sum, other roundings.)
  *
  * device_status: optional DEVICE pointer to a uint32 that the kernels OR their
  * status bits into (1: a valid pixel had a non-finite field or R <= 0; 2: a
@@ -410,11 +415,11 @@ typedef struct {
                             a multiple of 8 in 8..128 and at most L rounded up to 8 (the
                             MMA's N is 2 NT; default min(128, L rounded up to 8)).  FP32
                             tier: n values per CTA tile, 64 or 128 (default 128); the CTA
-                            tile is tile_n x 64 (l).  NUFFT tier: ignored.  0 = default */
+                            tile of the CUDA-core sum is tile_n x 64 (l).  NUFFT tier: ignored.  0 = default */
   int32_t group_chunks;  /* tensor-core tiers: 32-pixel chunks summed in one tensor-memory
                             accumulator before it is drained into round-to-nearest FP32
                             sums.  The accumulator rounds toward zero, so the cap bounds the
-                            error: 1..40 for split tiers (default 40), 1..384 for plain
+                            error: 1..40 for split tiers (default 8), 1..384 for plain
                             16-bit tiers (default 96).  Other tiers: ignored.  0 = default */
   int32_t reserved;
 } rsim_plan;
@@ -431,7 +436,8 @@ rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* params, int64_
                           rsim_tier tier, rsim_plan* chosen, rsim_stream stream);
 
 /* Pin `plan` for the bucket of (params, P, tier) in the context's cache (replaces a tuned
- * or default plan).  splits in 1..64; grid 0 (one CTA per SM) or a positive CTA count
+ * or default plan).  For RSIM_TIER_FP32 the plan is one of the CUDA-core sum, which then
+ * runs the bucket.  splits in 1..64; grid 0 (one CTA per SM) or a positive CTA count
  * (more than the SM count runs as one per SM); variant 0; tile_n and group_chunks 0 or in
  * the ranges stated in rsim_plan.  Host only.  Errors: INVALID_ARG. */
 rsim_status rsim_set_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_t P,

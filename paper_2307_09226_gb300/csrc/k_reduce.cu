@@ -11,18 +11,12 @@
 namespace rsim {
 namespace {
 
-// cube = scale * sum over splits s = 0, 1, ... (in this order) of partial[s], with
-// compensated FP32 additions (GB300's FP64 rate is a small fraction of its FP32 rate).
+// cube = sum over splits s = 0, 1, ... (in this order) of partial[s], with compensated FP32 additions (GB300's FP64 rate is a small fraction of its FP32 rate).
 // Loads of kReduceBatch splits are issued together; the additions keep the split order.
 __global__ void split_reduce(const FrameIO* __restrict__ frames, int64_t count, int splits,
-                             int out_dtype, int scale_mode) {
+                             int out_dtype) {
   wait_prior_grid();
   const FrameIO& fr = frames[blockIdx.y];
-  float scale = 1.f;
-  if (scale_mode) {
-    const float m = __uint_as_float((unsigned)fr.meta[1]);
-    scale = (m > 0.f) ? ldexpf(1.f, ilogbf(m) + 1) : 1.f;
-  }
   const float2* __restrict__ part = fr.partial;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -40,8 +34,6 @@ __global__ void split_reduce(const FrameIO* __restrict__ frames, int64_t count, 
         }
       }
     }
-    re *= scale;  // power of two: exact
-    im *= scale;
     if (out_dtype == RSIM_C128)
       reinterpret_cast<double2*>(fr.cube)[i] = make_double2((double)re, (double)im);
     else
@@ -62,11 +54,8 @@ __global__ void __launch_bounds__(256, 6) split_reduce_tiles(const FrameIO* __re
                                    int64_t sstride, int splits, int out_dtype, int scale_mode) {
   wait_prior_grid();
   const FrameIO& fr = frames[blockIdx.y];
-  float scale = 1.f;
-  if (scale_mode) {
-    const float m = __uint_as_float((unsigned)fr.meta[1]);
-    scale = (m > 0.f) ? ldexpf(1.f, ilogbf(m) + 1) : 1.f;
-  }
+  // the FP16 tiers' power of two, undone (exact)
+  const float2 scale = pow2_factors(scale_mode ? sigma_exponent(fr.meta[1]) : 0);
   const int64_t rows = (int64_t)k.V * k.Ns;
   const int64_t n4 = sstride / 2;
   const int pairs = NT / 2;
@@ -95,16 +84,18 @@ __global__ void __launch_bounds__(256, 6) split_reduce_tiles(const FrameIO* __re
         }
       }
     }
+    s0 = s0 * scale.x * scale.y, s1 = s1 * scale.x * scale.y;
+    s2 = s2 * scale.x * scale.y, s3 = s3 * scale.x * scale.y;
     const int64_t o = row * k.L + l;
     const bool two = (l + 1 < k.L);
     if (out_dtype == RSIM_C128) {
       double2* cd = reinterpret_cast<double2*>(fr.cube);
-      cd[o] = make_double2((double)(s0 * scale), (double)(s1 * scale));
-      if (two) cd[o + 1] = make_double2((double)(s2 * scale), (double)(s3 * scale));
+      cd[o] = make_double2((double)s0, (double)s1);
+      if (two) cd[o + 1] = make_double2((double)s2, (double)s3);
     } else {
       float2* cf = reinterpret_cast<float2*>(fr.cube);
-      cf[o] = make_float2(s0 * scale, s1 * scale);
-      if (two) cf[o + 1] = make_float2(s2 * scale, s3 * scale);
+      cf[o] = make_float2(s0, s1);
+      if (two) cf[o + 1] = make_float2(s2, s3);
     }
   }
 }
@@ -112,14 +103,13 @@ __global__ void __launch_bounds__(256, 6) split_reduce_tiles(const FrameIO* __re
 }  // namespace
 
 cudaError_t launch_reduce(const Consts& k, const FrameIO* frames, int F, int splits, int out_dtype,
-                          float scale_mode, cudaStream_t st) {
+                          cudaStream_t st) {
   const int64_t count = (int64_t)k.V * k.Ns * k.L;
   if (count <= 0 || F <= 0) return cudaSuccess;
   int64_t blocks = (count + 255) / 256;
   if (blocks > 4096) blocks = 4096;
   dim3 grid((unsigned)blocks, F);
-  return launch_dependent(split_reduce, grid, dim3(256), 0, st, frames, count, splits, out_dtype,
-                          scale_mode != 0.f ? 1 : 0);
+  return launch_dependent(split_reduce, grid, dim3(256), 0, st, frames, count, splits, out_dtype);
 }
 
 cudaError_t launch_reduce_tiles(const Consts& k, const FrameIO* frames, int F, int splits, int nt,

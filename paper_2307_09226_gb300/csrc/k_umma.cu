@@ -8,8 +8,8 @@
 //     A_r[(v,n)][2q + {0,1}] = (Re F, Im F),
 //     B_r[2q + {0,1}][l]     = (Re D, -Im D),   B_r[2q + {0,1}][NT + l] = (Im D, Re D),
 // with K = 2 * (valid pixels) and N = 2 * NT columns per column tile (NT <= 128
-// values of l).  Split-precision tiers write each operand as hi + lo 16-bit parts and
-// accumulate A_hi B_hi + A_hi B_lo + A_lo B_hi in FP32.
+// values of l).  Split-precision tiers (and the FP32 tier) write each operand as hi + lo
+// 16-bit parts and accumulate A_hi B_hi + A_hi B_lo + A_lo B_hi in FP32.
 //
 // B (sigma x slow-time phasors) is shared by every row tile, so an operand-builder
 // kernel writes it once per frame as ready-made shared-memory images: for each
@@ -19,7 +19,9 @@
 // phasors) differs for every row tile and is never reused, so it is generated on chip
 // and never touches HBM.
 //
-// The contraction runs one persistent CTA per SM, warp-specialised:
+// This file: the operand builder, the launches, and the contraction of the plain 16-bit
+// tiers; the split tiers run on pairs of CTAs (k_umma_pair.cu).  The plain contraction runs
+// one persistent CTA per SM, warp-specialised:
 //   warps 0-15  produce A for a 128-row tile straight into tensor memory (one row per
 //               thread, tcgen05.st).  Two groups of 8 warps take alternate stages; in a
 //               stage, two warps share a lane quarter with 16 pixels each.  The same
@@ -29,23 +31,25 @@
 //   warp 17     takes work units from a device counter and bulk-copies each chunk's
 //               phases of the tile's channels into a shared-memory ring;
 //   warp 18     bulk-copies each chunk's B images into the operand stages.
-// A and B have rings of their own: four A stages in tensor memory (the columns the
-// accumulator leaves free) and three B stages in shared memory (what its 227 KB hold),
-// so a producer group has four MMA stages of time, not three, to make its next A stage.
+// A and B have rings of their own: eight A stages in tensor memory (the columns the
+// accumulator leaves free) and six B stages in shared memory (192 of its 227 KB, which also
+// keeps a second CTA, and its claim on tensor memory, off the SM).  The kernel is bound by the
+// making of A: with four and three stages of twice the size, shared with the split tiers,
+// BF16 on 256 x 256 pixels (V = 12, N_s = 256, L = 128) took 170 us a call, now 155.
 // Each slot of either ring has a "full" mbarrier (the producer group's arrivals, or the
 // B copy's bytes) and an "empty" mbarrier, completed by a tcgen05.commit after the MMAs
 // that read it.  Every wait is bounded in time and a timeout sets a status bit instead
 // of hanging.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include "rsim_internal.h"
+#include "umma.h"
 
 namespace rsim {
 namespace {
 
-constexpr int kStages = 3;                 // B operand stages in shared memory (64 KB each: hi + lo)
-constexpr int kAStages = 4;                // A operand stages in tensor memory (64 columns each: hi + lo)
+using namespace umma;
+
+constexpr int kStages = 6;                 // B operand stages in shared memory (32 KB each)
+constexpr int kAStages = 8;                // A operand stages in tensor memory (32 columns each)
 constexpr int kPixStages = 6;              // ring of staged per-chunk pixel phases
 constexpr int kUnitSlots = 4;              // ring of work-unit ids
 constexpr int kMaxCh = 8;                  // channels a row tile may span for staging
@@ -53,13 +57,10 @@ constexpr int kAWarps = 16;                // A producers: two groups that take 
 constexpr int kAGroupWarps = kAWarps / 2;  // 8 warps per group, two per lane quarter
 constexpr int kAPx = kChunkPx / (kAGroupWarps / 4);  // pixels per A warp per stage
 constexpr int kThreads = 32 * (kAWarps + 3);  // + MMA warp, pixel loader, B loader
-constexpr int kBRowsMax = 256;             // N = 2 * NT <= 256
-constexpr int kBBytes = kBRowsMax * 128;   // one 16-bit operand part of one stage
-constexpr int kStageBytes = 2 * kBBytes;   // hi + lo
+constexpr int kStageBytes = 256 * 128;     // a B stage: N = 2 NT <= 256 rows of 128 bytes
 constexpr int kAccCols = 256;              // accumulator columns (N <= 256 FP32)
 constexpr int kTmemCols = 512;
-static_assert(kAccCols + kAStages * 64 <= kTmemCols, "accumulator and A stages fit in tensor memory");
-constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s per wait, then give up
+static_assert(kAccCols + kAStages * 32 <= kTmemCols, "accumulator and A stages fit in tensor memory");
 
 // Per-chunk fast-time/channel phases staged by the pixel loader (bulk copies).
 struct PixStage {
@@ -84,132 +85,19 @@ struct Shared {
   int abort;
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
+  return umma::mbar_wait(b, parity, &sh->abort, status);
+}
+__device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
+  return umma::warp_wait(b, parity, &sh->abort, status);
 }
 
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(b))
-               : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Wait for the phase of parity `parity` to complete; false on timeout or abort.
-__device__ __noinline__ bool mbar_wait(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
-  uint64_t t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try(b, parity)) return true;
-    if ((it & 255u) == 255u) {
-      if (*(volatile int*)&sh->abort) return false;
-      const uint64_t now = globaltimer();
-      if (t0 == 0) {
-        t0 = now;
-      } else if (now - t0 > kWaitNs) {
-        atomicOr(status, kStatusTimeout);
-        *(volatile int*)&sh->abort = 1;
-        return false;
-      }
-    }
-  }
-}
-
-// Inline fast path of mbar_wait for the MMA thread: one probe of a phase that has
-// usually completed already, the bounded polling loop only when it has not.
-__device__ __forceinline__ bool mbar_wait_fast(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
-  return mbar_try(b, parity) || mbar_wait(b, parity, sh, status);
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(
-                   smem_u32(b)),
-               "r"(bytes)
-               : "memory");
-}
-
-// L2 eviction priorities.  A chunk's B images are read by every row tile at about the
-// same time and then never again, while the split partial sums wait in L2 for the
-// reduction after the contraction: the B copies take evict_first and the partial-sum
-// stores and reductions evict_last.  (The partial sums are found in L2 by the reduction
-// with evict_normal stores too; what it pays for is that most of its reads are served by
-// the other die's L2 partition, over the link between the two partitions.)
-// bulk_g2s with a createpolicy policy for the source lines:
-__device__ __forceinline__ void bulk_g2s_hint(void* dst, const void* src, uint32_t bytes, uint64_t* bar,
-                                              uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
-      : "memory");
-}
-__device__ __forceinline__ uint64_t policy_evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ uint64_t policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-// 16-byte store and FP32 add-reduction with a policy (the reduction is one instruction,
-// like atomicAdd on a float4, so each address's additions keep the issuing thread's order).
-__device__ __forceinline__ void st_hint_v4(float4* a, float4 v, uint64_t policy) {
-  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(a), "f"(v.x), "f"(v.y), "f"(v.z),
-               "f"(v.w), "l"(policy)
-               : "memory");
-}
+// FP32 add-reduction of 16 bytes with a policy (one instruction, like atomicAdd on a float4, so
+// each address's additions keep the issuing thread's order).
 __device__ __forceinline__ void red_hint_v4(float4* a, float4 v, uint64_t policy) {
   asm volatile("red.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(a), "f"(v.x), "f"(v.y),
                "f"(v.z), "f"(v.w), "l"(policy)
                : "memory");
-}
-
-// 1-D bulk copy global -> shared (16-byte aligned, size a multiple of 16) that
-// completes `bytes` of the barrier's transaction count.
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ void fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
-// 128-byte-swizzled K-major shared-memory matrix descriptor (tcgen05 format): rows of
-// 128 B, 8-row groups 1024 B apart (stride byte offset), version 1, swizzle mode 2.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr) {
-  uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;              // leading byte offset (unused for this layout)
-  d |= (uint64_t)(1024 >> 4) << 32;    // stride byte offset
-  d |= (uint64_t)1 << 46;              // descriptor version
-  d |= (uint64_t)2 << 61;              // 128-byte swizzle
-  return d;
 }
 
 // Instruction descriptor of kind::f16: FP32 accumulator, K-major A and B, M = 128.
@@ -218,18 +106,12 @@ __host__ __device__ constexpr uint32_t idesc_f16(int bf16, int n) {
          ((uint32_t)(128 >> 4) << 24);
 }
 
-// All MMAs of one 32-pixel operand stage (K = 64 16-bit elements = four K = 16 steps),
-// in one block so that nothing is recomputed between issues.  `a`: tensor-memory column
-// of the stage's hi A part (the lo part starts 32 columns on); `bd`: shared-memory
-// descriptor of the stage's hi B image (the lo image starts kBBytes on).  K step ks
-// reads A columns a + 8 ks and B bytes + 32 ks (2 in the descriptor's 16-byte address
-// field).  Split tiers add A_hi B_lo and A_lo B_hi after each A_hi B_hi.  `acc` = 0
+// All MMAs of one 32-pixel operand stage (K = 64 16-bit elements = four K = 16 steps), in one
+// block so that nothing is recomputed between issues.  `a`: tensor-memory column of the
+// stage's A; `bd`: shared-memory descriptor of its B image.  K step ks reads A columns
+// a + 8 ks and B bytes + 32 ks (2 in the descriptor's 16-byte address field).  `acc` = 0
 // starts a new accumulation with the stage's first MMA.
-template <int SPLIT>
-__device__ __forceinline__ void mma_stage(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc);
-
-template <>
-__device__ __forceinline__ void mma_stage<0>(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_stage(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p, t;\n\t"
       "setp.ne.b32 p, %10, 0;\n\t"
@@ -240,31 +122,6 @@ __device__ __forceinline__ void mma_stage<0>(uint32_t d, uint32_t a, uint64_t bd
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %8, %9, t;\n\t}" ::"r"(d),
       "r"(a), "r"(a + 8), "r"(a + 16), "r"(a + 24), "l"(bd), "l"(bd + 2), "l"(bd + 4), "l"(bd + 6),
       "r"(idesc), "r"(acc)
-      : "memory");
-}
-
-template <>
-__device__ __forceinline__ void mma_stage<1>(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc) {
-  constexpr uint64_t kLo = kBBytes >> 4;
-  asm volatile(
-      "{\n\t.reg .pred p, t;\n\t"
-      "setp.ne.b32 p, %18, 0;\n\t"
-      "setp.ne.b32 t, %17, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %9, %17, p;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %13, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%5], %9, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%2], %10, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%2], %14, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%6], %10, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%3], %11, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%3], %15, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%7], %11, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %12, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %16, %17, t;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%8], %12, %17, t;\n\t}" ::"r"(d),
-      "r"(a), "r"(a + 8), "r"(a + 16), "r"(a + 24), "r"(a + 32), "r"(a + 40), "r"(a + 48), "r"(a + 56),
-      "l"(bd), "l"(bd + 2), "l"(bd + 4), "l"(bd + 6), "l"(bd + kLo), "l"(bd + kLo + 2), "l"(bd + kLo + 4),
-      "l"(bd + kLo + 6), "r"(idesc), "r"(acc)
       : "memory");
 }
 
@@ -281,49 +138,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
       "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
       "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
       : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                 "=r"(v[7])
-               : "r"(taddr)
-               : "memory");
-}
-
-__device__ __forceinline__ float2 cis_q32(uint32_t ph) {
-  const float ang = (float)(int32_t)ph * 1.46291807926715968e-09f;  // 2 pi / 2^32
-  float s, c;
-  __sincosf(ang, &s, &c);
-  return make_float2(c, s);
-}
-
-// exp(j 2 pi x) for a 2^-32-cycle phase, the fraction taken from the top 23 bits by
-// placing them in the mantissa of a float in [1, 2) (no integer-to-float conversion);
-// the quantisation to 2^-23 cycle adds at most 7.5e-7 rad.
-__device__ __forceinline__ float2 cis_q32_fast(uint32_t ph) {
-  const float x = __int_as_float(0x3F800000u | ((ph ^ 0x80000000u) >> 9)) - 1.5f;  // [-1/2, 1/2)
-  float s, c;
-  __sincosf(x * 6.28318530717958648f, &s, &c);
-  return make_float2(c, s);
-}
-
-// Split (x, y) into 16-bit hi and lo pairs, packed low = x, high = y.
-template <int BF>
-__device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t& lo) {
-  if (BF) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    float2 hf = __bfloat1622float2(h);
-    __nv_bfloat162 l = __floats2bfloat162_rn(x - hf.x, y - hf.y);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-  } else {
-    __half2 h = __floats2half2_rn(x, y);
-    float2 hf = __half22float2(h);
-    __half2 l = __floats2half2_rn(x - hf.x, y - hf.y);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-  }
 }
 
 struct Geo {
@@ -370,18 +184,6 @@ __device__ __forceinline__ int64_t unit_groups(const Unit& x, int gmax) {
 }
 __device__ __forceinline__ int64_t group_begin(const Unit& x, int64_t ngr, int64_t k) {
   return x.c0 + (x.c1 - x.c0) * k / ngr;
-}
-
-// sigma scale of the FP16 tiers: 2^-e with max(|re|, |im|) * 2^-e in [1/2, 1)
-__device__ __forceinline__ float sigma_scale(const FrameIO& fr, int scaled) {
-  if (!scaled) return 1.f;
-  const float m = __uint_as_float((unsigned)fr.meta[1]);
-  return m > 0.f ? ldexpf(1.f, -(ilogbf(m) + 1)) : 1.f;
-}
-
-// Warp-collective wait: all lanes poll, the decision is made uniform.
-__device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
-  return __all_sync(0xffffffffu, mbar_wait(b, parity, sh, status));
 }
 
 // Next work unit id from the ring filled by the pixel loader (-1: no more work).
@@ -451,7 +253,7 @@ build_b_images(const FrameIO* __restrict__ frames, Consts k, int NT, int ntiles,
     const FrameIO& fr = frames[it / (nch * ntiles)];
     const int64_t pv = (int64_t)fr.meta[0];
     if (c * kChunkPx >= pv) continue;
-    const float sc = sigma_scale(fr, scaled);
+    const float2 sc = pow2_factors(scaled ? -sigma_exponent(fr.meta[1]) : 0);
     unsigned char* base = fr.bimg + ((int64_t)nt * fr.bimg_nch + c) * 2 * part;
     const int64_t q0c = c * kChunkPx;
     // element (l, 16-byte column cp): four pixels' D at l, written to the re-row l and
@@ -465,8 +267,8 @@ build_b_images(const FrameIO* __restrict__ frames, Consts k, int NT, int ntiles,
     const float4 s01 = *reinterpret_cast<const float4*>(fr.sig + q0);
     const float4 s23 = *reinterpret_cast<const float4*>(fr.sig + q0 + 2);
     const uint32_t bv[4] = {b4.x, b4.y, b4.z, b4.w};
-    const float sa[4] = {s01.x * sc, s01.z * sc, s23.x * sc, s23.z * sc};
-    const float sb[4] = {s01.y * sc, s01.w * sc, s23.y * sc, s23.w * sc};
+    const float sa[4] = {s01.x * sc.x * sc.y, s01.z * sc.x * sc.y, s23.x * sc.x * sc.y, s23.z * sc.x * sc.y};
+    const float sb[4] = {s01.y * sc.x * sc.y, s01.w * sc.x * sc.y, s23.y * sc.x * sc.y, s23.w * sc.x * sc.y};
     for (int e = threadIdx.x; e < NT * 8; e += blockDim.x) {
       const int row = e >> 3;
       const int l = nt * NT + row;
@@ -497,13 +299,13 @@ build_b_images(const FrameIO* __restrict__ frames, Consts k, int NT, int ntiles,
   }
 }
 
-template <int BF, int SPLIT>
+template <int BF>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, int out_dtype,
               unsigned* status, int* unit_counter) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* bstage = smem;  // kStages x (hi, lo) x 32 KB, 1024-aligned
+  unsigned char* bstage = smem;  // kStages x 32 KB, 1024-aligned
   PixStage* pix = (PixStage*)(smem + kStages * kStageBytes);
   Shared* sh = (Shared*)(pix + kPixStages);
 
@@ -567,7 +369,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
     struct Pending {
       const FrameIO* fr;
       int64_t gr;
-      float oscale;
+      float2 oscale;
       int l0, s, mt, nt;
       bool row_ok, none, first, set;
     };
@@ -600,12 +402,13 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
             const int64_t o = d.gr * k.L + l;
             if (out_dtype == RSIM_C128) {
               double2* cd = reinterpret_cast<double2*>(dfr.cube);
-              cd[o] = make_double2((double)a0 * d.oscale, (double)b0 * d.oscale);
-              if (two) cd[o + 1] = make_double2((double)a1 * d.oscale, (double)b1 * d.oscale);
+              cd[o] = make_double2((double)(a0 * d.oscale.x * d.oscale.y), (double)(b0 * d.oscale.x * d.oscale.y));
+              if (two)
+                cd[o + 1] = make_double2((double)(a1 * d.oscale.x * d.oscale.y), (double)(b1 * d.oscale.x * d.oscale.y));
             } else {
               float2* cf = reinterpret_cast<float2*>(dfr.cube);
-              cf[o] = make_float2(a0 * d.oscale, b0 * d.oscale);
-              if (two) cf[o + 1] = make_float2(a1 * d.oscale, b1 * d.oscale);
+              cf[o] = make_float2(a0 * d.oscale.x * d.oscale.y, b0 * d.oscale.x * d.oscale.y);
+              if (two) cf[o + 1] = make_float2(a1 * d.oscale.x * d.oscale.y, b1 * d.oscale.x * d.oscale.y);
             }
           }
         } else {
@@ -644,7 +447,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
       const int vl = row_ok ? v - x.v_first : 0;
       const uint32_t* pA = fr.phA + (int64_t)(row_ok ? v : 0) * fr.Pcap;
       const uint32_t* pC = fr.phC + (int64_t)(row_ok ? v : 0) * fr.Pcap;
-      const float oscale = 1.f / sigma_scale(fr, scaled);
+      const float2 oscale = sigma_unscale(fr, scaled);
       const int l0 = x.nt * g.NT;
       const int64_t ngr = unit_groups(x, g.group);
       for (int64_t gk = 0; gk < ngr; ++gk) {
@@ -658,7 +461,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
             alive = false;
             break;
           }
-          uint32_t hi[kAPx], lo[kAPx];
+          uint32_t hi[kAPx];
           const int j0 = part * kAPx;
           const int64_t q0 = c * kChunkPx + j0;
 #pragma unroll
@@ -676,15 +479,14 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
               const float2 f = cis_q32_fast(av[t] * n + cv[t]);
-              split2<BF>(f.x, f.y, hi[j4 + t], lo[j4 + t]);
+              hi[j4 + t] = pack2<BF>(f.x, f.y);
             }
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(&sh->pix_empty[ps]);
-          static_assert(kAPx == 16, "one x16 tensor-memory store per operand part");
-          const uint32_t col = tmem + lane_base + kAccCols + st * 64 + j0;
+          static_assert(kAPx == 16, "one x16 tensor-memory store per stage");
+          const uint32_t col = tmem + lane_base + kAccCols + st * 32 + j0;
           tmem_st16(col, hi);
-          if (SPLIT) tmem_st16(col + 32, lo);
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           fence_before();
           mbar_arrive(&sh->a_full[st]);
@@ -715,7 +517,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
       uint32_t kk = 0, gi = 0, ui = 0;
       long long u;
       bool alive = true;
-      const uint64_t desc0 = sdesc_sw128(smem_u32(bstage));  // hi image of B stage 0
+      const uint64_t desc0 = sdesc_sw128(smem_u32(bstage));  // B stage 0
       while (alive && next_unit(sh, ui++, status, &u, false)) {
         const Unit x = decode(g, frames, k, u);
         const int64_t ngr = unit_groups(x, g.group);
@@ -730,14 +532,14 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
           for (int64_t c = g0; c < g1; ++c, ++kk) {
             const uint32_t sa = kk % kAStages, pa = (kk / kAStages) & 1u;
             const uint32_t sb = kk % kStages, pb = (kk / kStages) & 1u;
-            if (!mbar_wait_fast(&sh->a_full[sa], pa, sh, status) ||
-                !mbar_wait_fast(&sh->b_full[sb], pb, sh, status)) {
+            if (!mbar_wait(&sh->a_full[sa], pa, sh, status) ||
+                !mbar_wait(&sh->b_full[sb], pb, sh, status)) {
               alive = false;
               break;
             }
             fence_after();
-            mma_stage<SPLIT>(tmem, tmem + kAccCols + sa * 64, desc0 + (uint64_t)(sb * (kStageBytes >> 4)),
-                             idesc, accum);
+            mma_stage(tmem, tmem + kAccCols + sa * 32, desc0 + (uint64_t)(sb * (kStageBytes >> 4)), idesc,
+                      accum);
             accum = 1;
             mma_commit(&sh->a_empty[sa]);
             mma_commit(&sh->b_empty[sb]);
@@ -809,9 +611,8 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
           }
           const unsigned char* src = fr.bimg + ((int64_t)x.nt * fr.bimg_nch + c) * 2 * part;
           unsigned char* dst = bstage + st * kStageBytes;
-          mbar_expect_tx(&sh->b_full[st], SPLIT ? 2 * part : part);
+          mbar_expect_tx(&sh->b_full[st], part);
           bulk_g2s_hint(dst, src, part, &sh->b_full[st], pol_b);
-          if (SPLIT) bulk_g2s_hint(dst + kBBytes, src + part, part, &sh->b_full[st], pol_b);
         }
       }
     }
@@ -841,7 +642,7 @@ __global__ void order_frames(const FrameIO* __restrict__ frames, int F, int32_t*
 }
 
 template <int BF, int SPLIT>
-cudaError_t launch_t(const Consts& k, const FrameIO* frames, Geo g, int grid, int num_sms, int scaled,
+cudaError_t launch_t(const Consts& k, const FrameIO* frames, Geo g, int grid, int num_sms, int scaled, bool fine,
                      int out_dtype, int64_t nch_max, int fast_dtype, unsigned* status, int* counter,
                      cudaStream_t st, cudaEvent_t mid) {
   cudaError_t e;
@@ -858,25 +659,19 @@ cudaError_t launch_t(const Consts& k, const FrameIO* frames, Geo g, int grid, in
     if (e != cudaSuccess) return e;
   }
   if (mid) cudaEventRecord(mid, st);
+  if (SPLIT)
+    return launch_umma_pairs(BF, fine, k, frames, g.F, g.splits, g.NT, g.group, g.direct == 0, grid, num_sms,
+                             nch_max, scaled, out_dtype, g.order, status, st);
   const int smem = kStages * kStageBytes + kPixStages * (int)sizeof(PixStage) + (int)sizeof(Shared) + 1024;
-  auto fn = umma_contract<BF, SPLIT>;
+  auto fn = umma_contract<BF>;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
   // persistent: at most one CTA per SM (shared memory and tensor memory allow no more)
   int ctas = grid > 0 ? std::min(grid, num_sms) : num_sms;
   if (ctas < 1) ctas = 1;
   if (ctas > g.total_units) ctas = (int)g.total_units;
-  cfg.gridDim = dim3(ctas);
-  return cudaLaunchKernelEx(&cfg, fn, frames, k, g, scaled, out_dtype, status, counter);
+  return launch_dependent(fn, dim3(ctas), dim3(kThreads), (size_t)smem, st, frames, k, g, scaled, out_dtype, status,
+                          counter);
 }
 
 }  // namespace
@@ -885,10 +680,11 @@ cudaError_t launch_umma(const Consts& k, const FrameIO* frames, int F, int split
                         int out_dtype, int grid, int nt, int group, bool use_partial, int num_sms,
                         int64_t max_p, int fast_terms_dtype, unsigned* status, int* unit_counter,
                         cudaStream_t st, cudaEvent_t mid) {
-  // N = 2 NT must be a multiple of 16 in 16..256 (kind::f16 with M = 128), and a group
-  // holds at least one chunk
-  if (nt < 8 || nt > kBRowsMax / 2 || nt % 8 != 0 || group < 1) return cudaErrorInvalidValue;
+  // N = 2 NT must be a multiple of 16 in 16..256 (kind::f16 with M = 128; of 32 for pairs,
+  // M = 256), and a group holds at least one chunk
+  if (nt < 8 || nt > kAccCols / 2 || nt % 8 != 0 || group < 1) return cudaErrorInvalidValue;
   Geo g;
+  nt = operand_nt(tier, nt);
   const int64_t rows = (int64_t)k.V * k.Ns;
   g.NT = nt;
   g.ntiles = (k.L + g.NT - 1) / g.NT;
@@ -919,17 +715,18 @@ cudaError_t launch_umma(const Consts& k, const FrameIO* frames, int F, int split
     return cudaErrorInvalidValue;
   switch (tier) {
     case RSIM_TIER_BF16:
-      return launch_t<1, 0>(k, frames, g, grid, num_sms, 0, out_dtype, nch_max, fast_terms_dtype, status, unit_counter, st,
-                          mid);
+      return launch_t<1, 0>(k, frames, g, grid, num_sms, 0, false, out_dtype, nch_max, fast_terms_dtype, status,
+                            unit_counter, st, mid);
     case RSIM_TIER_SPLIT_BF16:
-      return launch_t<1, 1>(k, frames, g, grid, num_sms, 0, out_dtype, nch_max, fast_terms_dtype, status, unit_counter, st,
-                          mid);
+      return launch_t<1, 1>(k, frames, g, grid, num_sms, 0, false, out_dtype, nch_max, fast_terms_dtype, status,
+                            unit_counter, st, mid);
     case RSIM_TIER_SPLIT_FP16:
-      return launch_t<0, 1>(k, frames, g, grid, num_sms, 1, out_dtype, nch_max, fast_terms_dtype, status, unit_counter, st,
-                          mid);
+    case kTierFp32Tensor:
+      return launch_t<0, 1>(k, frames, g, grid, num_sms, 1, tier == kTierFp32Tensor, out_dtype, nch_max,
+                            fast_terms_dtype, status, unit_counter, st, mid);
     case RSIM_TIER_FP16:
-      return launch_t<0, 0>(k, frames, g, grid, num_sms, 1, out_dtype, nch_max, fast_terms_dtype, status, unit_counter, st,
-                          mid);
+      return launch_t<0, 0>(k, frames, g, grid, num_sms, 1, false, out_dtype, nch_max, fast_terms_dtype, status,
+                            unit_counter, st, mid);
     default:
       return cudaErrorInvalidValue;
   }

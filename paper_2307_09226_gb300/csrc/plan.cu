@@ -8,6 +8,20 @@
 
 namespace rsim {
 
+namespace {
+// The FP32 tier runs on the tensor cores from frames of kFp32TensorPixels pixels on: hi + lo
+// FP16 operands, three products, at most kFp32Group chunks in an accumulator, FP32 sums of
+// those.  At every shape measured it is closer to FP64 than the FP32 sum on the CUDA cores
+// and faster (relative error and time, tensor / CUDA cores):
+//   512 x 512 pixels, V = 8,  N_s = 512, L = 256   6.7e-7 / 1.77e-6   2583 / 29370 us
+//   256 x 256,        V = 12, N_s = 256, L = 128   5.6e-7 / 1.27e-6    277 / 2806 us
+//   128 x 128,        V = 8,  N_s = 256, L = 128   3.5e-7 / 6.6e-7      81 / 489 us
+//   32 x 32,          V = 8,  N_s = 64,  L = 32    3.3e-7 / 4.7e-7      31 / 57 us
+// Frames of a few chunks take as long either way (5 x 3 pixels: 25-29 / 26 us).
+constexpr int kFp32Group = 2;
+constexpr int64_t kFp32TensorPixels = 128;
+}  // namespace
+
 int tile_nt(int L) { return L >= 128 ? 128 : ((L + 7) / 8) * 8; }
 
 int64_t tensor_split_stride(int V, int Ns, int L, int nt) {
@@ -18,27 +32,34 @@ int64_t tensor_split_stride(int V, int Ns, int L, int nt) {
 bool uses_partial(int tier, int64_t P, int splits, int group) {
   if (tier == RSIM_TIER_NUFFT) return false;
   if (splits > 1) return true;
-  if (tier == RSIM_TIER_FP32) return false;
+  if (tier == RSIM_TIER_FP32 || pair_tier(tier)) return false;  // they sum groups in registers
   const int64_t chunks = (P + kChunkPx - 1) / kChunkPx;
   return chunks > group;
 }
 
+// Pairs of CTAs read a finished group out beside the next group's MMAs, so that groups of 8
+// chunks take 1% longer than groups of 40 (split-FP16 error 2.0e-6 instead of 8.7e-6).
 int group_chunks(int tier) {
-  return (tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16) ? 40 : 96;
+  if (tier == kTierFp32Tensor) return kFp32Group;
+  return pair_tier(tier) ? 8 : 96;
 }
 
 // The split tiers' 2e-5 bar leaves room for the round-toward-zero bias of at most 40
 // chunks (480 accumulating MMAs, a relative shrink of about 1e-5); the plain 16-bit tiers
 // (1e-2) allow 384 chunks (1536 MMAs, about 3e-5).
 int group_chunks_max(int tier) {
-  return (tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16) ? 40 : 384;
+  if (tier == kTierFp32Tensor) return kFp32Group;
+  return pair_tier(tier) ? 40 : 384;
 }
+
+bool fp32_on_tensor_cores(int64_t P) { return P >= kFp32TensorPixels; }
 
 int units_per_split(int tier, int V, int Ns, int L, int tile_n) {
   if (tier == RSIM_TIER_FP32) return V * ((Ns + tile_n - 1) / tile_n) * ((L + kDirectTileL - 1) / kDirectTileL);
   const int64_t rows = (int64_t)V * Ns;
-  const int nt = (L + tile_n - 1) / tile_n;
-  return (int)(((rows + 127) / 128) * nt);
+  const int nt = operand_nt(tier, tile_n);
+  const int64_t trows = pair_tier(tier) ? 256 : 128;  // a pair of CTAs takes two row tiles
+  return (int)(((rows + trows - 1) / trows) * ((L + nt - 1) / nt));
 }
 
 int default_splits(int tier, int V, int Ns, int L, int tile_n, int64_t P, int num_sms) {
@@ -68,15 +89,17 @@ int default_splits(int tier, int V, int Ns, int L, int tile_n, int64_t P, int nu
     }
     return (int)bs;
   }
-  // tensor tiers: one persistent CTA per SM takes equal units from a counter; pick the
-  // split count whose unit count fills whole rounds of SMs best, with a small cost per
-  // split for the partial buffer it adds
+  // tensor tiers: one persistent CTA (or half a pair) per SM takes equal units in turn; pick
+  // the split count whose unit count fills whole rounds best, with a cost per split for the
+  // partial sums it adds.  A hundredth of the contraction per split: 64 frames of 12 tiles
+  // then take 6 splits instead of 19 (10.40 ms against 11.21), one frame the same time
+  const int slots = std::max(pair_tier(tier) ? num_sms / 2 : num_sms, 1);
   double best = -1.0;
   int bs = 1;
   for (int s = 1; s <= smax; ++s) {
     const int64_t units = (int64_t)tiles * s;
-    const int64_t rounds = (units + num_sms - 1) / num_sms;
-    const double eff = (double)units / (double)(rounds * num_sms) - 0.003 * s;
+    const int64_t rounds = (units + slots - 1) / slots;
+    const double eff = (double)units / (double)(rounds * slots) - 0.01 * s;
     if (eff > best + 1e-9) {
       best = eff;
       bs = s;

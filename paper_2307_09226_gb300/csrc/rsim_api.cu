@@ -141,6 +141,36 @@ rsim_plan choose_plan(rsim_ctx* ctx, int tier, const Consts& k, int64_t P) {
   return default_plan(tier, k, P, ctx->num_sms);
 }
 
+// The arithmetic that runs a call of `tier` over F frames of at most P pixels: `tier` itself,
+// or, for the FP32 tier, the tensor cores where the pixel count says so
+// (fp32_on_tensor_cores), no plan for the CUDA-core kernel is pinned or tuned for the shape's
+// bucket, and one frame's workspace fits tensor_bytes_cap(budget).
+size_t tensor_bytes_cap(size_t budget) { return budget ? std::min(budget, kFp32TensorBytes) : kFp32TensorBytes; }
+
+int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budget) {
+  if (tier != RSIM_TIER_FP32 || !(ctx->cc_major == 10 && ctx->cc_minor == 3) || !fp32_on_tensor_cores(P))
+    return tier;
+  {
+    std::lock_guard<std::mutex> g(ctx->plan_mu);
+    auto it = ctx->plans.find(plan_key(tier, k, P));
+    if (it != ctx->plans.end() && plan_problem(tier, k, it->second).empty()) return tier;
+  }
+  const rsim_plan plan = choose_plan(ctx, kTierFp32Tensor, k, P);
+  return batch_bytes(k, &P, 1, plan, kTierFp32Tensor) > tensor_bytes_cap(budget) ? tier : kTierFp32Tensor;
+}
+
+// A plan as its caller sees it: the tensor-core engine of the FP32 tier shows its splits and
+// grid, and the tier's n tile (128 rows, which it uses too).
+rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int engine) {
+  if (engine == tier) return plan;
+  rsim_plan p{};
+  resolve_tile(tier, k, &p);
+  p.splits = plan.splits;
+  p.grid = plan.grid;
+  p.tuned = plan.tuned;
+  return p;
+}
+
 // Workspace bytes of the per-frame regions of F frames of P_f pixels.
 size_t frames_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& plan, int tier) {
   int64_t mp = 0;
@@ -150,7 +180,8 @@ size_t frames_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& p
   o = align_up(o + 16 * (size_t)F, 256);                  // meta
   o = align_up(o + 16 + 4 * (size_t)F, 256);              // unit counter + frame order
   for (int f = 0; f < F; ++f) {
-    FrameLayout fl = frame_layout(k.V, k.Ns, k.L, P[f], plan.splits, up, tensor_tier(tier), plan.tile_n, o);
+    FrameLayout fl = frame_layout(k.V, k.Ns, k.L, P[f], plan.splits, up, tensor_tier(tier),
+                                  operand_nt(tier, plan.tile_n), o);
     o = fl.total;
   }
   return o;
@@ -253,7 +284,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
                        int out_dtype, const rsim_plan& plan, unsigned* status, cudaStream_t st) {
   std::vector<int64_t> Ps(F);
   for (int f = 0; f < F; ++f) Ps[f] = frames[f].P;
-  static const char* const kTierName[] = {"fp32", "bf16", "split_bf16", "split_fp16", "fp16", "nufft"};
+  static const char* const kTierName[] = {"fp32", "bf16", "split_bf16", "split_fp16", "fp16", "nufft", "fp32 tensor"};
   char what[160];
   snprintf(what, sizeof what, "synth %s F=%d V=%d Ns=%d L=%d P=%lld splits=%d tile=%d", kTierName[tier], F, k.V,
            k.Ns, k.L, (long long)max_P(frames, F), plan.splits, plan.tile_n);
@@ -269,7 +300,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
   FrameIO* table = nullptr;
   int* counter = nullptr;
   rsim_status s = stage_frames(ctx, ws, k, frames, F, cubes, splits, use_partial,
-                               tensor_tier(tier), plan.tile_n, st, host, &table, &counter);
+                               tensor_tier(tier), operand_nt(tier, plan.tile_n), st, host, &table, &counter);
   if (s != RSIM_OK) return s;
   // stage events when profiling this context's own calls
   // ev: start, after compaction + phases, after the contraction, after the reduction,
@@ -363,7 +394,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     if (prof) cudaEventRecord(ev[2], st);
     if (prof) cudaEventRecord(ev[5], st);
     if (use_partial) {
-      e = launch_reduce(k, table, F, splits, out_dtype, 0.f, st);
+      e = launch_reduce(k, table, F, splits, out_dtype, st);
       if (e != cudaSuccess) return cuda_fail(e, "split reduction");
     }
   } else {
@@ -375,8 +406,8 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     if (prof) cudaEventRecord(ev[2], st);
     if (prof) cudaEventRecord(ev[5], st);
     if (use_partial) {
-      const bool scaled = (tier == RSIM_TIER_SPLIT_FP16 || tier == RSIM_TIER_FP16);
-      e = launch_reduce_tiles(k, table, F, splits, plan.tile_n, out_dtype, scaled, ctx->num_sms, st);
+      e = launch_reduce_tiles(k, table, F, splits, operand_nt(tier, plan.tile_n), out_dtype, scaled_tier(tier),
+                              ctx->num_sms, st);
       if (e != cudaSuccess) return cuda_fail(e, "split reduction");
     }
   }
@@ -456,8 +487,9 @@ rsim_status rsim_workspace_size(rsim_ctx* ctx, const rsim_radar_params* params, 
   Consts k;
   rsim_status s = check_params(params, &k);
   if (s != RSIM_OK) return s;
-  rsim_plan plan = choose_plan(ctx, tier, k, P);
-  *bytes = batch_bytes(k, &P, 1, plan, tier);
+  const int engine = engine_tier(ctx, tier, k, P, ctx->budget);
+  rsim_plan plan = choose_plan(ctx, engine, k, P);
+  *bytes = batch_bytes(k, &P, 1, plan, engine);
   return RSIM_OK;
 }
 
@@ -601,9 +633,31 @@ rsim_status rsim_synth_batch(rsim_ctx* ctx, const rsim_radar_params* params,
   cudaStream_t st = (cudaStream_t)stream;
   // the plan of a batch is the plan of its largest frame: every frame uses the same
   // splits rule, so a frame gives the same bits alone and in a batch of equal-P frames
-  rsim_plan plan = choose_plan(ctx, tier, k, maxp);
   std::vector<int64_t> Ps(F);
   for (int f = 0; f < F; ++f) Ps[f] = frames[f].P;
+  const int engine = engine_tier(ctx, tier, k, maxp, ctx->budget);
+  if (engine != tier) {
+    // the FP32 tier on the tensor cores needs more workspace than its CUDA-core kernel (2 KB
+    // a pixel and column tile): a batch beyond the cap runs a few frames at a time (the same
+    // bits), and where the memory cannot be had at all the CUDA-core kernel takes the call
+    // below
+    const size_t cap = tensor_bytes_cap(ctx->budget);
+    const rsim_plan plan = choose_plan(ctx, engine, k, maxp);
+    int done = 0;
+    while (done < F) {
+      int n = F - done;
+      while (n > 1 && batch_bytes(k, Ps.data() + done, n, plan, engine) > cap) n = (n + 1) / 2;
+      s = ensure_workspace(ctx, batch_bytes(k, Ps.data() + done, n, plan, engine), st);
+      if (s == RSIM_ERR_OOM && done == 0) break;
+      if (s == RSIM_OK)
+        s = run_frames(ctx, (char*)ctx->ws, ctx->ws_bytes, k, frames + done, n, cubes + done, engine, out_dtype, plan,
+                       ctx->status_dev, st);
+      if (s != RSIM_OK) return s;
+      done += n;
+    }
+    if (done == F) return RSIM_OK;
+  }
+  rsim_plan plan = choose_plan(ctx, tier, k, maxp);
   const size_t need = batch_bytes(k, Ps.data(), F, plan, tier);
   s = ensure_workspace(ctx, need, st);
   if (s != RSIM_OK) return s;
@@ -768,7 +822,8 @@ rsim_status rsim_get_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_
   Consts k;
   rsim_status s = check_params(params, &k);
   if (s != RSIM_OK) return s;
-  *plan = choose_plan(ctx, tier, k, P);
+  const int engine = engine_tier(ctx, tier, k, P, ctx->budget);
+  *plan = reported_plan(tier, k, choose_plan(ctx, engine, k, P), engine);
   return RSIM_OK;
 }
 

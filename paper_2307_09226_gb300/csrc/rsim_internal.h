@@ -87,7 +87,7 @@ struct FrameLayout {
   size_t idx, phA, phC, phB, sig, blk, meta, partial, bimg, total;
   int64_t Pcap, bimg_nch;
 };
-// nt: the plan's column tile of the tensor tiers (ignored otherwise).
+// nt: operand_nt of the plan's column tile (tensor tiers; ignored otherwise).
 FrameLayout frame_layout(int V, int Ns, int L, int64_t P, int splits, bool use_partial, bool tensor,
                          int nt, size_t base);
 // Default columns of l per tensor-core column tile: min(128, L rounded up to 8).
@@ -97,11 +97,28 @@ int tile_nt(int L);
 // columns], so that a warp's 32 accumulator rows drain into 512 contiguous bytes.
 int64_t tensor_split_stride(int V, int Ns, int L, int nt);
 
-// Tensor-core tiers (the tcgen05 contraction and its operand images).
+// The FP32 tier on the tensor cores (see fp32_on_tensor_cores): internal, beside the tiers of
+// rsim.h.  A call's tier becomes this one where the rule says so.
+constexpr int kTierFp32Tensor = 6;
+
+// Tensor-core tiers (the tcgen05 contractions and their operand images).
 inline bool tensor_tier(int tier) {
   return tier == RSIM_TIER_BF16 || tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16 ||
-         tier == RSIM_TIER_FP16;
+         tier == RSIM_TIER_FP16 || tier == kTierFp32Tensor;
 }
+// Workspace the FP32 tier takes on the tensor cores at most, per call.
+constexpr size_t kFp32TensorBytes = size_t(16) << 30;
+// Those of hi + lo operands, which run on pairs of CTAs.
+inline bool pair_tier(int tier) {
+  return tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16 || tier == kTierFp32Tensor;
+}
+// Those whose sigma is scaled by a power of two into FP16's range.
+inline bool scaled_tier(int tier) {
+  return tier == RSIM_TIER_SPLIT_FP16 || tier == RSIM_TIER_FP16 || tier == kTierFp32Tensor;
+}
+// Columns of l that a plan's column tile takes up in the operand images and the accumulator
+// (a pair's MMA has N = 2 NT, a multiple of 32).
+inline int operand_nt(int tier, int nt) { return pair_tier(tier) ? (nt + 15) / 16 * 16 : nt; }
 
 // NUFFT tier: grid and tile geometry of one frame shape.
 struct NuGeo {
@@ -220,6 +237,18 @@ __device__ __forceinline__ uint64_t frac_u64(double x) {
   return (bits >> 63) ? (uint64_t)0 - f : f;
 }
 
+// The power of two 2^-e that the FP16 tiers scale sigma by puts max(|re|, |im|) (its float
+// bits: meta[1]) into [2^14, 2^15): every component stays below FP16's largest number, and
+// pixels down to 2^-29 of the strongest keep all their bits.  Applied as two factors, so that
+// no factor leaves FP32's range; exact.
+__device__ __forceinline__ int sigma_exponent(unsigned long long max_bits) {
+  const float m = __uint_as_float((unsigned)max_bits);
+  return m > 0.f ? ilogbf(m) - 14 : 0;
+}
+__device__ __forceinline__ float2 pow2_factors(int e) {
+  return make_float2(ldexpf(1.f, e / 2), ldexpf(1.f, e - e / 2));
+}
+
 // Round a 2^-64 fixed-point fraction to the nearest 2^-32 unit (mod 1).
 __device__ __forceinline__ uint32_t top32(uint64_t x) {
   return (uint32_t)((x + 0x80000000ull) >> 32);
@@ -274,7 +303,7 @@ cudaError_t launch_prep(const Consts& k, FrameIO* frames, const FrameIO* one, in
 cudaError_t launch_direct(const Consts& k, const FrameIO* frames, int F, int splits, int tile_n,
                           int out_dtype, cudaStream_t st);
 cudaError_t launch_reduce(const Consts& k, const FrameIO* frames, int F, int splits, int out_dtype,
-                          float scale_from_meta, cudaStream_t st);
+                          cudaStream_t st);
 // The same reduction over the tensor tiers' tiled partial sums.
 cudaError_t launch_reduce_tiles(const Consts& k, const FrameIO* frames, int F, int splits, int nt,
                                 int out_dtype, bool scale_from_meta, int num_sms, cudaStream_t st);
@@ -290,6 +319,12 @@ cudaError_t launch_umma(const Consts& k, const FrameIO* frames, int F, int split
 
 // cubes: HOST array of the F cube pointers; cubes_dev: the same on the device, or NULL to pass
 // them by value (F <= 64).
+// The contraction of the pair tiers (launch_umma calls it).  nch_max: chunks of the largest
+// frame; fine: the FP32 tier's phase arithmetic; order: device array, or NULL for one frame.
+cudaError_t launch_umma_pairs(int bf16, bool fine, const Consts& k, const FrameIO* frames, int F, int splits, int nt,
+                              int group, bool use_partial, int grid, int num_sms, int64_t nch_max, int scaled,
+                              int out_dtype, const int32_t* order, unsigned* status, cudaStream_t st);
+
 cudaError_t launch_range_doppler(const float2* const* cubes, const float2* const* cubes_dev, float2* tmp, float* power,
                                  int F, int V, int Ns, int L, int skip_static, double v_per_bin, float* v_est,
                                  int32_t* peak, int num_sms, cudaStream_t st);
@@ -303,6 +338,8 @@ int units_per_split(int tier, int V, int Ns, int L, int tile_n);
 // the length bounds the error; see k_umma.cu).
 int group_chunks(int tier);
 int group_chunks_max(int tier);
+// Whether a frame of the FP32 tier runs on the tensor cores: a rule on its pixel count.
+bool fp32_on_tensor_cores(int64_t P);
 // Default n tile of the FP32 direct sum, and its l tile (fixed).
 constexpr int kDirectTileN = 128;
 constexpr int kDirectTileL = 64;

@@ -48,6 +48,7 @@ struct Req {
   Consts k{};
   rsim_plan plan{};
   size_t bytes = 0;
+  int engine = 0;  // the arithmetic that runs it (engine_tier)
   int state = kQueued;
   rsim_status result = RSIM_OK;
   Clock::time_point t_submit, t_admit, t_done;
@@ -232,7 +233,7 @@ bool admit_one(rsim_server* s) {
   char what[64];
   snprintf(what, sizeof what, "request %llu", (unsigned long long)r.ticket);
   NvtxRange request_range(what);
-  rsim_status st = run_frames(s->ctx, (char*)r.ws, r.bytes, r.k, &r.r.pixels, 1, cubes, r.r.tier,
+  rsim_status st = run_frames(s->ctx, (char*)r.ws, r.bytes, r.k, &r.r.pixels, 1, cubes, r.engine,
                               r.r.out_dtype, r.plan, sl.status, rs);
   // P_valid of this request, read by retire() once the stream reaches it
   size_t o = ((sizeof(FrameIO) + 255) / 256) * 256;
@@ -344,13 +345,14 @@ rsim_status rsim_server_submit(rsim_server* s, const rsim_request* req, uint64_t
   if (!req->cube) return fail(RSIM_ERR_INVALID_ARG, "cube is NULL");
   if (tensor_tier(req->tier) && !(s->ctx->cc_major == 10 && s->ctx->cc_minor == 3))
     return fail(RSIM_ERR_UNSUPPORTED, "tensor-core tiers need an sm_103 device");
-  r.plan = choose_plan(s->ctx, req->tier, r.k, req->pixels.P);
   int64_t P = req->pixels.P;
-  r.bytes = batch_bytes(r.k, &P, 1, r.plan, req->tier);
+  r.engine = engine_tier(s->ctx, req->tier, r.k, P, s->opts.hbm_budget_bytes);
+  r.plan = choose_plan(s->ctx, r.engine, r.k, P);
+  r.bytes = batch_bytes(r.k, &P, 1, r.plan, r.engine);
   // estimated device time from the path-samples at the tier's nominal rate (CUDA cores
   // about 6e12/s, tensor cores and the NUFFT about 6e13/s): high priority under 2 ms
   const double work = (double)req->pixels.P * r.k.V * r.k.Ns * r.k.L;
-  r.est_ms = work / (req->tier == RSIM_TIER_FP32 ? 6e12 : 6e13) * 1e3;
+  r.est_ms = work / (r.engine == RSIM_TIER_FP32 ? 6e12 : 6e13) * 1e3;
   r.prio = r.est_ms < 2.0 ? 0 : 1;
   std::lock_guard<std::mutex> g(s->mu);
   if (s->opts.hbm_budget_bytes && r.bytes > s->opts.hbm_budget_bytes)

@@ -73,18 +73,31 @@ extern "C" rsim_status rsim_synth_static(const rsim_radar_params* params, const 
     return fail(RSIM_ERR_UNSUPPORTED, "tensor-core tiers need an sm_103 device");
 
   // the plan is the library's default rule for this shape (what rsim_synth uses
-  // without a tuned plan); the scratch layout mirrors the context workspace
+  // without a tuned plan); the scratch layout mirrors the context workspace.  The FP32 tier
+  // runs on the tensor cores under rsim_synth's rule where that fits the array, else on the
+  // CUDA cores
   const int64_t P = pixels->P;
-  const rsim_plan plan = default_plan(tier, k, P, sms);
-  const int splits = plan.splits;
-  const bool use_partial = uses_partial(tier, P, splits, plan.group_chunks);
-  size_t o = 0;
-  const size_t off_table = o;   o = up256(o + sizeof(FrameIO));
-  const size_t off_meta = o;    o = up256(o + 16);
-  const size_t off_counter = o; o = up256(o + 16 + 4);
-  FrameLayout fl = frame_layout(k.V, k.Ns, k.L, P, splits, use_partial, tensor_tier(tier), plan.tile_n, o);
-  o = fl.total;
-  const size_t off_status = o;  o = up256(o + 4);
+  int engine = tier;
+  if (tier == RSIM_TIER_FP32 && major == 10 && minor == 3 && fp32_on_tensor_cores(P)) engine = kTierFp32Tensor;
+  rsim_plan plan{};
+  FrameLayout fl{};
+  size_t off_meta = 0, off_counter = 0, off_status = 0, o = 0;
+  int splits = 1, nt = 0;
+  bool use_partial = false;
+  for (;;) {
+    plan = default_plan(engine, k, P, sms);
+    splits = plan.splits;
+    nt = operand_nt(engine, plan.tile_n);
+    use_partial = uses_partial(engine, P, splits, plan.group_chunks);
+    o = up256(sizeof(FrameIO));  // the frame table comes first
+    off_meta = o;    o = up256(o + 16);
+    off_counter = o; o = up256(o + 16 + 4);
+    fl = frame_layout(k.V, k.Ns, k.L, P, splits, use_partial, tensor_tier(engine), nt, o);
+    o = fl.total;
+    off_status = o;  o = up256(o + 4);
+    if (o <= kStaticWsBytes || engine == tier) break;
+    engine = tier;
+  }
   if (o > kStaticWsBytes)
     return fail(RSIM_ERR_BUDGET, "frame needs " + std::to_string(o) +
                                      " bytes of scratch; the static workspace holds " +
@@ -114,10 +127,10 @@ extern "C" rsim_status rsim_synth_static(const rsim_radar_params* params, const 
   io.blk_count = (int32_t*)(ws + fl.blk);
   io.meta = (unsigned long long*)(ws + off_meta);
   io.partial = use_partial ? (float2*)(ws + fl.partial) : nullptr;
-  io.bimg = tensor_tier(tier) ? (unsigned char*)(ws + fl.bimg) : nullptr;
+  io.bimg = tensor_tier(engine) ? (unsigned char*)(ws + fl.bimg) : nullptr;
   io.bimg_nch = fl.bimg_nch;
   io.splits = splits;
-  FrameIO* table = (FrameIO*)(ws + off_table);
+  FrameIO* table = (FrameIO*)ws;
   int* counter = (int*)(ws + off_counter);
 
   // the array keeps the previous call's contents: the first kernel stores the frame
@@ -125,20 +138,19 @@ extern "C" rsim_status rsim_synth_static(const rsim_radar_params* params, const 
   if (!device_status) e = cudaMemsetAsync(status, 0, 4, st);
   if (e != cudaSuccess) return cuda_fail(e, "static workspace set-up");
 
-  const bool defer = tensor_tier(tier);  // the operand builder computes the fast-time phases
+  const bool defer = tensor_tier(engine);  // the operand builder computes the fast-time phases
   e = launch_prep(k, table, &io, 1, P, pixels->dtype, false, defer, status, counter, st, false);
   if (e != cudaSuccess) return cuda_fail(e, "prep kernels");
-  if (tier == RSIM_TIER_FP32) {
+  if (engine == RSIM_TIER_FP32) {
     e = launch_direct(k, table, 1, splits, plan.tile_n, out_dtype, st);
     if (e != cudaSuccess) return cuda_fail(e, "direct-sum kernel");
-    if (use_partial) e = launch_reduce(k, table, 1, splits, out_dtype, 0.f, st);
+    if (use_partial) e = launch_reduce(k, table, 1, splits, out_dtype, st);
   } else {
-    e = launch_umma(k, table, 1, splits, tier, out_dtype, 0, plan.tile_n, plan.group_chunks, use_partial, sms,
+    e = launch_umma(k, table, 1, splits, engine, out_dtype, 0, plan.tile_n, plan.group_chunks, use_partial, sms,
                     P, pixels->dtype, status, counter, st);
     if (e == cudaErrorNotSupported) return fail(RSIM_ERR_UNSUPPORTED, "tensor-core tier not available");
     if (e != cudaSuccess) return cuda_fail(e, "tcgen05 contraction kernel");
-    const bool scaled = (tier == RSIM_TIER_SPLIT_FP16 || tier == RSIM_TIER_FP16);
-    if (use_partial) e = launch_reduce_tiles(k, table, 1, splits, plan.tile_n, out_dtype, scaled, sms, st);
+    if (use_partial) e = launch_reduce_tiles(k, table, 1, splits, nt, out_dtype, scaled_tier(engine), sms, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "split reduction");
   return RSIM_OK;

@@ -131,13 +131,14 @@ void load_plan_cache(rsim_ctx* ctx) {
 using namespace rsim;
 
 extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* params, int64_t P,
-                                     rsim_tier tier, rsim_plan* chosen, rsim_stream stream) {
+                                     rsim_tier asked, rsim_plan* chosen, rsim_stream stream) {
   if (!ctx || !chosen) return fail(RSIM_ERR_INVALID_ARG, "NULL argument");
-  if (!tier_ok(tier)) return fail(RSIM_ERR_INVALID_ARG, "unknown tier");
+  if (!tier_ok(asked)) return fail(RSIM_ERR_INVALID_ARG, "unknown tier");
   if (P < 1) return fail(RSIM_ERR_INVALID_ARG, "P must be >= 1");
   Consts k;
   rsim_status s = check_params(params, &k);
   if (s != RSIM_OK) return s;
+  const int tier = engine_tier(ctx, asked, k, P, ctx->budget);  // the arithmetic that runs the shape
   cudaSetDevice(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
 
@@ -233,7 +234,7 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
   // 3. the accumulation-group length (tensor tiers), never above the tier's cap
   if (tensor) {
     const int gmax = group_chunks_max(tier);
-    std::vector<int> cand = (tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16)
+    std::vector<int> cand = pair_tier(tier)
                                 ? std::vector<int>{32, gmax}
                                 : std::vector<int>{192, gmax};
     const rsim_plan base = best;
@@ -262,6 +263,6 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
     ctx->plans[plan_key(tier, k, P)] = best;
     save_plan_cache(ctx);
   }
-  *chosen = best;
+  *chosen = reported_plan(asked, k, best, tier);
   return RSIM_OK;
 }
