@@ -80,7 +80,7 @@ struct rsim_server {
   std::deque<uint64_t> queue;
   std::map<uint64_t, rsim::Req> reqs;
   std::mutex mu;
-  std::condition_variable cv_sched, cv_done;
+  std::condition_variable cv_done;
   std::thread sched;
   bool stop = false;
   uint64_t next_ticket = 1;
@@ -99,10 +99,23 @@ struct rsim_server {
   // that host function) would never return.
   std::mutex cb_mu;
   std::vector<int> completed_slots;
+  // What the scheduler sleeps on: `wakes` counts submissions, completions and the stop, under
+  // cb_mu, so that none is missed between its look at the queue and its sleep (a notification
+  // outside the lock could be, and cost a whole 50 ms poll).
+  std::condition_variable cv_wake;
+  uint64_t wakes = 0;
 };
 
 namespace rsim {
 namespace {
+
+void wake_scheduler(rsim_server* s) {
+  {
+    std::lock_guard<std::mutex> g(s->cb_mu);
+    s->wakes++;
+  }
+  s->cv_wake.notify_one();
+}
 
 struct HostFnArg {
   rsim_server* s;
@@ -116,8 +129,9 @@ void CUDART_CB on_complete(void* p) {
   {
     std::lock_guard<std::mutex> g(s->cb_mu);
     s->completed_slots.push_back(a->slot);
+    s->wakes++;
+    s->cv_wake.notify_one();  // under the lock: the server may be gone once the scheduler has seen the slot
   }
-  s->cv_sched.notify_all();  // a missed wake-up costs at most the scheduler's 50 ms poll
   delete a;
 }
 
@@ -258,9 +272,11 @@ void scheduler(rsim_server* s) {
   while (true) {
     bool progressed = false;
     std::vector<int> done;
+    uint64_t seen;
     {
       std::lock_guard<std::mutex> g(s->cb_mu);
       done.swap(s->completed_slots);
+      seen = s->wakes;
     }
     for (int si : done) {
       retire(s, si);
@@ -273,7 +289,13 @@ void scheduler(rsim_server* s) {
       std::lock_guard<std::mutex> g(s->cb_mu);
       if (s->completed_slots.empty()) break;
     }
-    s->cv_sched.wait_for(lk, std::chrono::milliseconds(50));
+    lk.unlock();
+    {
+      // the poll is for the age limit of queued requests
+      std::unique_lock<std::mutex> g(s->cb_mu);
+      s->cv_wake.wait_for(g, std::chrono::milliseconds(50), [&] { return s->wakes != seen; });
+    }
+    lk.lock();
   }
 }
 
@@ -368,7 +390,7 @@ rsim_status rsim_server_submit(rsim_server* s, const rsim_request* req, uint64_t
   *ticket = r.ticket;
   s->reqs[r.ticket] = r;
   s->queue.push_back(r.ticket);
-  s->cv_sched.notify_all();
+  wake_scheduler(s);
   return RSIM_OK;
 }
 
@@ -450,7 +472,7 @@ rsim_status rsim_server_destroy(rsim_server* s) {
     }
     s->queue.clear();
   }
-  s->cv_sched.notify_all();
+  wake_scheduler(s);
   if (s->sched.joinable()) s->sched.join();
   cudaSetDevice(s->ctx->device);
   for (Slot& sl : s->slots) {
