@@ -111,3 +111,16 @@ def test_rendered_walking_frame_synthesises_and_sees_the_walker(ctx):
     r = radar.resolved()
     bin_v = r.lam / (2 * r.t_slow * r.L)
     assert abs(float(v_est.item()) - truth["closing_speed"]) <= 2 * bin_v + 0.35
+
+
+@pytest.mark.parametrize("n_az,n_el", [(1, 1), (1, 300), (3, 90), (31, 9), (32, 8), (33, 9), (300, 1)])
+@pytest.mark.parametrize("n_prims", [24, 25])
+def test_image_tiles_and_primitives_by_value(ctx, n_az, n_el, n_prims):
+    """Images narrower than a tile, exactly one tile and ragged, with as many primitives as
+    travel in the kernel's arguments and one more: FP64 as in the tests above."""
+    scene = synth.random_scene(seed=13, n_prims=n_prims)
+    got = _host(ctx.raycast(scene, n_az, n_el, FOV, dtype=torch.float64))
+    want = rc.raycast(scene, n_az, n_el, *FOV)
+    np.testing.assert_array_equal(got["az"], want["az"])
+    np.testing.assert_array_equal(got["el"], want["el"])
+    _compare(scene, got, want, 1e-11, 1e-9, 1e-9, max_ambiguous=0.03)
