@@ -14,29 +14,45 @@
 // Fourier transform Psi_x(n') Psi_y(l'), is the cube (relative error ~10^-(w-1): ~1e-6
 // at w = 7).
 //
+// The channels' positions of one pixel differ little (x_p by v k_da u_p), so the pixels are
+// sorted once for a group of channels whose positions lie within one cell of one another
+// (all of them for the radars in use), and every channel of the group walks the same order.
+//
 // Kernels, per frame:
-//   nu_bin_count  each (channel, point) is binned by the 32 x 32 grid tile of its
-//                 nearest cell: a shared-memory histogram per block of one channel's
-//                 points, one global addition per (block, bin).  An extra row of blocks
-//                 builds the geometry's tables: 1 / (Psi_x(n') Psi_y(l')) (one warp per
-//                 mode, a 128-node midpoint rule of Psi(k) = (w/2) int phi(z) cos(pi k w z
-//                 / G) dz) and the twiddles of both FFTs.  The last counting block scans
-//                 the counts and cuts every bin into work items of 512 records;
-//   nu_bin_fill   records (x, y, q') stored bin by bin (one global reservation per
-//                 (block, bin), ranks within the block from shared memory);
-//   nu_spread     persistent CTAs take the work items in turn; a warp takes one record
-//                 at a time, lane k adding tap k of its w x w taps into a shared-memory tile
-//                 with a w/2 halo, as fixed-point integers (each term split in
-//                 16-bit halves summed by non-returning 32-bit atomics), then the tile is
-//                 added into the global 64-bit integer grid.  Integer sums are exact and do
-//                 not depend on the order of the atomic additions, so the result is
-//                 bit-reproducible.  The work items share the crowded tiles among many SMs:
-//                 a scene fills only the part of the grid that its ranges and speeds reach;
+//   nu_bin_count  each pixel is binned by the 32 x 32 grid tile of its nearest cell in the
+//                 group's first channel: a shared-memory histogram per block, one global
+//                 addition per (block, bin).  Extra blocks build the geometry's tables:
+//                 1 / (Psi_x(n') Psi_y(l')) (one warp per mode, a 128-node midpoint rule of
+//                 Psi(k) = (w/2) int phi(z) cos(pi k w z / G) dz) and the twiddles of both
+//                 FFTs.  The last counting block scans the counts and cuts every bin into
+//                 sorting and spreading items;
+//   nu_bin_fill   (cell, pixel) pairs stored bin by bin (one global reservation per (block,
+//                 bin), ranks within the block from shared memory).  Extra blocks clear the
+//                 grid rows that some bin reaches, and mark them;
+//   nu_sort       a block counting-sorts up to 8192 pixels of a bin by cell (and quarter of a
+//                 cell along x);
+//   nu_spread     persistent CTAs take (1024 sorted pixels, channel) units in turn; a warp takes
+//                 one pixel at a time, lane k holding tap k of its w x w taps.  Successive
+//                 pixels of one cell are summed in registers and leave for a shared-memory
+//                 tile with a halo when the cell changes, as fixed-point integers (each term
+//                 split in 16-bit halves summed by non-returning 32-bit atomics), then the
+//                 tile is added into the global 64-bit integer grid.  Integer sums are exact
+//                 and do not depend on the order of the additions, so the result is
+//                 bit-reproducible.  The units share the crowded tiles among many SMs: a scene
+//                 fills only the part of the grid that its ranges and speeds reach;
 //   nu_fft_y      rows of the grid: integer -> float, Stockham inverse-sign FFT over the
 //                 slow-time axis (radix-16 passes in registers, shared memory between
 //                 passes), only the L centred modes kept;
 //   nu_fft_x      columns: the same over the fast-time axis, only the N_s centred modes
 //                 kept, times the deconvolution factors, written to the cube.
+// Measured (V = 12, N_s = 256, L = 128, w = 7), before and after the pixels were sorted for all
+// channels: a frame of 256 x 256 pixels 99.3 -> 93.6 us, 64 walking frames 2956 -> 2487 us, the
+// same bits.  Before, every (channel, pixel) was binned as a 16-byte record (21 us of the
+// frame's time, now 18 with the sort), each tap went to the tile by atomics of its own, and the
+// whole grid was cleared.  The spreading (45 us, 68% of the issue slots) is bound by its
+// instructions, 57 a pixel and channel.  Not kept: 64-bit register sums by wide multiply-adds
+// (56 us), three blocks of 40 registers per SM (59 us), items of 2048 or 4096 pixels (frame
+// +7 and +15 us, the 64 frames -4 and -7%).
 #include <math.h>
 
 #include <algorithm>
@@ -51,14 +67,19 @@ constexpr int kNWMin = 4, kNWMax = 8;       // kernel widths in cells (the defau
 constexpr float kNBetaPerW = 2.30f;         // ES shape beta = 2.30 w for an oversampling of 2
 constexpr int kNTile = 32;                  // grid cells per tile side
 constexpr int kNQuad = 128;                 // midpoint nodes for Psi
-constexpr int kSpreadChunk = 512;           // records per spreading work item
-constexpr int kBinThreads = 256;            // binning blocks: one channel, kBinItems points
+constexpr int kSpreadChunk = 1024;          // sorted pixels per spreading work item
+constexpr int kSortChunk = 8192;            // pixels a block sorts (whole spreading items)
+constexpr int kSortThreads = 1024;
+constexpr int kSortFrom = 12288;            // pixels of the frames that are sorted (see launch_nufft)
+constexpr int kSub = 4;                     // sort keys per cell: the quarter along x
+static_assert(kSortChunk % kSpreadChunk == 0 && kSortChunk % kSortThreads == 0, "sorting items");
+constexpr int kBinThreads = 256;            // binning blocks: one group, kBinItems pixels
 constexpr int kBinItems = 4 * kBinThreads;
 static_assert(kBinThreads % 32 == 0 && kBinThreads <= 1024, "binning blocks are whole warps");
 
+// A binned pixel: its sort key (cell within the tile, then quarter of the cell) and index.
 struct NuRec {
-  uint32_t x, y;  // positions, 2^-32 cycles
-  float2 q;       // shifted strength q'
+  uint32_t key, q;
 };
 
 // FFT of length n = 2^k (16 <= n <= 4096) along one grid axis: T = n / 16 threads per
@@ -93,12 +114,13 @@ __device__ __forceinline__ void nearest_cell(uint32_t xq, int G, int& c, float& 
   d = (float)(uint32_t)s * 2.3283064365386963e-10f - 0.5f;  // frac(X + 1/2) - 1/2
 }
 
-// Channel-local bin (tile) of a point's nearest cell.
-__device__ __forceinline__ int bin_of(uint32_t xq, uint32_t yq, const NuGeo& g) {
+// Bin (tile) of a point's nearest cell, and its sort key within the tile.
+__device__ __forceinline__ int bin_of(uint32_t xq, uint32_t yq, const NuGeo& g, uint32_t* key = nullptr) {
   int cx, cy;
-  float d;
-  nearest_cell(xq, g.Gx, cx, d);
-  nearest_cell(yq, g.Gy, cy, d);
+  float dx, dy;
+  nearest_cell(xq, g.Gx, cx, dx);
+  nearest_cell(yq, g.Gy, cy, dy);
+  if (key) *key = (uint32_t)(((cx % g.Tx) * g.Ty + cy % g.Ty) * kSub) + min(kSub - 1, (int)((dx + 0.5f) * kSub));
   return (cx / g.Tx) * g.nty + cy / g.Ty;
 }
 
@@ -119,17 +141,12 @@ __device__ __forceinline__ float grid_scale(const FrameIO& fr, bool inverse) {
   return inverse ? ldexpf(m, -30) : ldexpf(1.f, 30) / m;
 }
 
-// Add a 32-bit signed term v to a sum kept as two 32-bit words with non-returning
-// atomics: `lo` takes v itself (wrapping mod 2^32) and `hi` its signed high part
-// v >> 16.  With H = sum of (v >> 16) and LO = sum of v mod 2^32, the sum of the low
-// halves v & 0xffff is (LO - H 2^16) mod 2^32, and the exact sum is H 2^16 plus that
-// (join_split), while a word receives fewer than 2^16 terms (a work item holds
-// kSpreadChunk records, each adding once per cell): then |H| < 2^31 and the low halves
-// sum below 2^32.
-__device__ __forceinline__ void add_split(unsigned* lo, int* hi, int v) {
-  atomicAdd(lo, (unsigned)v);
-  atomicAdd(hi, v >> 16);
-}
+// A sum of 32-bit signed terms v is kept as two 32-bit words: `lo` takes v itself (wrapping
+// mod 2^32) and `hi` its signed high part v >> 16, in registers and in the shared-memory tile
+// (non-returning atomics).  With H = sum of (v >> 16) and LO = sum of v mod 2^32, the sum of
+// the low halves v & 0xffff is (LO - H 2^16) mod 2^32, and the exact sum is H 2^16 plus that
+// (join_split), while a word receives fewer than 2^16 terms (a work item holds kSpreadChunk
+// pixels, each adding once per cell): then |H| < 2^31 and the low halves sum below 2^32.
 __device__ __forceinline__ long long join_split(unsigned lo, int hi) {
   const unsigned low_halves = lo - ((unsigned)hi << 16);
   return (long long)hi * 65536ll + (long long)low_halves;
@@ -194,17 +211,18 @@ __device__ void table_block(const NuGeo& g, const NuTables& tb, int vb) {
   }
 }
 
-// Spreading work items of a frame: bin offsets and cursors, and the item table
-// (item_bin[i] the bin of item i, item_first[i] its first record, items[0] their number).
+// Work items of a frame: bin offsets and cursors, the spreading items (item_bin[i] the bin of
+// item i, item_first[i] its first pixel, items[0] their number) and the sorting items
+// (sort_bin, sort_first, items[1]).
 struct NuItems {
-  int *off, *cursor, *items, *item_bin, *item_first;
+  int *off, *cursor, *items, *item_bin, *item_first, *sort_bin, *sort_first;
 };
 
 // Exclusive scan of n bin counts by one block into `off` and `cursor`, and of their chunk
-// counts into the work-item table.  The counts were added by other blocks' atomics, so
+// counts into the work-item tables.  The counts were added by other blocks' atomics, so
 // they are read from L2.
 __device__ void scan_bins(const int* __restrict__ count, int n, const NuItems& it) {
-  __shared__ int wsum[32], wcsum[32];
+  __shared__ int wsum[32], wcsum[32], n_sort;
   const int nt = blockDim.x, nw = nt >> 5;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int per = (n + nt - 1) / nt;
@@ -213,6 +231,7 @@ __device__ void scan_bins(const int* __restrict__ count, int n, const NuItems& i
   int* __restrict__ cursor = it.cursor;
   int* __restrict__ item_bin = it.item_bin;
   int* __restrict__ item_first = it.item_first;
+  if (t == 0) n_sort = 0;
   // counts in batches of 8 loads issued together (the first batch kept for the second pass)
   constexpr int kBatch = 8;
   int first[kBatch];
@@ -269,6 +288,12 @@ __device__ void scan_bins(const int* __restrict__ count, int n, const NuItems& i
         item_bin[crun] = b + j;
         item_first[crun] = run + q;
       }
+      // the order of the sorting items does not matter: a slot each from a shared counter
+      for (int q = 0; q < kk[j]; q += kSortChunk) {
+        const int slot = atomicAdd(&n_sort, 1);
+        it.sort_bin[slot] = b + j;
+        it.sort_first[slot] = run + q;
+      }
       run += kk[j];
     }
   }
@@ -276,21 +301,23 @@ __device__ void scan_bins(const int* __restrict__ count, int n, const NuItems& i
     off[n] = wsum[nw - 1];
     it.items[0] = wcsum[nw - 1];
   }
+  __syncthreads();
+  if (t == 0) it.items[1] = n_sort;
 }
 
-// Binning blocks: blockIdx.y = channel, blockIdx.x = a range of kBinItems points.  The row
-// blockIdx.y = V builds the geometry's tables.  The last counting block to finish (a
+// Binning blocks: blockIdx.y = channel group, blockIdx.x = a range of kBinItems pixels.  The row
+// blockIdx.y = groups builds the geometry's tables.  The last counting block to finish (a
 // ticket taken after its counts are visible: count[nbins]) scans the counts into the work
 // items, so no block waits for another.
 __global__ void __launch_bounds__(kBinThreads) nu_bin_count(const FrameIO* __restrict__ fp, NuGeo g,
                                                             int* __restrict__ count, NuTables tb, NuItems it) {
   wait_prior_grid();
-  if ((int)blockIdx.y == g.V) {
+  if ((int)blockIdx.y == g.groups) {
     for (int vb = blockIdx.x; vb < tb.blocks; vb += gridDim.x) table_block(g, tb, vb);
     return;
   }
-  extern __shared__ int hist[];  // this channel's bins
-  const int nb = g.ntx * g.nty, v = blockIdx.y;
+  extern __shared__ int hist[];  // this group's bins
+  const int nb = g.ntx * g.nty, grp = blockIdx.y, v = grp * g.gch;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) hist[b] = 0;
   __syncthreads();
   const FrameIO& fr = *fp;
@@ -301,73 +328,153 @@ __global__ void __launch_bounds__(kBinThreads) nu_bin_count(const FrameIO* __res
     atomicAdd(&hist[bin_of(fr.phA[(int64_t)v * fr.Pcap + p], fr.phB[p], g)], 1);
   __syncthreads();
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
-    if (hist[b]) atomicAdd(&count[v * nb + b], hist[b]);
+    if (hist[b]) atomicAdd(&count[grp * nb + b], hist[b]);
   __shared__ int ticket;
   __threadfence();
   __syncthreads();
-  const int nbins = g.V * nb;
+  const int nbins = g.groups * nb;
   if (threadIdx.x == 0) ticket = atomicAdd(&count[nbins], 1);
   __syncthreads();
-  if (ticket != (int)(gridDim.x * g.V) - 1) return;
+  if (ticket != (int)(gridDim.x * g.groups) - 1) return;
   __threadfence();
   scan_bins(count, nbins, it);
 }
 
-__global__ void __launch_bounds__(kBinThreads) nu_bin_fill(const FrameIO* __restrict__ fp, NuGeo g,
-                                                           int* __restrict__ cursor, NuRec* __restrict__ rec) {
+// The first groups x fill_blocks blocks store the pixels; each of the groups x G_x blocks after
+// them looks whether a bin of its group reaches grid row gx (its tile's rows and the halo of
+// g.H + 1 rows), and if so clears that row of the group's channels and marks it in row_used.
+__global__ void __launch_bounds__(kBinThreads) nu_bin_fill(const FrameIO* __restrict__ fp, NuGeo g, int fill_blocks,
+                                                           int* __restrict__ cursor, NuRec* __restrict__ rec,
+                                                           uint32_t* __restrict__ ord,
+                                                           const int* __restrict__ count,
+                                                           unsigned long long* __restrict__ grid,
+                                                           int* __restrict__ row_used) {
   wait_prior_grid();
   extern __shared__ int hist[];  // [nb] counts in this block, then [nb] reserved bases
-  const int nb = g.ntx * g.nty, v = blockIdx.y;
+  const int nb = g.ntx * g.nty;
+  int block = blockIdx.x;
+  if (block >= g.groups * fill_blocks) {
+    block -= g.groups * fill_blocks;
+    const int grp = block / g.Gx, gx = block % g.Gx, halo = g.W / 2 + 1;
+    bool hit = false;
+    for (int e = threadIdx.x; e < nb; e += blockDim.x) {
+      // rows of tile tx and its halo, counted from their first row, modulo G_x
+      const int tx = e / g.nty;
+      if (((gx - tx * g.Tx + halo) & (g.Gx - 1)) < min(g.Gx, g.Tx + 2 * halo)) hit |= count[grp * nb + e] != 0;
+    }
+    hit = __syncthreads_or(hit);
+    for (int v = grp * g.gch; v < min(g.V, (grp + 1) * g.gch); ++v) {
+      const int64_t row = (int64_t)v * g.Gx + gx;
+      if (threadIdx.x == 0) row_used[row] = hit;
+      if (hit)
+        for (int y = threadIdx.x; y < g.Gy; y += blockDim.x)
+          reinterpret_cast<ulonglong2*>(grid)[row * g.Gy + y] = make_ulonglong2(0ull, 0ull);
+    }
+    return;
+  }
+  const int grp = block / fill_blocks, v = grp * g.gch;
   int* base = hist + nb;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) hist[b] = 0;
   __syncthreads();
   const FrameIO& fr = *fp;
   const int64_t pv = (int64_t)fr.meta[0];
-  const int64_t p0 = (int64_t)blockIdx.x * kBinItems;
+  const int64_t p0 = (int64_t)(block % fill_blocks) * kBinItems;
   constexpr int kPer = kBinItems / kBinThreads;
-  // this thread's points: every load issued before the first use
-  uint32_t xq[kPer], yq[kPer], cq[kPer];
-  float2 sg[kPer];
+  // this thread's pixels: every load issued before the first use
+  uint32_t xq[kPer], yq[kPer];
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     const int64_t p = p0 + threadIdx.x + (int64_t)i * blockDim.x;
     const bool in = p < pv;
     xq[i] = in ? fr.phA[(int64_t)v * fr.Pcap + p] : 0u;
     yq[i] = in ? fr.phB[p] : 0u;
-    cq[i] = in ? fr.phC[(int64_t)v * fr.Pcap + p] : 0u;
-    sg[i] = in ? fr.sig[p] : make_float2(0.f, 0.f);
   }
   int bins[kPer], rank[kPer];
+  uint32_t key[kPer];
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     const int64_t p = p0 + threadIdx.x + (int64_t)i * blockDim.x;
     bins[i] = -1;
-    rank[i] = 0;
     if (p < pv) {
-      bins[i] = bin_of(xq[i], yq[i], g);
+      bins[i] = bin_of(xq[i], yq[i], g, &key[i]);
       rank[i] = atomicAdd(&hist[bins[i]], 1);
     }
   }
-  // q' = sigma exp(j 2 pi (c + x s_x + y s_y)), the phase exact mod 1 in 2^-32 cycles
-  float2 q[kPer];
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const uint32_t ph = cq[i] + xq[i] * (uint32_t)g.sx + yq[i] * (uint32_t)g.sy;
-    float sn, cs;
-    sincospif((float)(int32_t)ph * 4.656612873077393e-10f, &sn, &cs);  // angle pi ph / 2^31
-    q[i] = make_float2(sg[i].x * cs - sg[i].y * sn, sg[i].x * sn + sg[i].y * cs);
-  }
   __syncthreads();
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) base[b] = hist[b] ? atomicAdd(&cursor[v * nb + b], hist[b]) : 0;
+  for (int b = threadIdx.x; b < nb; b += blockDim.x)
+    base[b] = hist[b] ? atomicAdd(&cursor[grp * nb + b], hist[b]) : 0;
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     if (bins[i] < 0) continue;
-    NuRec r;
-    r.x = xq[i];
-    r.y = yq[i];
-    r.q = q[i];
-    rec[base[bins[i]] + rank[i]] = r;
+    const uint32_t q = (uint32_t)(p0 + threadIdx.x + (int64_t)i * blockDim.x);
+    if (rec)
+      rec[base[bins[i]] + rank[i]] = NuRec{key[i], q};
+    else
+      ord[base[bins[i]] + rank[i]] = q;  // frames too small to be sorted
+  }
+}
+
+// Counting sort of up to kSortChunk pixels of one bin by key: `ord` receives their indices.
+// Pixels of one key come in any order (the spreading sums are exact).
+__global__ void __launch_bounds__(kSortThreads) nu_sort(const int* __restrict__ off, const int* __restrict__ items,
+                                                        const int* __restrict__ sort_bin,
+                                                        const int* __restrict__ sort_first,
+                                                        const NuRec* __restrict__ rec, uint32_t* __restrict__ ord) {
+  constexpr int kKeys = kNTile * kNTile * kSub, kPer = kSortChunk / kSortThreads, kOwn = kKeys / kSortThreads;
+  static_assert(kKeys % kSortThreads == 0, "keys per thread");
+  __shared__ int hist[kKeys], wsum[32];
+  wait_prior_grid();
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int n_sorts = items[1];
+  for (int item = blockIdx.x; item < n_sorts; item += gridDim.x) {
+    const int first = sort_first[item], n = min(kSortChunk, off[sort_bin[item] + 1] - first);
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) hist[t + i * kSortThreads] = 0;
+    __syncthreads();
+    NuRec r[kPer];
+    int rank[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (t + i * kSortThreads < n) r[i] = rec[first + t + i * kSortThreads];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (t + i * kSortThreads < n) rank[i] = atomicAdd(&hist[r[i].key], 1);
+    __syncthreads();
+    // exclusive scan of the keys' counts, kOwn consecutive ones per thread
+    int own[kOwn], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) {
+      own[i] = hist[t * kOwn + i];
+      sum += own[i];
+    }
+    int incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+      int x = wsum[lane];
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      wsum[lane] = x;
+    }
+    __syncthreads();
+    int run = (w ? wsum[w - 1] : 0) + incl - sum;
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) {
+      hist[t * kOwn + i] = run;
+      run += own[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (t + i * kSortThreads < n) ord[first + hist[r[i].key] + rank[i]] = r[i].q;
+    __syncthreads();  // the next item clears the counts
   }
 }
 
@@ -384,40 +491,43 @@ __global__ void __launch_bounds__(kBinThreads) nu_bin_fill(const FrameIO* __rest
 //   [lo re | lo im | hi re | hi im] tile words, then the staging, then a zero row.
 constexpr int kSpreadThreads = 512;
 constexpr int kSpreadWarps = kSpreadThreads / 32;
-constexpr int kSpreadBlocksPerSm = 3;  // persistent CTAs per SM (about 70 KB of shared memory each at w = 7)
-constexpr int kStageLd = 33;           // staged values of 32 records per jx (or jy), padded
+constexpr int kSpreadBlocksPerSm = 2;  // persistent CTAs per SM (about 73 KB of shared memory each at w = 7)
+// Staged values of 32 pixels per jx (jy), in rows of 34 float2 (36 floats): 16-byte loads of four
+// pixels' values from the rows of a warp's taps then fall on distinct banks.
+constexpr int kAxLd = 34, kWyLd = 36;
 
 template <int W>
 struct SpreadLayout {
-  static constexpr int H = W / 2;                         // halo cells
-  static constexpr int PAD = kNTile + 2 * H;              // padded tile side
+  static constexpr int H = W / 2;                         // halo cells along y
+  static constexpr int HX = H + 1;                        // along x: one more for the other channels
+  static constexpr int PADX = kNTile + 2 * HX, PAD = kNTile + 2 * H;  // padded tile sides
   static constexpr int STRIDE = W + 32;                   // tile row stride, W (mod 32)
-  static constexpr int WORDS = (PAD * STRIDE + 3) / 4 * 4;  // one tile array, 16-byte words
+  static constexpr int WORDS = (PADX * STRIDE + 3) / 4 * 4;  // one tile array, 16-byte words
   static constexpr bool TWO = W * W > 32;                 // a second pass of lanes
   static constexpr size_t kTiles = 4 * sizeof(unsigned) * WORDS;
-  static constexpr size_t kAx = sizeof(float2) * kSpreadWarps * W * kStageLd;
-  static constexpr size_t kWy = sizeof(float) * kSpreadWarps * W * kStageLd;
+  static constexpr size_t kAx = sizeof(float2) * kSpreadWarps * W * kAxLd;
+  static constexpr size_t kWy = sizeof(float) * kSpreadWarps * W * kWyLd;
   static constexpr size_t kBase = sizeof(int) * kSpreadWarps * 32;
-  static constexpr size_t kZero = sizeof(float2) * kStageLd;
+  static constexpr size_t kZero = sizeof(float2) * kAxLd;
   static constexpr size_t bytes = kTiles + kAx + kWy + kBase + kZero;
   static_assert(STRIDE >= PAD && STRIDE % 32 == W, "tile row stride");
   static_assert(W * W <= 64, "two passes of 32 lanes cover the taps");
   // a spare lane's word base + lane stays inside the tile array
-  static_assert((PAD - W) * STRIDE + (PAD - W) + 31 < WORDS, "spare-lane words in range");
+  static_assert((PADX - W) * STRIDE + (PAD - W) + 31 < WORDS, "spare-lane words in range");
 };
 
-// Persistent CTAs take the work items in turn (their number is known on the device only).
+// Persistent CTAs take the units (work item, channel of its group) in turn (their number is
+// known on the device only).
 template <int W>
 __global__ void __launch_bounds__(kSpreadThreads, kSpreadBlocksPerSm) nu_spread(const FrameIO* __restrict__ fp, NuGeo g,
                                                             const int* __restrict__ off,
                                                             const int* __restrict__ items,
                                                             const int* __restrict__ item_bin,
                                                             const int* __restrict__ item_first,
-                                                            const NuRec* __restrict__ rec,
-                                                            unsigned long long* __restrict__ grid,
-                                                            int* __restrict__ row_used) {
+                                                            const uint32_t* __restrict__ ord,
+                                                            unsigned long long* __restrict__ grid) {
   using Lay = SpreadLayout<W>;
-  constexpr int H = Lay::H, PAD = Lay::PAD, STRIDE = Lay::STRIDE, WORDS = Lay::WORDS;
+  constexpr int H = Lay::H, HX = Lay::HX, PADX = Lay::PADX, PAD = Lay::PAD, STRIDE = Lay::STRIDE, WORDS = Lay::WORDS;
   constexpr float beta = kNBetaPerW * W, k2w = 2.f / (float)W;
   wait_prior_grid();
   extern __shared__ __align__(16) unsigned char smem_sp[];
@@ -425,14 +535,15 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadBlocksPerSm) nu_spread(
   unsigned* lo_im = lo_re + WORDS;
   int* hi_re = reinterpret_cast<int*>(lo_im + WORDS);
   int* hi_im = hi_re + WORDS;
-  float2(*s_ax)[W][kStageLd] = reinterpret_cast<float2(*)[W][kStageLd]>(smem_sp + Lay::kTiles);
-  float(*s_wy)[W][kStageLd] = reinterpret_cast<float(*)[W][kStageLd]>(smem_sp + Lay::kTiles + Lay::kAx);
+  float2(*s_ax)[W][kAxLd] = reinterpret_cast<float2(*)[W][kAxLd]>(smem_sp + Lay::kTiles);
+  float(*s_wy)[W][kWyLd] = reinterpret_cast<float(*)[W][kWyLd]>(smem_sp + Lay::kTiles + Lay::kAx);
   int(*s_base)[32] = reinterpret_cast<int(*)[32]>(smem_sp + Lay::kTiles + Lay::kAx + Lay::kWy);
   float2* s_zero = reinterpret_cast<float2*>(smem_sp + Lay::kTiles + Lay::kAx + Lay::kWy + Lay::kBase);
-  for (int i = threadIdx.x; i < kStageLd; i += blockDim.x) s_zero[i] = make_float2(0.f, 0.f);
-  const int n_items = items[0];
+  for (int i = threadIdx.x; i < kAxLd; i += blockDim.x) s_zero[i] = make_float2(0.f, 0.f);
+  const int n_units = items[0] * g.gch;
   const int nb = g.ntx * g.nty;
-  const float scale = grid_scale(*fp, false);
+  const FrameIO& fr = *fp;
+  const float scale = grid_scale(fr, false);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // This lane's taps on the two passes (a spare lane: the zero row, word base + lane).
   const bool act0 = lane < W * W;
@@ -446,42 +557,72 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadBlocksPerSm) nu_spread(
   const float* wy0 = s_wy[warp][jy0];
   const float* wy1 = s_wy[warp][jy1];
   const int* sb = s_base[warp];
-  auto pass = [&](int base, float2 a, float w, int offs) {
-    const int at = base + offs;
-    add_split(&lo_re[at], &hi_re[at], __float2int_rn(a.x * w));
-    add_split(&lo_im[at], &hi_im[at], __float2int_rn(a.y * w));
+  // the run's sums of both passes: low and high words (see join_split)
+  unsigned l0r, l0i, l1r, l1i;
+  int h0r, h0i, h1r, h1i;
+  auto clear = [&] {
+    l0r = l0i = l1r = l1i = 0u;
+    h0r = h0i = h1r = h1i = 0;
   };
-  auto taps = [&](int r) {
-    const int base = sb[r];
-    pass(base, ax0[r], wy0[r], off0);
-    if (Lay::TWO) pass(base, ax1[r], wy1[r], off1);
+  auto flush = [&](int base) {
+    atomicAdd(&lo_re[base + off0], l0r);
+    atomicAdd(&hi_re[base + off0], h0r);
+    atomicAdd(&lo_im[base + off0], l0i);
+    atomicAdd(&hi_im[base + off0], h0i);
+    if (Lay::TWO) {
+      atomicAdd(&lo_re[base + off1], l1r);
+      atomicAdd(&hi_re[base + off1], h1r);
+      atomicAdd(&lo_im[base + off1], l1i);
+      atomicAdd(&hi_im[base + off1], h1i);
+    }
   };
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+  // a tap's terms of four pixels
+  auto terms = [&](const float2* ax, const float* wy, int (&tr)[4], int (&ti)[4]) {
+    const float4 a01 = *reinterpret_cast<const float4*>(ax), a23 = *reinterpret_cast<const float4*>(ax + 2);
+    const float4 w = *reinterpret_cast<const float4*>(wy);
+    tr[0] = __float2int_rn(a01.x * w.x), ti[0] = __float2int_rn(a01.y * w.x);
+    tr[1] = __float2int_rn(a01.z * w.y), ti[1] = __float2int_rn(a01.w * w.y);
+    tr[2] = __float2int_rn(a23.x * w.z), ti[2] = __float2int_rn(a23.y * w.z);
+    tr[3] = __float2int_rn(a23.z * w.w), ti[3] = __float2int_rn(a23.w * w.w);
+  };
+  for (int unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
+    const int item = unit / g.gch;
     const int bin = item_bin[item];
-    const int v = bin / nb, ty = (bin % nb) % g.nty, tx = (bin % nb) / g.nty;
+    const int v = bin / nb * g.gch + unit % g.gch;
+    if (v >= g.V) continue;
+    const int ty = (bin % nb) % g.nty, tx = (bin % nb) / g.nty;
     const int r_begin = item_first[item];
-    const int r_end = min(off[bin + 1], r_begin + kSpreadChunk);
-    // the grid rows this item adds to (the padded tile's, mod G_x): the row pass skips
-    // rows that no item marks, which hold zeros only
-    for (int r = threadIdx.x; r < PAD; r += blockDim.x)
-      row_used[(int64_t)v * g.Gx + ((tx * g.Tx - H + r) & (g.Gx - 1))] = 1;
+    const int n = min(off[bin + 1] - r_begin, kSpreadChunk);
     for (int i = threadIdx.x; i < WORDS; i += blockDim.x)  // 4 arrays of WORDS / 4 16-byte words
       reinterpret_cast<uint4*>(smem_sp)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    for (int r0 = r_begin + warp * 32; r0 < r_end; r0 += kSpreadThreads) {
-      const int n = min(32, r_end - r0);
-      if (lane < n) {
-        const NuRec q = rec[r0 + lane];
+    // a warp takes consecutive pixels, 32 at a time
+    const int per = (n + kSpreadThreads - 1) / kSpreadThreads * 32;
+    const int w1 = min(n, (warp + 1) * per);
+    int cur = -1;
+    clear();
+    for (int r0 = warp * per; r0 < w1; r0 += 32) {
+      const int m = min(32, w1 - r0);
+      if (lane < m) {
+        const uint32_t q = ord[r_begin + r0 + lane];
+        const uint32_t xq = fr.phA[(int64_t)v * fr.Pcap + q], cq = fr.phC[(int64_t)v * fr.Pcap + q], yq = fr.phB[q];
+        const float2 sg = fr.sig[q];
+        // q' = sigma exp(j 2 pi (c + x s_x + y s_y)), the phase exact mod 1 in 2^-32 cycles
+        const uint32_t phq = cq + xq * (uint32_t)g.sx + yq * (uint32_t)g.sy;
+        float sn, cs;
+        sincospif((float)(int32_t)phq * 4.656612873077393e-10f, &sn, &cs);  // angle pi ph / 2^31
+        const float2 qs = make_float2(sg.x * cs - sg.y * sn, sg.x * sn + sg.y * cs);
         int cx, cy;
         float dx, dy;
-        nearest_cell(q.x, g.Gx, cx, dx);
-        nearest_cell(q.y, g.Gy, cy, dy);
+        nearest_cell(xq, g.Gx, cx, dx);
+        nearest_cell(yq, g.Gy, cy, dy);
         // first tap relative to the nearest cell
         const int sx = (W & 1) ? -(W - 1) / 2 : -W / 2 + (dx >= 0.f ? 1 : 0);
         const int sy = (W & 1) ? -(W - 1) / 2 : -W / 2 + (dy >= 0.f ? 1 : 0);
-        // the nearest cell lies in this tile: local padded coordinates of the first tap
-        const int lx = cx - tx * g.Tx + H + sx, ly = cy - ty * g.Ty + H + sy;
-        const float qr = q.q.x * scale, qi = q.q.y * scale;
+        // the nearest cell lies in this tile (along x, in the group's first channel; here at
+        // most one cell outside it, modulo G_x): local padded coordinates of the first tap
+        const int lx = ((cx - tx * g.Tx + 1) & (g.Gx - 1)) - 1 + HX + sx, ly = cy - ty * g.Ty + H + sy;
+        const float qr = qs.x * scale, qi = qs.y * scale;
         // tap j sits at z = (s + j - d) 2 / W in kernel units
         const float zx0 = ((float)sx - dx) * k2w, zy0 = ((float)sy - dy) * k2w;
         // the hardware exponential's few-ulp error sets an error floor near 1e-6, below the
@@ -495,20 +636,42 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadBlocksPerSm) nu_spread(
           s_wy[warp][j][lane] = W >= 8 ? es_kernel(zy, beta) : es_kernel_fast(zy, beta);
         }
         s_base[warp][lane] = lx * STRIDE + ly;
+      } else {
+        // past the end: no strength, and no cell
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+          s_ax[warp][j][lane] = make_float2(0.f, 0.f);
+          s_wy[warp][j][lane] = 0.f;
+        }
+        s_base[warp][lane] = -1;
       }
       __syncwarp();
-      int r = 0;
-      for (; r + 1 < n; r += 2) {
-        taps(r);
-        taps(r + 1);
+      for (int r = 0; r < m; r += 4) {
+        // four pixels at a time: their values in 16-byte loads, their terms, then the runs
+        const int4 b4 = *reinterpret_cast<const int4*>(sb + r);
+        const int bs[4] = {b4.x, b4.y, b4.z, b4.w};
+        int tr[2][4], ti[2][4];
+        terms(ax0 + r, wy0 + r, tr[0], ti[0]);
+        if (Lay::TWO) terms(ax1 + r, wy1 + r, tr[1], ti[1]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (bs[i] != cur) {
+            if (cur >= 0) flush(cur);
+            cur = bs[i];
+            clear();
+          }
+          l0r += (unsigned)tr[0][i], h0r += tr[0][i] >> 16, l0i += (unsigned)ti[0][i], h0i += ti[0][i] >> 16;
+          if (Lay::TWO)
+            l1r += (unsigned)tr[1][i], h1r += tr[1][i] >> 16, l1i += (unsigned)ti[1][i], h1i += ti[1][i] >> 16;
+        }
       }
-      if (r < n) taps(r);
       __syncwarp();
     }
+    if (cur >= 0) flush(cur);
     __syncthreads();
-    const int x0 = tx * g.Tx - H, y0 = ty * g.Ty - H;  // padded tile origin (cells)
+    const int x0 = tx * g.Tx - HX, y0 = ty * g.Ty - H;  // padded tile origin (cells)
     const int64_t gbase = (int64_t)v * g.Gx * g.Gy;
-    for (int i = threadIdx.x; i < PAD * PAD; i += blockDim.x) {
+    for (int i = threadIdx.x; i < PADX * PAD; i += blockDim.x) {
       const int row = i / PAD, col = i % PAD, at = row * STRIDE + col;
       const long long re = join_split(lo_re[at], hi_re[at]);
       const long long im = join_split(lo_im[at], hi_im[at]);
@@ -518,7 +681,7 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadBlocksPerSm) nu_spread(
       atomicAdd(cell, (unsigned long long)re);
       atomicAdd(cell + 1, (unsigned long long)im);
     }
-    __syncthreads();  // the tile is read before the next item clears it
+    __syncthreads();  // the tile is read before the next unit clears it
   }
 }
 
@@ -643,7 +806,7 @@ __global__ void nu_fft_y(const FrameIO* __restrict__ fp, NuGeo g, FftPlan pl, co
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_y + fft_smem_bytes(pl, 16) - 16);
   const int64_t rows = (int64_t)g.V * g.Gx, row0 = (int64_t)blockIdx.x * pl.S;
   const int live_rows = (int)min((int64_t)pl.S, rows - row0);
-  // rows no spreading item touched are zero, and so is their transform: no copy, no FFT
+  // rows that no bin reaches have not been cleared; their transform is zero: no copy, no FFT
   if (!__syncthreads_or((int)threadIdx.x < live_rows && row_used[row0 + threadIdx.x] != 0)) {
     for (int e = threadIdx.x; e < pl.S * g.L; e += blockDim.x) {
       const int rs = e % pl.S, l = e / pl.S;
@@ -657,7 +820,7 @@ __global__ void nu_fft_y(const FrameIO* __restrict__ fp, NuGeo g, FftPlan pl, co
   const int t = threadIdx.x % pl.T, s = threadIdx.x / pl.T;
   const float inv = grid_scale(*fp, true);
   const longlong2* src = raw + (int64_t)s * g.Gy;
-  const bool live = s < live_rows;
+  const bool live = s < live_rows && row_used[row0 + s] != 0;  // the others' cells are stale
   auto in = [=](int i) -> float2 {
     if (!live) return make_float2(0.f, 0.f);
     const longlong2 c = src[i];
@@ -773,21 +936,29 @@ struct FftX {
   static Fn fn() { return nu_fft_x<P, RL>; }
 };
 
-// Scratch of one frame: bin counts, cursors and offsets; the spreading work items; the
-// records; the 64-bit integer grid; the row-transformed grid; the deconvolution factors.
+// Scratch of one frame: bin counts, cursors and offsets; the work items; the binned and the
+// sorted pixels; the 64-bit integer grid; the row-transformed grid; the deconvolution factors.
 struct NuScratch {
-  int *count, *row_used, *cursor, *off, *items, *item_bin, *item_first;
+  int *count, *row_used, *cursor, *off, *items, *item_bin, *item_first, *sort_bin, *sort_first;
   NuRec* rec;
+  uint32_t* ord;
   unsigned long long* grid;
   float2* mid;
   float *inv_x, *inv_y;
   float2 *tw_x, *tw_y;
-  size_t grid_bytes, total;
+  size_t total;
 };
 
+// Chunks of `chunk` pixels that the bins can give at most: each bin's last one may be short,
+// and there are no more bins than pixels.
+size_t nu_max_items(const NuGeo& g, int chunk) {
+  const size_t nbins = (size_t)g.groups * g.ntx * g.nty, px = (size_t)g.groups * g.P;
+  return std::min(nbins, px) + (px + chunk - 1) / chunk;
+}
+
 NuScratch nufft_layout(const NuGeo& g, const FftPlan& plx, const FftPlan& ply, char* base) {
-  const size_t nbins = (size_t)g.V * g.ntx * g.nty;
-  const size_t max_items = nbins + ((size_t)g.V * g.P + kSpreadChunk - 1) / kSpreadChunk;
+  const size_t nbins = (size_t)g.groups * g.ntx * g.nty;
+  const size_t max_items = nu_max_items(g, kSpreadChunk), max_sorts = nu_max_items(g, kSortChunk);
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   NuScratch sc{};
   size_t o = 0;
@@ -796,17 +967,18 @@ NuScratch nufft_layout(const NuGeo& g, const FftPlan& plx, const FftPlan& ply, c
     o += up(bytes);
     return p;
   };
-  // the bin counts, the finished-block count, the grid rows in use (cleared together)
-  sc.count = (int*)take(4 * (nbins + 1 + (size_t)g.V * g.Gx));
-  sc.row_used = sc.count ? sc.count + nbins + 1 : nullptr;
+  sc.count = (int*)take(4 * (nbins + 1));  // the bin counts and the finished-block count
+  sc.row_used = (int*)take(4 * (size_t)g.V * g.Gx);
   sc.cursor = (int*)take(4 * nbins);
   sc.off = (int*)take(4 * (nbins + 1));
-  sc.items = (int*)take(4);
+  sc.items = (int*)take(8);
   sc.item_bin = (int*)take(4 * max_items);
   sc.item_first = (int*)take(4 * max_items);
-  sc.rec = (NuRec*)take(sizeof(NuRec) * (size_t)g.V * g.P);
-  sc.grid_bytes = 16 * (size_t)g.V * g.Gx * g.Gy;
-  sc.grid = (unsigned long long*)take(sc.grid_bytes);
+  sc.sort_bin = (int*)take(4 * max_sorts);
+  sc.sort_first = (int*)take(4 * max_sorts);
+  sc.rec = (NuRec*)take(sizeof(NuRec) * (size_t)g.groups * g.P);
+  sc.ord = (uint32_t*)take(4 * (size_t)g.groups * g.P);
+  sc.grid = (unsigned long long*)take(16 * (size_t)g.V * g.Gx * g.Gy);
   sc.mid = (float2*)take(8 * (size_t)g.V * g.Gx * g.L);
   sc.inv_x = (float*)take(4 * (size_t)(g.Ns + g.L));
   sc.inv_y = sc.inv_x ? sc.inv_x + g.Ns : nullptr;
@@ -834,8 +1006,14 @@ NuGeo nufft_geometry(const Consts& k, int64_t P) {
   g.P = std::max<int64_t>(P, 1);
   g.W = k.nu_w;
   g.beta = kNBetaPerW * (float)g.W;
+  // channels whose positions along x lie within 0.9 of a cell of the first's (|u| <= 1)
+  const double cells = fabs(k.k_da) * g.Gx;
+  g.gch = cells * (k.V - 1) <= 0.9 ? k.V : std::max(1, (int)(0.9 / cells) + 1);
+  g.groups = (k.V + g.gch - 1) / g.gch;
   return g;
 }
+
+int nufft_kernels(int64_t P) { return P >= kSortFrom ? 6 : 5; }
 
 bool nufft_supported(const Consts& k) {
   // FFT lengths up to 4096 in one CTA's shared memory, at least 8 cells per axis, and a
@@ -853,18 +1031,16 @@ cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int o
                          unsigned* status, cudaStream_t st, cudaEvent_t spread_begin, cudaEvent_t spread_end) {
   const NuGeo g = nufft_geometry(k, P);
   const int nb = g.ntx * g.nty;
-  const int nbins = g.V * nb;
-  const int64_t max_items = nbins + ((int64_t)g.V * g.P + kSpreadChunk - 1) / kSpreadChunk;
+  const int nbins = g.groups * nb;
   const FftPlan plx = fft_plan(g.Gx), ply = fft_plan(g.Gy);
   const NuScratch sc = nufft_layout(g, plx, ply, scratch);
   int dev = 0, num_sms = 0;
   cudaError_t e0 = cudaGetDevice(&dev);
   if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e0 != cudaSuccess) return e0;
-  cudaError_t e = cudaMemsetAsync(sc.count, 0, 4 * ((size_t)nbins + 1 + (size_t)g.V * g.Gx), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sc.grid, 0, sc.grid_bytes, st);
+  cudaError_t e = cudaMemsetAsync(sc.count, 0, 4 * ((size_t)nbins + 1), st);
   if (e != cudaSuccess) return e;
-  const dim3 bgrid((unsigned)((g.P + kBinItems - 1) / kBinItems), (unsigned)g.V);
+  const dim3 bgrid((unsigned)((g.P + kBinItems - 1) / kBinItems), (unsigned)g.groups);
   e = cudaFuncSetAttribute(nu_bin_count, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * nb);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(nu_bin_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * nb);
   if (e != cudaSuccess) return e;
@@ -877,14 +1053,23 @@ cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int o
   tb.inv_y = sc.inv_y;
   tb.twx = sc.tw_x;
   tb.twy = sc.tw_y;
-  const NuItems it{sc.off, sc.cursor, sc.items, sc.item_bin, sc.item_first};
+  // few pixels share a cell in a small frame: its sort (a launch and some 5 us) gains nothing
+  const bool sorted = g.P >= kSortFrom;
+  const NuItems it{sc.off, sc.cursor, sc.items, sc.item_bin, sc.item_first, sc.sort_bin, sc.sort_first};
   e = launch_dependent(nu_bin_count, dim3(bgrid.x, bgrid.y + 1), dim3(kBinThreads), (size_t)(4 * nb), st, frame, g,
                        sc.count, tb, it);
   if (e == cudaSuccess)
-    e = launch_dependent(nu_bin_fill, bgrid, dim3(kBinThreads), (size_t)(8 * nb), st, frame, g, sc.cursor, sc.rec);
+    e = launch_dependent(nu_bin_fill, dim3(bgrid.x * bgrid.y + (unsigned)(g.groups * g.Gx)), dim3(kBinThreads),
+                         (size_t)(8 * nb), st, frame, g, (int)bgrid.x, sc.cursor, sorted ? sc.rec : nullptr, sc.ord,
+                         (const int*)sc.count,
+                         sc.grid, sc.row_used);
+  if (e == cudaSuccess && sorted)
+    e = launch_dependent(nu_sort, dim3((unsigned)std::min<size_t>(nu_max_items(g, kSortChunk), (size_t)2 * num_sms)),
+                         dim3(kSortThreads), 0, st, (const int*)sc.off, (const int*)sc.items, (const int*)sc.sort_bin,
+                         (const int*)sc.sort_first, (const NuRec*)sc.rec, sc.ord);
   // the spreading kernel of the gridding kernel's width, and its shared memory
-  using SpreadFn = void (*)(const FrameIO*, NuGeo, const int*, const int*, const int*, const int*, const NuRec*,
-                            unsigned long long*, int*);
+  using SpreadFn = void (*)(const FrameIO*, NuGeo, const int*, const int*, const int*, const int*, const uint32_t*,
+                            unsigned long long*);
   SpreadFn spread = nu_spread<7>;
   size_t spread_smem = SpreadLayout<7>::bytes;
   switch (g.W) {
@@ -897,10 +1082,11 @@ cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int o
   if (e == cudaSuccess) e = cudaFuncSetAttribute(spread, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)spread_smem);
   if (e == cudaSuccess && spread_begin) e = cudaEventRecord(spread_begin, st);
   if (e == cudaSuccess)
-    e = launch_dependent(spread, dim3((unsigned)std::min<int64_t>(max_items, kSpreadBlocksPerSm * num_sms)),
-                         dim3(kSpreadThreads), spread_smem, st, frame, g, (const int*)sc.off,
-                         (const int*)sc.items, (const int*)sc.item_bin, (const int*)sc.item_first,
-                         (const NuRec*)sc.rec, sc.grid, sc.row_used);
+    e = launch_dependent(spread,
+                         dim3((unsigned)std::min<size_t>(nu_max_items(g, kSpreadChunk) * g.gch,
+                                                         (size_t)kSpreadBlocksPerSm * num_sms)),
+                         dim3(kSpreadThreads), spread_smem, st, frame, g, (const int*)sc.off, (const int*)sc.items,
+                         (const int*)sc.item_bin, (const int*)sc.item_first, (const uint32_t*)sc.ord, sc.grid);
   if (e == cudaSuccess && spread_end) e = cudaEventRecord(spread_end, st);
   if (e != cudaSuccess) return e;
   const int ysmem = fft_smem_bytes(ply, 16);

@@ -321,14 +321,20 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     // order (1 for a batch), contraction (1); NUFFT: the NUFFT kernels of each frame; the
     // split reduction (1 when the partial buffer is used)
     const bool tensor = tensor_tier(tier);
-    ctx->prof_kernels += (tier == RSIM_TIER_NUFFT ? kNufftKernels * F
-                              : tensor ? 1 + (mp > 0 ? 1 : 0) + (F > 1 ? 1 : 0) : 1) + (use_partial ? 1 : 0);
+    if (tier == RSIM_TIER_NUFFT) {
+      for (int f = 0; f < F; ++f) ctx->prof_kernels += nufft_kernels(frames[f].P);
+    } else {
+      ctx->prof_kernels += (tensor ? 1 + (mp > 0 ? 1 : 0) + (F > 1 ? 1 : 0) : 1) + (use_partial ? 1 : 0);
+    }
     cudaEventRecord(ev[0], st);
   }
   cudaError_t e;
   // the tensor tiers' operand builder computes the fast-time and channel phases
   const bool defer = tensor_tier(tier);
-  {
+  // NUFFT batches: every frame's compaction goes to the frame's own stream (below), where its
+  // FP64 work runs beside other frames' spreading
+  const bool per_frame = tier == RSIM_TIER_NUFFT && nufft_slots(F) > 1;
+  if (!per_frame) {
     NvtxRange r(defer ? "compaction + slow-time phases" : "compaction + FP64 phases");
     int launched = 0;
     e = launch_prep(k, table, F == 1 ? host.data() : nullptr, F, mp, frames[0].dtype, false, defer, status,
@@ -363,7 +369,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
       ctx->nu_ready = true;
     }
     // frame f runs on stream f mod S with scratch slot f mod S; every stream first waits
-    // for the compaction and phases on `st`, and `st` then waits for every stream
+    // for `st` (the frame table), and `st` then waits for every stream
     if (S > 1) {
       e = cudaEventRecord(ctx->nu_ev[rsim_ctx::kNuStreams], st);
       for (int i = 0; i < S && e == cudaSuccess; ++i)
@@ -375,6 +381,14 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     for (int f = 0; f < F && le == cudaSuccess; ++f) {
       // the first frame's spreading kernel is bracketed by ev[4] and ev[5]
       cudaStream_t fs = S > 1 ? ctx->nu_st[f % S] : st;
+      if (per_frame) {
+        // the two-kernel form: a cooperative grid would wait for room beside the other streams
+        int launched = 0;
+        le = launch_prep(k, table + f, nullptr, 1, frames[f].P, frames[f].dtype, false, false, status, nullptr, fs,
+                         false, &launched);
+        if (prof) ctx->prof_kernels += launched;
+        if (le != cudaSuccess) break;
+      }
       le = launch_nufft(k, table + f, frames[f].P, out_dtype, scratch + (size_t)(f % S) * slot, status, fs,
                         prof && f == 0 ? ev[4] : nullptr, prof && f == 0 ? ev[5] : nullptr);
     }

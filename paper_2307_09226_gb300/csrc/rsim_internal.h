@@ -130,10 +130,11 @@ struct NuGeo {
   int64_t P;      // pixel bound (items per channel)
   int W;          // gridding kernel width (cells)
   float beta;     // its shape parameter, 2.30 W
+  int gch, groups;  // channels sorted together, and such groups
 };
-// Kernels launch_nufft starts per frame (binning with the tables and the scan, record
-// fill, spreading, two FFT passes).
-constexpr int kNufftKernels = 5;
+// Kernels launch_nufft starts for a frame of P pixels (binning with the tables and the scan,
+// fill, sort in larger frames, spreading, two FFT passes).
+int nufft_kernels(int64_t P);
 NuGeo nufft_geometry(const Consts& k, int64_t P);
 bool nufft_supported(const Consts& k);
 size_t nufft_scratch_bytes(const Consts& k, int64_t P);

@@ -131,3 +131,24 @@ def test_shared_atomic_rate_probe(ctx):
     rate = _abi.rsim_measure_smem_atomics(ctx.h)
     print(f"shared atomics: {rate / 1e12:.3f} T lane-op/s")
     assert 1e12 < rate < 1.2 * 152 * 32 * 2.1e9
+
+
+@pytest.mark.parametrize("d_rx_lambda,groups", [(0.5, "one group"), (8.0, "several channels a group"), (400.0, "one channel a group")])
+@pytest.mark.parametrize("n_az,n_el", [(64, 64), (112, 110)])
+@pytest.mark.parametrize("w", [6, 7])
+def test_channel_groups_and_sorting(ctx, d_rx_lambda, groups, n_az, n_el, w):
+    """Antenna spacings whose channels shift a pixel by a fraction of a cell, by about a cell
+    and by many cells (so that one, some or each of the channels are sorted on their own), in
+    frames below and above the size from which pixels are sorted, with ranges down to the first
+    cells so that shifts cross the grid's edge.  A frame of another scene runs in between: its
+    cells stay in the scratch and must not be seen.  Against the CPU reference at the same
+    width, with the bar of the tests above (5e-6)."""
+    radar = synth.Radar(M=2, N=4, Ns=64, L=32, d_rx=d_rx_lambda * 3.9e-3, nufft_width=w)
+    px = synth.random_frame(radar, n_az, n_el, seed=61, mask_frac=0.1, r_lo=0.001, r_hi=3.0)
+    other = synth.random_frame(radar, n_az, n_el, seed=62, mask_frac=0.0, r_lo=3.0, r_hi=40.0)
+    first = ctx.synth(radar, device.upload(px), "nufft").cpu().numpy()
+    ctx.synth(radar, device.upload(other), "nufft")
+    again = ctx.synth(radar, device.upload(px), "nufft").cpu().numpy()
+    assert ctx.sync_status() == _abi.OK
+    assert np.array_equal(first, again)
+    assert oracle.rel_l2(first, nu.cube_nufft(radar, px, w=w)) <= 5e-6
