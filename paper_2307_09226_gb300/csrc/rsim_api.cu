@@ -328,7 +328,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     }
     cudaEventRecord(ev[0], st);
   }
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   // the tensor tiers' operand builder computes the fast-time and channel phases
   const bool defer = tensor_tier(tier);
   // NUFFT batches: every frame's compaction goes to the frame's own stream (below), where its
