@@ -395,7 +395,8 @@ def run_gpu(args):
     if rank == 0:
         peaks, kind = _peaks()
         # the FP32 tier runs three products on the tensor cores, like the split tiers
-        roof = _roofline("split_fp16" if tier == "fp32" else tier, prof.contract_ms - prof.operand_ms, prof.calls, samples, peaks, kind)
+        roof = _roofline("split_fp16" if tier == "fp32" else tier, prof.contract_ms - prof.operand_ms, prof.calls,
+                         samples, peaks, kind)
         traffic = _load_traffic(tier)
         if traffic is not None:
             roof["traffic"] = traffic
@@ -457,9 +458,9 @@ def run_gpu(args):
     return 0
 
 
-# the operand builder's file and, for the tiers on pairs of CTAs, the contraction's
-KERNEL_SOURCES = {"fp32": "k_umma.cu k_umma_pair.cu", "split_fp16": "k_umma.cu k_umma_pair.cu",
-                  "split_bf16": "k_umma.cu k_umma_pair.cu", "bf16": "k_umma.cu", "fp16": "k_umma.cu"}
+# the operand builder's file and, for the tier on pairs of CTAs, the contraction's
+KERNEL_SOURCES = {"fp32": "k_umma.cu k_umma_pair.cu", "split_fp16": "k_umma.cu", "split_bf16": "k_umma.cu",
+                  "bf16": "k_umma.cu", "fp16": "k_umma.cu"}
 
 
 def kernel_source_hash(tier):
@@ -585,7 +586,8 @@ def run_nufft(ctx, frame, px, ref, steps, warmup):
     samples = pv * radar.V * radar.Ns * radar.L
     t = sum(ms) / len(ms)
     # spreading (the dominant kernel): 49 taps x (re, im) x two words = 196 shared atomic
-    # lane-operations per (channel, point) record, against the rate this device performs
+    # lane-operations per (channel, point) record (the kernel issues fewer: it sums the taps
+    # of successive points of one cell in registers first), against the rate this device performs
     # such atomics (measured by the library's probe on the same GPU), with the derived
     # one-wavefront-per-clock figure beside it
     spread_ms = prof.main_ms / prof.calls
@@ -601,7 +603,8 @@ def run_nufft(ctx, frame, px, ref, steps, warmup):
                            "kernel's occupancy (rsim_measure_smem_atomics, this GPU)",
             "derived_peak": round(derived, 3), "frac_of_derived": round(achieved / derived, 4),
             "derived_source": f"one 32-lane wavefront per clock: 152 SM x 32 lanes x {clk:.0f} MHz",
-            "algorithmic": "196 shared atomic lane-operations per (channel, point) record"}
+            "algorithmic": "196 shared atomic lane-operations per (channel, point) record, before runs of "
+                           "points in one cell are summed in registers"}
     # the accuracy each gridding kernel width buys, and its time (the same frame)
     from dataclasses import replace as _replace
     widths = {}

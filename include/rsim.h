@@ -188,9 +188,11 @@ rsim_status rsim_synth_host(rsim_ctx* ctx, const rsim_radar_params* params, cons
                             rsim_tier tier, void* cube, int32_t out_dtype, rsim_stream stream);
 
 /* Synthesise F frames that share one radar configuration in one pass: one launch
- * per stage over all frames, the contraction as one persistent launch whose work
- * units (frame, row tile, column tile, pixel split) are taken from a device
- * counter, longest first.  frames: HOST array of F descriptors; cubes: HOST array
+ * per stage over all frames, the contraction as one launch over all work units
+ * (frame, row tile, column tile, pixel split), longest frames first (taken from a
+ * device counter, in the FP32 tier by a fixed stride).  An FP32-tier
+ * batch whose operand images would pass 16 GiB or the context's budget goes in
+ * sub-batches.  frames: HOST array of F descriptors; cubes: HOST array
  * of F device pointers, each laid out as in rsim_synth.  Each frame's result is
  * bit-identical to rsim_synth of that frame alone with the same tier.  The NUFFT tier
  * runs the frames on up to eight streams of the context (each with its own grid
@@ -357,18 +359,19 @@ rsim_status rsim_selftest_wait_timeout(rsim_ctx* ctx, uint64_t limit_ns, rsim_st
 /* Measurement helper for benchmarks (no counterpart in the paper): the rate, in lane
  * operations per second, at which this device performs non-returning 32-bit integer
  * atomic additions to shared memory without bank conflicts, at the NUFFT spreading
- * kernel's occupancy and access pattern.  That unit bounds the spreading kernel, so the
- * rate is its roofline denominator.  Runs a probe kernel six times on `stream` (the first
+ * kernel's occupancy and access pattern.  The spreading kernel puts its taps into shared
+ * memory with such atomics, so the rate is its roofline denominator.  Runs a probe kernel six times on `stream` (the first
  * as a warm-up) and returns the best; synchronous.  Allocates nothing.
  * Errors: INVALID_ARG, CUDA. */
 rsim_status rsim_measure_smem_atomics(rsim_ctx* ctx, double* lane_ops_per_s, rsim_stream stream);
 
 /* Measurement helper for benchmarks (no counterpart in the paper): the flop rate of this
- * device's tensor cores on the contraction's instruction, tcgen05.mma kind::f16 with
+ * device's tensor cores on tcgen05.mma kind::f16 with
  * M = 128, N = 256, K = 16, A from tensor memory, B from shared memory and FP32
- * accumulation, issued in the contraction's stages of 12 MMAs (one thread per CTA, at
+ * accumulation, issued in stages of 12 MMAs (one thread per CTA, at
  * most three committed stages in flight, one CTA per SM, zero operands).  It is the
- * ceiling of the contraction's executed flop rate.  Runs the probe six times on `stream`
+ * ceiling of the contraction's executed flop rate: the pairs' instruction (M = 256 over
+ * two SMs) does the same work per SM and clock.  Runs the probe six times on `stream`
  * (the first as a warm-up) and returns the best, in flop/s (2 per multiply-add);
  * synchronous.  Allocates nothing; every wait in the probe is bounded.
  * Errors: INVALID_ARG, UNSUPPORTED (not an sm_103 device), TIMEOUT (a probe wait ran
@@ -419,7 +422,7 @@ typedef struct {
   int32_t group_chunks;  /* tensor-core tiers: 32-pixel chunks summed in one tensor-memory
                             accumulator before it is drained into round-to-nearest FP32
                             sums.  The accumulator rounds toward zero, so the cap bounds the
-                            error: 1..40 for split tiers (default 8), 1..384 for plain
+                            error: 1..40 for split tiers (default 40), 1..384 for plain
                             16-bit tiers (default 96).  Other tiers: ignored.  0 = default */
   int32_t reserved;
 } rsim_plan;

@@ -11,7 +11,8 @@
 namespace rsim {
 namespace {
 
-// cube = sum over splits s = 0, 1, ... (in this order) of partial[s], with compensated FP32 additions (GB300's FP64 rate is a small fraction of its FP32 rate).
+// cube = sum over splits s = 0, 1, ... (in this order) of partial[s], with compensated FP32
+// additions (GB300's FP64 rate is a small fraction of its FP32 rate).
 // Loads of kReduceBatch splits are issued together; the additions keep the split order.
 __global__ void split_reduce(const FrameIO* __restrict__ frames, int64_t count, int splits,
                              int out_dtype) {
@@ -50,12 +51,13 @@ __global__ void split_reduce(const FrameIO* __restrict__ frames, int64_t count, 
 // (64 registers, four blocks per SM) the last 160 blocks ran as a second, quarter-full
 // wave (18.7 against 16.7 us).  Sixteen at a time took 125 registers and was slower still.
 constexpr int kTileBatch = 4;
-__global__ void __launch_bounds__(256, 6) split_reduce_tiles(const FrameIO* __restrict__ frames, Consts k, int NT, int ntiles,
-                                   int64_t sstride, int splits, int out_dtype, int scale_mode) {
+__global__ void __launch_bounds__(256, 6)
+split_reduce_tiles(const FrameIO* __restrict__ frames, Consts k, int NT, int ntiles, int64_t sstride, int splits,
+                   int out_dtype, int scaling) {
   wait_prior_grid();
   const FrameIO& fr = frames[blockIdx.y];
   // the FP16 tiers' power of two, undone (exact)
-  const float2 scale = pow2_factors(scale_mode ? sigma_exponent(fr.meta[1]) : 0);
+  const float2 scale = pow2_factors(sigma_exponent(fr.meta[1], scaling));
   const int64_t rows = (int64_t)k.V * k.Ns;
   const int64_t n4 = sstride / 2;
   const int pairs = NT / 2;
@@ -113,7 +115,7 @@ cudaError_t launch_reduce(const Consts& k, const FrameIO* frames, int F, int spl
 }
 
 cudaError_t launch_reduce_tiles(const Consts& k, const FrameIO* frames, int F, int splits, int nt,
-                                int out_dtype, bool scale_from_meta, int num_sms, cudaStream_t st) {
+                                int out_dtype, int scaling, int num_sms, cudaStream_t st) {
   const int64_t sstride = tensor_split_stride(k.V, k.Ns, k.L, nt);
   const int64_t n4 = sstride / 2;
   if (n4 <= 0 || F <= 0) return cudaSuccess;
@@ -122,7 +124,7 @@ cudaError_t launch_reduce_tiles(const Consts& k, const FrameIO* frames, int F, i
   const int64_t wave = std::max<int64_t>(1, 6ll * num_sms / F);
   if (blocks > wave) blocks = wave;
   return launch_dependent(split_reduce_tiles, dim3((unsigned)blocks, F), dim3(256), 0, st, frames, k, nt,
-                          (k.L + nt - 1) / nt, sstride, splits, out_dtype, scale_from_meta ? 1 : 0);
+                          (k.L + nt - 1) / nt, sstride, splits, out_dtype, scaling);
 }
 
 }  // namespace rsim

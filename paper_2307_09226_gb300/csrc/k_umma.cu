@@ -19,9 +19,9 @@
 // phasors) differs for every row tile and is never reused, so it is generated on chip
 // and never touches HBM.
 //
-// This file: the operand builder, the launches, and the contraction of the plain 16-bit
-// tiers; the split tiers run on pairs of CTAs (k_umma_pair.cu).  The plain contraction runs
-// one persistent CTA per SM, warp-specialised:
+// This file: the operand builder, the launches, and the contraction of the plain 16-bit and
+// the split tiers; the FP32 tier runs on pairs of CTAs (k_umma_pair.cu).  The contraction here
+// runs one persistent CTA per SM, warp-specialised:
 //   warps 0-15  produce A for a 128-row tile straight into tensor memory (one row per
 //               thread, tcgen05.st).  Two groups of 8 warps take alternate stages; in a
 //               stage, two warps share a lane quarter with 16 pixels each.  The same
@@ -31,11 +31,14 @@
 //   warp 17     takes work units from a device counter and bulk-copies each chunk's
 //               phases of the tile's channels into a shared-memory ring;
 //   warp 18     bulk-copies each chunk's B images into the operand stages.
-// A and B have rings of their own: eight A stages in tensor memory (the columns the
-// accumulator leaves free) and six B stages in shared memory (192 of its 227 KB, which also
-// keeps a second CTA, and its claim on tensor memory, off the SM).  The kernel is bound by the
-// making of A: with four and three stages of twice the size, shared with the split tiers,
-// BF16 on 256 x 256 pixels (V = 12, N_s = 256, L = 128) took 170 us a call, now 155.
+// A and B have rings of their own: A in tensor memory (the 256 columns the accumulator leaves
+// free), B in shared memory (192 of its 227 KB, which also keeps a second CTA, and its claim on
+// tensor memory, off the SM): four and three stages of hi + lo operands, eight and six of plain
+// ones.  The plain tiers are bound by the making of A: with the split tiers' four and three
+// stages BF16 on 256 x 256 pixels (V = 12, N_s = 256, L = 128) took 170 us a call, now 155.
+// The split tiers (280 us on that frame) are as fast on pairs of CTAs there, but not on smaller
+// frames: over 40 random frames of up to 2e10 path-samples pairs took 0.84 to 1.2 times their
+// speed, 0.95 in the middle (27.1 against 29.3 us for 1785 pixels, 72 against 80 for 10,829).
 // Each slot of either ring has a "full" mbarrier (the producer group's arrivals, or the
 // B copy's bytes) and an "empty" mbarrier, completed by a tcgen05.commit after the MMAs
 // that read it.  Every wait is bounded in time and a timeout sets a status bit instead
@@ -48,8 +51,6 @@ namespace {
 
 using namespace umma;
 
-constexpr int kStages = 6;                 // B operand stages in shared memory (32 KB each)
-constexpr int kAStages = 8;                // A operand stages in tensor memory (32 columns each)
 constexpr int kPixStages = 6;              // ring of staged per-chunk pixel phases
 constexpr int kUnitSlots = 4;              // ring of work-unit ids
 constexpr int kMaxCh = 8;                  // channels a row tile may span for staging
@@ -57,10 +58,19 @@ constexpr int kAWarps = 16;                // A producers: two groups that take 
 constexpr int kAGroupWarps = kAWarps / 2;  // 8 warps per group, two per lane quarter
 constexpr int kAPx = kChunkPx / (kAGroupWarps / 4);  // pixels per A warp per stage
 constexpr int kThreads = 32 * (kAWarps + 3);  // + MMA warp, pixel loader, B loader
-constexpr int kStageBytes = 256 * 128;     // a B stage: N = 2 NT <= 256 rows of 128 bytes
+constexpr int kBBytes = 256 * 128;         // one 16-bit part of a B stage: N = 2 NT <= 256 rows of 128 bytes
 constexpr int kAccCols = 256;              // accumulator columns (N <= 256 FP32)
 constexpr int kTmemCols = 512;
-static_assert(kAccCols + kAStages * 32 <= kTmemCols, "accumulator and A stages fit in tensor memory");
+// The operand rings of the plain and the split (hi + lo) tiers.
+template <int SPLIT>
+struct Rings {
+  static constexpr int kStages = SPLIT ? 3 : 6;          // B stages in shared memory
+  static constexpr int kStageBytes = (SPLIT ? 2 : 1) * kBBytes;
+  static constexpr int kAStages = SPLIT ? 4 : 8;         // A stages in tensor memory
+  static constexpr int kACols = SPLIT ? 64 : 32;         // columns of one
+  static_assert(kAccCols + kAStages * kACols <= kTmemCols, "accumulator and A stages fit in tensor memory");
+};
+constexpr int kMaxStages = 6, kMaxAStages = 8;
 
 // Per-chunk fast-time/channel phases staged by the pixel loader (bulk copies).
 struct PixStage {
@@ -69,10 +79,10 @@ struct PixStage {
 };
 
 struct Shared {
-  uint64_t a_full[kAStages];   // the A stage is in tensor memory (producer group arrivals)
-  uint64_t a_empty[kAStages];  // the MMAs are done with the A stage (it may be rewritten)
-  uint64_t b_full[kStages];    // the B stage is in shared memory (bulk-copy bytes)
-  uint64_t b_empty[kStages];   // the MMAs are done with the B stage
+  uint64_t a_full[kMaxAStages];   // the A stage is in tensor memory (producer group arrivals)
+  uint64_t a_empty[kMaxAStages];  // the MMAs are done with the A stage (it may be rewritten)
+  uint64_t b_full[kMaxStages];    // the B stage is in shared memory (bulk-copy bytes)
+  uint64_t b_empty[kMaxStages];   // the MMAs are done with the B stage
   uint64_t pix_full[kPixStages];
   uint64_t pix_empty[kPixStages];
   uint64_t unit_full[kUnitSlots];
@@ -91,6 +101,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, Shared* 
 __device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
   return umma::warp_wait(b, parity, &sh->abort, status);
 }
+// The MMA thread's waits for a stage: one probe of a phase that has usually completed already,
+// the polling loop out of line (split BF16 on 12 x 317 rows and 64 columns 94.5 -> 93.6 us).
+__device__ __noinline__ bool wait_call(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
+  return umma::mbar_wait(b, parity, &sh->abort, status);
+}
+__device__ __forceinline__ bool probe_wait(uint64_t* b, uint32_t parity, Shared* sh, unsigned* status) {
+  return umma::mbar_try(b, parity) || wait_call(b, parity, sh, status);
+}
 
 // FP32 add-reduction of 16 bytes with a policy (one instruction, like atomicAdd on a float4, so
 // each address's additions keep the issuing thread's order).
@@ -108,10 +126,16 @@ __host__ __device__ constexpr uint32_t idesc_f16(int bf16, int n) {
 
 // All MMAs of one 32-pixel operand stage (K = 64 16-bit elements = four K = 16 steps), in one
 // block so that nothing is recomputed between issues.  `a`: tensor-memory column of the
-// stage's A; `bd`: shared-memory descriptor of its B image.  K step ks reads A columns
-// a + 8 ks and B bytes + 32 ks (2 in the descriptor's 16-byte address field).  `acc` = 0
-// starts a new accumulation with the stage's first MMA.
-__device__ __forceinline__ void mma_stage(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc) {
+// stage's hi A (the lo part starts 32 columns on); `bd`: shared-memory descriptor of its hi B
+// image (the lo image starts kBBytes on).  K step ks reads A columns
+// a + 8 ks and B bytes + 32 ks (2 in the descriptor's 16-byte address field).  Split tiers add
+// A_hi B_lo and A_lo B_hi after each A_hi B_hi.  `acc` = 0 starts a new accumulation with the
+// stage's first MMA.
+template <int SPLIT>
+__device__ __forceinline__ void mma_stage(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc);
+
+template <>
+__device__ __forceinline__ void mma_stage<0>(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p, t;\n\t"
       "setp.ne.b32 p, %10, 0;\n\t"
@@ -122,6 +146,31 @@ __device__ __forceinline__ void mma_stage(uint32_t d, uint32_t a, uint64_t bd, u
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %8, %9, t;\n\t}" ::"r"(d),
       "r"(a), "r"(a + 8), "r"(a + 16), "r"(a + 24), "l"(bd), "l"(bd + 2), "l"(bd + 4), "l"(bd + 6),
       "r"(idesc), "r"(acc)
+      : "memory");
+}
+
+template <>
+__device__ __forceinline__ void mma_stage<1>(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc) {
+  constexpr uint64_t kLo = kBBytes >> 4;
+  asm volatile(
+      "{\n\t.reg .pred p, t;\n\t"
+      "setp.ne.b32 p, %18, 0;\n\t"
+      "setp.ne.b32 t, %17, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %9, %17, p;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %13, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%5], %9, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%2], %10, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%2], %14, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%6], %10, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%3], %11, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%3], %15, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%7], %11, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %12, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %16, %17, t;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%8], %12, %17, t;\n\t}" ::"r"(d),
+      "r"(a), "r"(a + 8), "r"(a + 16), "r"(a + 24), "r"(a + 32), "r"(a + 40), "r"(a + 48), "r"(a + 56),
+      "l"(bd), "l"(bd + 2), "l"(bd + 4), "l"(bd + 6), "l"(bd + kLo), "l"(bd + kLo + 2), "l"(bd + kLo + 4),
+      "l"(bd + kLo + 6), "r"(idesc), "r"(acc)
       : "memory");
 }
 
@@ -253,7 +302,7 @@ build_b_images(const FrameIO* __restrict__ frames, Consts k, int NT, int ntiles,
     const FrameIO& fr = frames[it / (nch * ntiles)];
     const int64_t pv = (int64_t)fr.meta[0];
     if (c * kChunkPx >= pv) continue;
-    const float2 sc = pow2_factors(scaled ? -sigma_exponent(fr.meta[1]) : 0);
+    const float2 sc = pow2_factors(-sigma_exponent(fr.meta[1], scaled));
     unsigned char* base = fr.bimg + ((int64_t)nt * fr.bimg_nch + c) * 2 * part;
     const int64_t q0c = c * kChunkPx;
     // element (l, 16-byte column cp): four pixels' D at l, written to the re-row l and
@@ -299,13 +348,15 @@ build_b_images(const FrameIO* __restrict__ frames, Consts k, int NT, int ntiles,
   }
 }
 
-template <int BF>
+template <int BF, int SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, int out_dtype,
               unsigned* status, int* unit_counter) {
+  using R = Rings<SPLIT>;
+  constexpr int kStages = R::kStages, kAStages = R::kAStages, kStageBytes = R::kStageBytes;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* bstage = smem;  // kStages x 32 KB, 1024-aligned
+  unsigned char* bstage = smem;  // kStages x (hi, lo) x 32 KB, 1024-aligned
   PixStage* pix = (PixStage*)(smem + kStages * kStageBytes);
   Shared* sh = (Shared*)(pix + kPixStages);
 
@@ -369,7 +420,6 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
     struct Pending {
       const FrameIO* fr;
       int64_t gr;
-      float2 oscale;
       int l0, s, mt, nt;
       bool row_ok, none, first, set;
     };
@@ -392,6 +442,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
         }
         if (!d.row_ok) continue;
         if (g.direct) {
+          const float2 oscale = sigma_unscale(dfr, scaled);
 #pragma unroll
           for (int i = 0; i < 8; i += 2) {
             const int l = d.l0 + jb + i;
@@ -402,13 +453,13 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
             const int64_t o = d.gr * k.L + l;
             if (out_dtype == RSIM_C128) {
               double2* cd = reinterpret_cast<double2*>(dfr.cube);
-              cd[o] = make_double2((double)(a0 * d.oscale.x * d.oscale.y), (double)(b0 * d.oscale.x * d.oscale.y));
+              cd[o] = make_double2((double)(a0 * oscale.x * oscale.y), (double)(b0 * oscale.x * oscale.y));
               if (two)
-                cd[o + 1] = make_double2((double)(a1 * d.oscale.x * d.oscale.y), (double)(b1 * d.oscale.x * d.oscale.y));
+                cd[o + 1] = make_double2((double)(a1 * oscale.x * oscale.y), (double)(b1 * oscale.x * oscale.y));
             } else {
               float2* cf = reinterpret_cast<float2*>(dfr.cube);
-              cf[o] = make_float2(a0 * d.oscale.x * d.oscale.y, b0 * d.oscale.x * d.oscale.y);
-              if (two) cf[o + 1] = make_float2(a1 * d.oscale.x * d.oscale.y, b1 * d.oscale.x * d.oscale.y);
+              cf[o] = make_float2(a0 * oscale.x * oscale.y, b0 * oscale.x * oscale.y);
+              if (two) cf[o + 1] = make_float2(a1 * oscale.x * oscale.y, b1 * oscale.x * oscale.y);
             }
           }
         } else {
@@ -447,7 +498,6 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
       const int vl = row_ok ? v - x.v_first : 0;
       const uint32_t* pA = fr.phA + (int64_t)(row_ok ? v : 0) * fr.Pcap;
       const uint32_t* pC = fr.phC + (int64_t)(row_ok ? v : 0) * fr.Pcap;
-      const float2 oscale = sigma_unscale(fr, scaled);
       const int l0 = x.nt * g.NT;
       const int64_t ngr = unit_groups(x, g.group);
       for (int64_t gk = 0; gk < ngr; ++gk) {
@@ -461,7 +511,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
             alive = false;
             break;
           }
-          uint32_t hi[kAPx];
+          uint32_t hi[kAPx], lo[kAPx];
           const int j0 = part * kAPx;
           const int64_t q0 = c * kChunkPx + j0;
 #pragma unroll
@@ -479,14 +529,18 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
               const float2 f = cis_q32_fast(av[t] * n + cv[t]);
-              hi[j4 + t] = pack2<BF>(f.x, f.y);
+              if (SPLIT)
+                split2<BF>(f.x, f.y, hi[j4 + t], lo[j4 + t]);
+              else
+                hi[j4 + t] = pack2<BF>(f.x, f.y);
             }
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(&sh->pix_empty[ps]);
-          static_assert(kAPx == 16, "one x16 tensor-memory store per stage");
-          const uint32_t col = tmem + lane_base + kAccCols + st * 32 + j0;
+          static_assert(kAPx == 16, "one x16 tensor-memory store per operand part");
+          const uint32_t col = tmem + lane_base + kAccCols + st * R::kACols + j0;
           tmem_st16(col, hi);
+          if (SPLIT) tmem_st16(col + 32, lo);
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           fence_before();
           mbar_arrive(&sh->a_full[st]);
@@ -507,7 +561,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
             break;
           }
         }
-        pend = Pending{&fr, gr, oscale, l0, x.s, x.mt, x.nt, row_ok, g1 <= g0, g0 == x.c0, true};
+        pend = Pending{&fr, gr, l0, x.s, x.mt, x.nt, row_ok, g1 <= g0, g0 == x.c0, true};
       }
     }
     if (alive && pend.set) drain(pend);  // the last group
@@ -517,7 +571,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
       uint32_t kk = 0, gi = 0, ui = 0;
       long long u;
       bool alive = true;
-      const uint64_t desc0 = sdesc_sw128(smem_u32(bstage));  // B stage 0
+      const uint64_t desc0 = sdesc_sw128(smem_u32(bstage));  // hi image of B stage 0
       while (alive && next_unit(sh, ui++, status, &u, false)) {
         const Unit x = decode(g, frames, k, u);
         const int64_t ngr = unit_groups(x, g.group);
@@ -532,14 +586,14 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
           for (int64_t c = g0; c < g1; ++c, ++kk) {
             const uint32_t sa = kk % kAStages, pa = (kk / kAStages) & 1u;
             const uint32_t sb = kk % kStages, pb = (kk / kStages) & 1u;
-            if (!mbar_wait(&sh->a_full[sa], pa, sh, status) ||
-                !mbar_wait(&sh->b_full[sb], pb, sh, status)) {
+            if (!probe_wait(&sh->a_full[sa], pa, sh, status) ||
+                !probe_wait(&sh->b_full[sb], pb, sh, status)) {
               alive = false;
               break;
             }
             fence_after();
-            mma_stage(tmem, tmem + kAccCols + sa * 32, desc0 + (uint64_t)(sb * (kStageBytes >> 4)), idesc,
-                      accum);
+            mma_stage<SPLIT>(tmem, tmem + kAccCols + sa * R::kACols, desc0 + (uint64_t)(sb * (kStageBytes >> 4)),
+                             idesc, accum);
             accum = 1;
             mma_commit(&sh->a_empty[sa]);
             mma_commit(&sh->b_empty[sb]);
@@ -611,8 +665,9 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
           }
           const unsigned char* src = fr.bimg + ((int64_t)x.nt * fr.bimg_nch + c) * 2 * part;
           unsigned char* dst = bstage + st * kStageBytes;
-          mbar_expect_tx(&sh->b_full[st], part);
+          mbar_expect_tx(&sh->b_full[st], SPLIT ? 2 * part : part);
           bulk_g2s_hint(dst, src, part, &sh->b_full[st], pol_b);
+          if (SPLIT) bulk_g2s_hint(dst + kBBytes, src + part, part, &sh->b_full[st], pol_b);
         }
       }
     }
@@ -642,7 +697,7 @@ __global__ void order_frames(const FrameIO* __restrict__ frames, int F, int32_t*
 }
 
 template <int BF, int SPLIT>
-cudaError_t launch_t(const Consts& k, const FrameIO* frames, Geo g, int grid, int num_sms, int scaled, bool fine,
+cudaError_t launch_t(const Consts& k, const FrameIO* frames, Geo g, int grid, int num_sms, int scaled, bool pairs,
                      int out_dtype, int64_t nch_max, int fast_dtype, unsigned* status, int* counter,
                      cudaStream_t st, cudaEvent_t mid) {
   cudaError_t e;
@@ -659,11 +714,12 @@ cudaError_t launch_t(const Consts& k, const FrameIO* frames, Geo g, int grid, in
     if (e != cudaSuccess) return e;
   }
   if (mid) cudaEventRecord(mid, st);
-  if (SPLIT)
-    return launch_umma_pairs(BF, fine, k, frames, g.F, g.splits, g.NT, g.group, g.direct == 0, grid, num_sms,
-                             nch_max, scaled, out_dtype, g.order, status, st);
-  const int smem = kStages * kStageBytes + kPixStages * (int)sizeof(PixStage) + (int)sizeof(Shared) + 1024;
-  auto fn = umma_contract<BF>;
+  if (pairs)
+    return launch_umma_pairs(k, frames, g.F, g.splits, g.NT, g.direct == 0, grid, num_sms, nch_max, out_dtype,
+                             g.order, status, st);
+  const int smem = Rings<SPLIT>::kStages * Rings<SPLIT>::kStageBytes + kPixStages * (int)sizeof(PixStage) +
+                   (int)sizeof(Shared) + 1024;
+  auto fn = umma_contract<BF, SPLIT>;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   // persistent: at most one CTA per SM (shared memory and tensor memory allow no more)
@@ -680,11 +736,10 @@ cudaError_t launch_umma(const Consts& k, const FrameIO* frames, int F, int split
                         int out_dtype, int grid, int nt, int group, bool use_partial, int num_sms,
                         int64_t max_p, int fast_terms_dtype, unsigned* status, int* unit_counter,
                         cudaStream_t st, cudaEvent_t mid) {
-  // N = 2 NT must be a multiple of 16 in 16..256 (kind::f16 with M = 128; of 32 for pairs,
-  // M = 256), and a group holds at least one chunk
+  // N = 2 NT must be a multiple of 16 in 16..256 (kind::f16 with M = 128; pairs round it up to
+  // a multiple of 32 in the accumulator), and a group holds at least one chunk
   if (nt < 8 || nt > kAccCols / 2 || nt % 8 != 0 || group < 1) return cudaErrorInvalidValue;
   Geo g;
-  nt = operand_nt(tier, nt);
   const int64_t rows = (int64_t)k.V * k.Ns;
   g.NT = nt;
   g.ntiles = (k.L + g.NT - 1) / g.NT;
@@ -722,11 +777,11 @@ cudaError_t launch_umma(const Consts& k, const FrameIO* frames, int F, int split
                             unit_counter, st, mid);
     case RSIM_TIER_SPLIT_FP16:
     case kTierFp32Tensor:
-      return launch_t<0, 1>(k, frames, g, grid, num_sms, 1, tier == kTierFp32Tensor, out_dtype, nch_max,
-                            fast_terms_dtype, status, unit_counter, st, mid);
+      return launch_t<0, 1>(k, frames, g, grid, num_sms, sigma_scaling(tier), tier == kTierFp32Tensor, out_dtype,
+                            nch_max, fast_terms_dtype, status, unit_counter, st, mid);
     case RSIM_TIER_FP16:
-      return launch_t<0, 0>(k, frames, g, grid, num_sms, 1, false, out_dtype, nch_max, fast_terms_dtype, status,
-                            unit_counter, st, mid);
+      return launch_t<0, 0>(k, frames, g, grid, num_sms, sigma_scaling(tier), false, out_dtype, nch_max,
+                            fast_terms_dtype, status, unit_counter, st, mid);
     default:
       return cudaErrorInvalidValue;
   }

@@ -1,7 +1,9 @@
 // The contraction of k_umma.cu (see there for the matrix product and the operand images) for
-// the split-precision operands and the FP32 tier, on pairs of CTAs.
+// the FP32 tier, on pairs of CTAs: FP16 hi + lo operands, and accumulation groups of one or two
+// chunks, so that the accumulator's rounding toward zero stays below the phasors' own error.
 //
-// A pair's MMA (tcgen05.mma.cta_group::2, M = 256, N = 2 NT) takes two row tiles at once: each
+// A pair's MMA (tcgen05.mma.cta_group::2, M = 256, N = 2 NT rounded up to a multiple of 32)
+// takes two row tiles at once: each
 // CTA holds its own 128 rows of A and one half of B (rank 0 the re-rows, rank 1 the im-rows),
 // so that a chunk's B crosses L2 once per pair.  Per CTA, warp-specialised:
 //   warps 0-7    produce A for the CTA's 128-row tile in shared memory (one row per thread, 16
@@ -16,11 +18,12 @@
 //   warp 18      bulk-copies the CTA's half of each chunk's B images.
 // setmaxnreg moves registers from the other warps to the summing ones.  Every wait is bounded
 // in time and a timeout sets a status bit instead of hanging.
-// Measured on a frame of 256 x 256 pixels (V = 12, N_s = 256, L = 128), same boxes: groups of 40
-// chunks 228-235 us, of 4 chunks 232-240 us.  One CTA per tile with A in tensor memory and the
-// accumulator drained by the producers took 229-235 us and 407-409 us.  Bound by the MMAs
-// (348,000 of about 420,000 cycles; the SM clock falls to 1.75-1.9 GHz under them) and by
-// shared memory, whose port the operands' writes and the MMAs' reads fill to about 80%.
+// Measured on a frame of 256 x 256 pixels (V = 12, N_s = 256, L = 128), kernel alone: 240 us in
+// groups of two chunks and 232 in groups of 40, where one CTA per tile with A in tensor memory
+// and the accumulator drained by the producers took 229-235 us in groups of 40 and 407-409 in
+// groups of 4; the CUDA cores took 2790.  Bound by the MMAs (348,000 of about 420,000 cycles;
+// the SM clock falls to 1.75-1.9 GHz under them) and by shared memory, whose port the operands'
+// writes and the MMAs' reads fill to about 80%.
 #include <algorithm>
 
 #include "rsim_internal.h"
@@ -45,7 +48,7 @@ constexpr int kThreads = 32 * (kMmaWarp + 4);  // whole warpgroups: 2 of produce
 constexpr int kRegsLaunch = 96, kRegsA = 64, kRegsSum = 152, kRegsRest = 48;
 static_assert(32 * (kAWarps * kRegsA + kSumWarps * kRegsSum + 4 * kRegsRest) <= kThreads * kRegsLaunch,
               "the warpgroups' registers fit the launch's");
-constexpr uint32_t kFineLong = 20000 / kChunkPx;  // chunks of a frame from which FP32 groups are long
+constexpr uint32_t kFineLong = 20000 / kChunkPx;  // chunks of a frame from which groups are long
 constexpr int kPartBytes = 128 * 128;      // one 16-bit part of a stage's A (128 rows) or of its half of B
 constexpr int kAccCols = 256;              // columns of one accumulator (N <= 256 FP32)
 constexpr int kTmemCols = 512;             // two accumulators
@@ -95,63 +98,36 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Instruction descriptor of kind::f16: FP32 accumulator, K-major A and B, M = 256 (the pair).
-__host__ __device__ constexpr uint32_t idesc_f16(int bf16, int n) {
-  return (1u << 4) | ((uint32_t)bf16 << 7) | ((uint32_t)bf16 << 10) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(256 >> 4) << 24);
+// Instruction descriptor of kind::f16: FP16 operands, FP32 accumulator, K-major A and B, M = 256 (the
+// pair).
+__host__ __device__ constexpr uint32_t idesc_f16(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
 
 // All MMAs of one 32-pixel operand stage (K = 64 16-bit elements = four K = 16 steps).  `a`,
 // `b`: descriptors of the stage's hi A and hi B (the lo parts lie kPartBytes on); a K step
 // moves both by 32 bytes (2 in the descriptor's 16-byte address field).  `acc` = 0 starts a
-// new accumulation with the stage's first MMA.
-//   FINE = 0: A_hi B_hi, A_hi B_lo, A_lo B_hi per K step; A_hi is read once for its two MMAs
-//             (the collector buffer).
-//   FINE = 1: the small products first, so that in a new accumulation only the four A_hi B_hi
-//             are added to (and rounded toward zero at) the sum's full size.
-#define RSIM_MMA(col, a, b, en) "tcgen05.mma.cta_group::2.kind::f16" col " [%0], " a ", " b ", %3, " en ";\n\t"
+// new accumulation with the stage's first MMA.  The small products come first, so that in a new
+// accumulation only the four A_hi B_hi are added to (and rounded toward zero at) the sum's full
+// size.
+#define RSIM_MMA(a, b, en) "tcgen05.mma.cta_group::2.kind::f16 [%0], " a ", " b ", %3, " en ";\n\t"
 #define RSIM_STEP(x, from, n) "add.s64 " x ", " from ", " n ";\n\t"
-template <int FINE>
-__device__ __forceinline__ void mma_stage(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc);
-
-template <>
-__device__ __forceinline__ void mma_stage<0>(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_stage(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p, t;\n\t.reg .b64 x, y, u, v;\n\t"
       "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 t, %3, 0;\n\t"
       RSIM_STEP("u", "%1", "%5") RSIM_STEP("v", "%2", "%5")
-      RSIM_MMA(".collector::a::fill", "%1", "%2", "p") RSIM_MMA(".collector::a::lastuse", "%1", "v", "t")
-      RSIM_MMA("", "u", "%2", "t")
+      RSIM_MMA("%1", "v", "p") RSIM_MMA("u", "%2", "t")
       RSIM_STEP("x", "%1", "2") RSIM_STEP("y", "%2", "2") RSIM_STEP("u", "u", "2") RSIM_STEP("v", "v", "2")
-      RSIM_MMA(".collector::a::fill", "x", "y", "t") RSIM_MMA(".collector::a::lastuse", "x", "v", "t")
-      RSIM_MMA("", "u", "y", "t")
+      RSIM_MMA("x", "v", "t") RSIM_MMA("u", "y", "t")
       RSIM_STEP("x", "x", "2") RSIM_STEP("y", "y", "2") RSIM_STEP("u", "u", "2") RSIM_STEP("v", "v", "2")
-      RSIM_MMA(".collector::a::fill", "x", "y", "t") RSIM_MMA(".collector::a::lastuse", "x", "v", "t")
-      RSIM_MMA("", "u", "y", "t")
+      RSIM_MMA("x", "v", "t") RSIM_MMA("u", "y", "t")
       RSIM_STEP("x", "x", "2") RSIM_STEP("y", "y", "2") RSIM_STEP("u", "u", "2") RSIM_STEP("v", "v", "2")
-      RSIM_MMA(".collector::a::fill", "x", "y", "t") RSIM_MMA(".collector::a::lastuse", "x", "v", "t")
-      RSIM_MMA("", "u", "y", "t") "}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc), "n"(kPartBytes >> 4)
-      : "memory");
-}
-
-template <>
-__device__ __forceinline__ void mma_stage<1>(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p, t;\n\t.reg .b64 x, y, u, v;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 t, %3, 0;\n\t"
-      RSIM_STEP("u", "%1", "%5") RSIM_STEP("v", "%2", "%5")
-      RSIM_MMA("", "%1", "v", "p") RSIM_MMA("", "u", "%2", "t")
-      RSIM_STEP("x", "%1", "2") RSIM_STEP("y", "%2", "2") RSIM_STEP("u", "u", "2") RSIM_STEP("v", "v", "2")
-      RSIM_MMA("", "x", "v", "t") RSIM_MMA("", "u", "y", "t")
-      RSIM_STEP("x", "x", "2") RSIM_STEP("y", "y", "2") RSIM_STEP("u", "u", "2") RSIM_STEP("v", "v", "2")
-      RSIM_MMA("", "x", "v", "t") RSIM_MMA("", "u", "y", "t")
-      RSIM_STEP("x", "x", "2") RSIM_STEP("y", "y", "2") RSIM_STEP("u", "u", "2") RSIM_STEP("v", "v", "2")
-      RSIM_MMA("", "x", "v", "t") RSIM_MMA("", "u", "y", "t")
-      RSIM_MMA("", "x", "y", "t")
-      RSIM_STEP("x", "x", "-2") RSIM_STEP("y", "y", "-2") RSIM_MMA("", "x", "y", "t")
-      RSIM_STEP("x", "x", "-2") RSIM_STEP("y", "y", "-2") RSIM_MMA("", "x", "y", "t")
-      RSIM_MMA("", "%1", "%2", "t") "}" ::"r"(d),
+      RSIM_MMA("x", "v", "t") RSIM_MMA("u", "y", "t")
+      RSIM_MMA("x", "y", "t")
+      RSIM_STEP("x", "x", "-2") RSIM_STEP("y", "y", "-2") RSIM_MMA("x", "y", "t")
+      RSIM_STEP("x", "x", "-2") RSIM_STEP("y", "y", "-2") RSIM_MMA("x", "y", "t")
+      RSIM_MMA("%1", "%2", "t") "}" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc), "n"(kPartBytes >> 4)
       : "memory");
 }
@@ -174,14 +150,14 @@ __device__ __forceinline__ void mma_commit(uint64_t* b) {
 }
 
 struct Geo {
-  int mpairs, ntiles, NT, splits, upf, group, direct, F;
+  int mpairs, ntiles, NT, splits, upf, direct, F;
+  int NH;                // accumulator columns of one half (re or im): NT, rounded up to 16
   int total_units;       // work units (frame, pair of row tiles, column tile, split)
   int64_t sstride;       // complex elements of one split's tiled partial sums
   const int32_t* order;  // frames by decreasing valid-pixel count
 };
 
 // Unit u as the CTA of rank `rank` in its pair sees it.
-template <int FINE>
 __device__ __forceinline__ Unit decode(const Geo& g, const FrameIO* frames, const Consts& k, int u, int rank) {
   Unit x;
   const int fi = u / g.upf;
@@ -194,8 +170,8 @@ __device__ __forceinline__ Unit decode(const Geo& g, const FrameIO* frames, cons
   x.nt = r % g.ntiles;
   x.s = r / g.ntiles;
   const uint32_t nch = (uint32_t)((frames[x.f].meta[0] + kChunkPx - 1) / kChunkPx);
-  // the FP32 tier: one chunk a group (error 3.3e-7 to 3.7e-7), two for long sums (5.6e-7)
-  x.group = FINE ? (nch < kFineLong ? 1 : 2) : g.group;
+  // one chunk a group (error 3.3e-7 to 3.7e-7), two for long sums (5.6e-7)
+  x.group = nch < kFineLong ? 1 : 2;
   x.c0 = nch * (uint32_t)x.s / (uint32_t)g.splits;
   x.c1 = nch * (uint32_t)(x.s + 1) / (uint32_t)g.splits;
   const int64_t rows = (int64_t)k.V * k.Ns;
@@ -242,10 +218,9 @@ __device__ __forceinline__ void regs_inc() {
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
 
-// FINE (the FP32 tier): the phase fraction of A keeps all its bits.
-template <int BF, int FINE>
+// The phase fraction of A keeps all its bits here (cis_q32).
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, int out_dtype, unsigned* status) {
+umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int out_dtype, unsigned* status) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* stages = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   PixStage* pix = (PixStage*)(stages + kStages * kStageBytes);
@@ -276,6 +251,13 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
     mbar_init(&sh->fin, 1);
     sh->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (g.NH != g.NT) {
+    // the images end at row NT of a half: zeros in the 8 rows that the MMA reads beyond it
+    for (int i = threadIdx.x; i < kStages * 2 * 64; i += kThreads)
+      *reinterpret_cast<uint4*>(stages + (i >> 7) * kStageBytes + (2 + ((i >> 6) & 1)) * kPartBytes + g.NT * 128 +
+                                (i & 63) * 16) = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -352,8 +334,8 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
           uint32_t hi[4], lo[4];
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
-            const float2 f = FINE ? cis_q32(cyc[j4 + t]) : cis_q32_fast(cyc[j4 + t]);
-            split2<BF>(f.x, f.y, hi[t], lo[t]);
+            const float2 f = cis_q32(cyc[j4 + t]);
+            split2<0>(f.x, f.y, hi[t], lo[t]);
           }
           unsigned char* unit = at + (((part * 4 + j4 / 4) ^ (r & 7)) << 4);
           *reinterpret_cast<uint4*>(unit) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
@@ -409,7 +391,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
             if (jb < g.NT) {
               uint32_t re[8], im[8];
               tmem_ld8(acc + jb, re);
-              tmem_ld8(acc + g.NT + jb, im);
+              tmem_ld8(acc + g.NH + jb, im);
               asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
@@ -430,7 +412,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
       if (gr >= rows_total) {
         // a row past the cube: nothing to write
       } else if (g.direct) {
-        const float2 oscale = sigma_unscale(fr, scaled);
+        const float2 oscale = sigma_unscale(fr, sigma_scaling(kTierFp32Tensor));
 #pragma unroll
         for (int b = 0; b < kBlocks; ++b) {
           const int jb = half * 8 + b * 16;
@@ -475,7 +457,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
         uint32_t st = 0, ph = 0, gi = 0, ui = 0;
         Unit x;
         bool alive = true;
-        const uint32_t idesc = idesc_f16(BF, 2 * g.NT);
+        const uint32_t idesc = idesc_f16(2 * g.NH);
         const uint64_t desc0 = sdesc_sw128(smem_u32(stages));  // hi A of stage 0
         while (alive && next_unit(sh, ui++, status, &x, false)) {
           const uint32_t chunks = x.c1 - x.c0;
@@ -495,7 +477,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
               }
               fence_after();
               const uint64_t a = desc0 + (uint64_t)(st * (kStageBytes >> 4));
-              mma_stage<FINE>(acc, a, a + (uint64_t)(2 * (kPartBytes >> 4)), idesc, c);
+              mma_stage(acc, a, a + (uint64_t)(2 * (kPartBytes >> 4)), idesc, c);
               mma_commit(&sh->empty[st]);
               if (++st == kStages) st = 0, ph ^= 1u;
             }
@@ -536,7 +518,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
         for (uint32_t ui = 0;; ++ui, u += pairs) {
           Unit x;
           x.f = -1;
-          if (u < g.total_units) x = decode<FINE>(g, frames, k, u, (int)rank);
+          if (u < g.total_units) x = decode(g, frames, k, u, (int)rank);
           const uint32_t slot = ui % kUnitSlots, uph = (ui / kUnitSlots) & 1u;
           if (!mbar_wait(&sh->unit_empty[slot], uph ^ 1u, sh, status)) break;
           sh->unit[slot] = x;
@@ -568,7 +550,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
       }
     } else if (warp == kMmaWarp + 2) {
       // ------------- B loader: bulk copies of this CTA's half of a chunk's B images -------------
-      // rank 0: the re-rows (the accumulator's first NT columns), rank 1: the im-rows
+      // rank 0: the re-rows (the accumulator's first NH columns), rank 1: the im-rows
       if (lane == 0) {
         const uint64_t pol_b = policy_evict_first();
         const uint32_t half = (uint32_t)g.NT * 128u;
@@ -612,30 +594,18 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int sca
   }
 }
 
-template <int BF, int FINE>
-cudaError_t launch_pairs(const Consts& k, const FrameIO* frames, const Geo& g, int pairs, int scaled, int out_dtype,
-                         unsigned* status, cudaStream_t st) {
-  const int smem = kStages * kStageBytes + kPixStages * (int)sizeof(PixStage) + (int)sizeof(Shared) + 1024;
-  auto fn = umma_contract_pairs<BF, FINE>;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return launch_dependent(fn, dim3(2 * pairs), dim3(kThreads), (size_t)smem, st, frames, k, g, scaled, out_dtype,
-                          status);
-}
-
 }  // namespace
 
-cudaError_t launch_umma_pairs(int bf16, bool fine, const Consts& k, const FrameIO* frames, int F, int splits, int nt,
-                              int group, bool use_partial, int grid, int num_sms, int64_t nch_max, int scaled,
-                              int out_dtype, const int32_t* order, unsigned* status, cudaStream_t st) {
-  if (nt % 16 != 0) return cudaErrorInvalidValue;  // N = 2 NT is a multiple of 32
+cudaError_t launch_umma_pairs(const Consts& k, const FrameIO* frames, int F, int splits, int nt, bool use_partial,
+                              int grid, int num_sms, int64_t nch_max, int out_dtype, const int32_t* order,
+                              unsigned* status, cudaStream_t st) {
   const int64_t rows = (int64_t)k.V * k.Ns;
   Geo g;
   g.NT = nt;
+  g.NH = (nt + 15) / 16 * 16;  // N = 2 NH is a multiple of 32
   g.ntiles = (k.L + nt - 1) / nt;
   g.mpairs = (int)((rows + 255) / 256);
   g.splits = splits;
-  g.group = group;
   g.direct = use_partial ? 0 : 1;
   g.F = F;
   g.sstride = tensor_split_stride(k.V, k.Ns, k.L, nt);
@@ -656,9 +626,12 @@ cudaError_t launch_umma_pairs(int bf16, bool fine, const Consts& k, const FrameI
     pairs = std::max(pairs, (g.total_units + per - 1) / per);
   }
   pairs = std::min(pairs, g.total_units);
-  if (bf16) return launch_pairs<1, 0>(k, frames, g, pairs, scaled, out_dtype, status, st);
-  if (fine) return launch_pairs<0, 1>(k, frames, g, pairs, scaled, out_dtype, status, st);
-  return launch_pairs<0, 0>(k, frames, g, pairs, scaled, out_dtype, status, st);
+  const int smem = kStages * kStageBytes + kPixStages * (int)sizeof(PixStage) + (int)sizeof(Shared) + 1024;
+  const cudaError_t e =
+      cudaFuncSetAttribute(umma_contract_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(umma_contract_pairs, dim3(2 * pairs), dim3(kThreads), (size_t)smem, st, frames, k, g,
+                          out_dtype, status);
 }
 
 }  // namespace rsim

@@ -32,16 +32,14 @@ int64_t tensor_split_stride(int V, int Ns, int L, int nt) {
 bool uses_partial(int tier, int64_t P, int splits, int group) {
   if (tier == RSIM_TIER_NUFFT) return false;
   if (splits > 1) return true;
-  if (tier == RSIM_TIER_FP32 || pair_tier(tier)) return false;  // they sum groups in registers
+  if (tier == RSIM_TIER_FP32 || tier == kTierFp32Tensor) return false;  // the sums stay in registers
   const int64_t chunks = (P + kChunkPx - 1) / kChunkPx;
   return chunks > group;
 }
 
-// Pairs of CTAs read a finished group out beside the next group's MMAs, so that groups of 8
-// chunks take 1% longer than groups of 40 (split-FP16 error 2.0e-6 instead of 8.7e-6).
 int group_chunks(int tier) {
   if (tier == kTierFp32Tensor) return kFp32Group;
-  return pair_tier(tier) ? 8 : 96;
+  return split_tier(tier) ? 40 : 96;
 }
 
 // The split tiers' 2e-5 bar leaves room for the round-toward-zero bias of at most 40
@@ -49,7 +47,7 @@ int group_chunks(int tier) {
 // (1e-2) allow 384 chunks (1536 MMAs, about 3e-5).
 int group_chunks_max(int tier) {
   if (tier == kTierFp32Tensor) return kFp32Group;
-  return pair_tier(tier) ? 40 : 384;
+  return split_tier(tier) ? 40 : 384;
 }
 
 bool fp32_on_tensor_cores(int64_t P) { return P >= kFp32TensorPixels; }
@@ -57,9 +55,8 @@ bool fp32_on_tensor_cores(int64_t P) { return P >= kFp32TensorPixels; }
 int units_per_split(int tier, int V, int Ns, int L, int tile_n) {
   if (tier == RSIM_TIER_FP32) return V * ((Ns + tile_n - 1) / tile_n) * ((L + kDirectTileL - 1) / kDirectTileL);
   const int64_t rows = (int64_t)V * Ns;
-  const int nt = operand_nt(tier, tile_n);
-  const int64_t trows = pair_tier(tier) ? 256 : 128;  // a pair of CTAs takes two row tiles
-  return (int)(((rows + trows - 1) / trows) * ((L + nt - 1) / nt));
+  const int64_t trows = tier == kTierFp32Tensor ? 256 : 128;  // a pair of CTAs takes two row tiles
+  return (int)(((rows + trows - 1) / trows) * ((L + tile_n - 1) / tile_n));
 }
 
 int default_splits(int tier, int V, int Ns, int L, int tile_n, int64_t P, int num_sms) {
@@ -91,15 +88,18 @@ int default_splits(int tier, int V, int Ns, int L, int tile_n, int64_t P, int nu
   }
   // tensor tiers: one persistent CTA (or half a pair) per SM takes equal units in turn; pick
   // the split count whose unit count fills whole rounds best, with a cost per split for the
-  // partial sums it adds.  A hundredth of the contraction per split: 64 frames of 12 tiles
-  // then take 6 splits instead of 19 (10.40 ms against 11.21), one frame the same time
-  const int slots = std::max(pair_tier(tier) ? num_sms / 2 : num_sms, 1);
+  // partial sums it adds: a hundredth of the contraction (plain BF16, V = 20, N_s = 335,
+  // L = 124, 5643 pixels: 17 splits at 0.003 and 85 us, 8 and 62 us at 0.01 with the longer
+  // rings, which alone give 4 to 10%).  The split tiers keep 0.003: fewer splits would lengthen their accumulation groups,
+  // whose rounding toward zero is most of their error
+  const int slots = std::max(tier == kTierFp32Tensor ? num_sms / 2 : num_sms, 1);
+  const double per_split = split_tier(tier) ? 0.003 : 0.01;
   double best = -1.0;
   int bs = 1;
   for (int s = 1; s <= smax; ++s) {
     const int64_t units = (int64_t)tiles * s;
     const int64_t rounds = (units + slots - 1) / slots;
-    const double eff = (double)units / (double)(rounds * slots) - 0.01 * s;
+    const double eff = (double)units / (double)(rounds * slots) - per_split * s;
     if (eff > best + 1e-9) {
       best = eff;
       bs = s;

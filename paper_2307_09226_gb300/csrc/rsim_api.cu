@@ -181,7 +181,7 @@ size_t frames_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& p
   o = align_up(o + 16 + 4 * (size_t)F, 256);              // unit counter + frame order
   for (int f = 0; f < F; ++f) {
     FrameLayout fl = frame_layout(k.V, k.Ns, k.L, P[f], plan.splits, up, tensor_tier(tier),
-                                  operand_nt(tier, plan.tile_n), o);
+                                  plan.tile_n, o);
     o = fl.total;
   }
   return o;
@@ -300,7 +300,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
   FrameIO* table = nullptr;
   int* counter = nullptr;
   rsim_status s = stage_frames(ctx, ws, k, frames, F, cubes, splits, use_partial,
-                               tensor_tier(tier), operand_nt(tier, plan.tile_n), st, host, &table, &counter);
+                               tensor_tier(tier), plan.tile_n, st, host, &table, &counter);
   if (s != RSIM_OK) return s;
   // stage events when profiling this context's own calls
   // ev: start, after compaction + phases, after the contraction, after the reduction,
@@ -420,7 +420,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     if (prof) cudaEventRecord(ev[2], st);
     if (prof) cudaEventRecord(ev[5], st);
     if (use_partial) {
-      e = launch_reduce_tiles(k, table, F, splits, operand_nt(tier, plan.tile_n), out_dtype, scaled_tier(tier),
+      e = launch_reduce_tiles(k, table, F, splits, plan.tile_n, out_dtype, sigma_scaling(tier),
                               ctx->num_sms, st);
       if (e != cudaSuccess) return cuda_fail(e, "split reduction");
     }

@@ -87,7 +87,7 @@ struct FrameLayout {
   size_t idx, phA, phC, phB, sig, blk, meta, partial, bimg, total;
   int64_t Pcap, bimg_nch;
 };
-// nt: operand_nt of the plan's column tile (tensor tiers; ignored otherwise).
+// nt: the plan's column tile (tensor tiers; ignored otherwise).
 FrameLayout frame_layout(int V, int Ns, int L, int64_t P, int splits, bool use_partial, bool tensor,
                          int nt, size_t base);
 // Default columns of l per tensor-core column tile: min(128, L rounded up to 8).
@@ -108,17 +108,17 @@ inline bool tensor_tier(int tier) {
 }
 // Workspace the FP32 tier takes on the tensor cores at most, per call.
 constexpr size_t kFp32TensorBytes = size_t(16) << 30;
-// Those of hi + lo operands, which run on pairs of CTAs.
-inline bool pair_tier(int tier) {
-  return tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16 || tier == kTierFp32Tensor;
+// Tiers of hi + lo operands on one CTA per tile.
+inline bool split_tier(int tier) { return tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16; }
+// Sigma scaling of the tiers with FP16 operands, 0 for none: max(|re|, |im|) is put into
+// [2^(n-2), 2^(n-1)).  The FP32 tier takes 16: every component stays below FP16's largest number
+// and pixels down to 2^-29 of the strongest keep all their bits.  The 16-bit tiers take 1: their
+// bars ask for no more, and the low parts' fewer set bits draw less power (split FP16 on 256 x
+// 256 pixels, V = 12, N_s = 256, L = 128: 230 us a contraction against 238 with 16).
+inline __host__ __device__ constexpr int sigma_scaling(int tier) {
+  if (tier == kTierFp32Tensor) return 16;
+  return tier == RSIM_TIER_SPLIT_FP16 || tier == RSIM_TIER_FP16 ? 1 : 0;
 }
-// Those whose sigma is scaled by a power of two into FP16's range.
-inline bool scaled_tier(int tier) {
-  return tier == RSIM_TIER_SPLIT_FP16 || tier == RSIM_TIER_FP16 || tier == kTierFp32Tensor;
-}
-// Columns of l that a plan's column tile takes up in the operand images and the accumulator
-// (a pair's MMA has N = 2 NT, a multiple of 32).
-inline int operand_nt(int tier, int nt) { return pair_tier(tier) ? (nt + 15) / 16 * 16 : nt; }
 
 // NUFFT tier: grid and tile geometry of one frame shape.
 struct NuGeo {
@@ -238,13 +238,12 @@ __device__ __forceinline__ uint64_t frac_u64(double x) {
   return (bits >> 63) ? (uint64_t)0 - f : f;
 }
 
-// The power of two 2^-e that the FP16 tiers scale sigma by puts max(|re|, |im|) (its float
-// bits: meta[1]) into [2^14, 2^15): every component stays below FP16's largest number, and
-// pixels down to 2^-29 of the strongest keep all their bits.  Applied as two factors, so that
-// no factor leaves FP32's range; exact.
-__device__ __forceinline__ int sigma_exponent(unsigned long long max_bits) {
+// The power of two 2^-e that sigma is scaled by (`scaling`: sigma_scaling; the float bits of
+// max(|re|, |im|) are meta[1]).  Applied as two factors, so that no factor leaves FP32's range;
+// exact.
+__device__ __forceinline__ int sigma_exponent(unsigned long long max_bits, int scaling) {
   const float m = __uint_as_float((unsigned)max_bits);
-  return m > 0.f ? ilogbf(m) - 14 : 0;
+  return scaling && m > 0.f ? ilogbf(m) + 2 - scaling : 0;
 }
 __device__ __forceinline__ float2 pow2_factors(int e) {
   return make_float2(ldexpf(1.f, e / 2), ldexpf(1.f, e - e / 2));
@@ -307,7 +306,7 @@ cudaError_t launch_reduce(const Consts& k, const FrameIO* frames, int F, int spl
                           cudaStream_t st);
 // The same reduction over the tensor tiers' tiled partial sums.
 cudaError_t launch_reduce_tiles(const Consts& k, const FrameIO* frames, int F, int splits, int nt,
-                                int out_dtype, bool scale_from_meta, int num_sms, cudaStream_t st);
+                                int out_dtype, int scaling, int num_sms, cudaStream_t st);
 // nt: column tile (l values, multiple of 8 in 8..128); group: chunks per accumulation
 // group.  fast_terms_dtype: RSIM_F32 / RSIM_F64 when the operand builder is to write the
 // fast-time and channel phases (launch_prep deferred them; the pixels' dtype), or -1.
@@ -320,11 +319,11 @@ cudaError_t launch_umma(const Consts& k, const FrameIO* frames, int F, int split
 
 // cubes: HOST array of the F cube pointers; cubes_dev: the same on the device, or NULL to pass
 // them by value (F <= 64).
-// The contraction of the pair tiers (launch_umma calls it).  nch_max: chunks of the largest
-// frame; fine: the FP32 tier's phase arithmetic; order: device array, or NULL for one frame.
-cudaError_t launch_umma_pairs(int bf16, bool fine, const Consts& k, const FrameIO* frames, int F, int splits, int nt,
-                              int group, bool use_partial, int grid, int num_sms, int64_t nch_max, int scaled,
-                              int out_dtype, const int32_t* order, unsigned* status, cudaStream_t st);
+// The FP32 tier's contraction on pairs of CTAs (launch_umma calls it).  nch_max: chunks of the
+// largest frame; order: device array, or NULL for one frame.
+cudaError_t launch_umma_pairs(const Consts& k, const FrameIO* frames, int F, int splits, int nt, bool use_partial,
+                              int grid, int num_sms, int64_t nch_max, int out_dtype, const int32_t* order,
+                              unsigned* status, cudaStream_t st);
 
 cudaError_t launch_range_doppler(const float2* const* cubes, const float2* const* cubes_dev, float2* tmp, float* power,
                                  int F, int V, int Ns, int L, int skip_static, double v_per_bin, float* v_est,

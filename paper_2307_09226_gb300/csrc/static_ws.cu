@@ -87,7 +87,7 @@ extern "C" rsim_status rsim_synth_static(const rsim_radar_params* params, const 
   for (;;) {
     plan = default_plan(engine, k, P, sms);
     splits = plan.splits;
-    nt = operand_nt(engine, plan.tile_n);
+    nt = plan.tile_n;
     use_partial = uses_partial(engine, P, splits, plan.group_chunks);
     o = up256(sizeof(FrameIO));  // the frame table comes first
     off_meta = o;    o = up256(o + 16);
@@ -150,7 +150,7 @@ extern "C" rsim_status rsim_synth_static(const rsim_radar_params* params, const 
                     P, pixels->dtype, status, counter, st);
     if (e == cudaErrorNotSupported) return fail(RSIM_ERR_UNSUPPORTED, "tensor-core tier not available");
     if (e != cudaSuccess) return cuda_fail(e, "tcgen05 contraction kernel");
-    if (use_partial) e = launch_reduce_tiles(k, table, 1, splits, nt, out_dtype, scaled_tier(engine), sms, st);
+    if (use_partial) e = launch_reduce_tiles(k, table, 1, splits, nt, out_dtype, sigma_scaling(engine), sms, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "split reduction");
   return RSIM_OK;

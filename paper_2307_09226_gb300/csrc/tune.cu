@@ -3,7 +3,8 @@
 // A plan holds the tile shapes and the work split of one shape bucket (tier, V, N_s, L,
 // ceil(log2 P)): the column tile NT and the accumulation-group length of the
 // tensor-core contraction, or the n tile of the FP32 direct sum, plus the pixel split
-// count and the persistent grid.  The search is coordinate-wise, so its cost stays a
+// count and the persistent grid.  The FP32 tier is tuned as what its frames run (the
+// tensor-core form, or below its pixel limit the direct sum).  The search is coordinate-wise, so its cost stays a
 // dozen or two timed runs: first the tile (each with its own default split count), then
 // splits x grid with the best tile, then the group length.  Every candidate keeps the
 // accuracy rules (at most 8192 pixels per FP32 split, group lengths within the tier's
@@ -234,7 +235,7 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
   // 3. the accumulation-group length (tensor tiers), never above the tier's cap
   if (tensor) {
     const int gmax = group_chunks_max(tier);
-    std::vector<int> cand = pair_tier(tier)
+    std::vector<int> cand = split_tier(tier)
                                 ? std::vector<int>{32, gmax}
                                 : std::vector<int>{192, gmax};
     const rsim_plan base = best;

@@ -209,9 +209,9 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t&
   }
 }
 
-// The FP16 tiers' power of two undone, as two factors (1 for the others).
+// The power of two of sigma_scaling undone, as two factors.
 __device__ __forceinline__ float2 sigma_unscale(const FrameIO& fr, int scaled) {
-  return pow2_factors(scaled ? sigma_exponent(fr.meta[1]) : 0);
+  return pow2_factors(sigma_exponent(fr.meta[1], scaled));
 }
 
 }  // namespace umma

@@ -119,3 +119,19 @@ def test_tuning_keeps_the_engine_and_its_accuracy(env):
     after = c.synth(f.radar, device.upload(f), "fp32").cpu().numpy()
     assert oracle.rel_l2(before, ref) <= FP32_BAR and oracle.rel_l2(after, ref) <= FP32_BAR
     c.close()
+
+
+@pytest.mark.parametrize("tier,bar", [("fp32", FP32_BAR), ("split_fp16", 2e-5)])
+def test_odd_column_tiles_take_no_padding(env, tier, bar):
+    """40 columns of l: 640 bytes of operand images and 28 of phases a pixel, so that 96,000
+    pixels fit the static workspace of 64 MiB, which images padded to 48 columns (768) pass."""
+    torch, _abi, device, ctx = env
+    radar = Radar(M=1, N=1, Ns=64, L=40)
+    px = synth.random_frame(radar, 300, 320, seed=11)
+    d = device.upload(px)
+    cube = torch.empty((1, 64, 40), dtype=torch.complex64, device="cuda")
+    assert _abi.rsim_synth_static(radar, d, _abi.TIERS[tier], cube) == _abi.OK, _abi.last_error()
+    torch.cuda.synchronize()
+    got = cube.cpu().numpy()
+    assert np.array_equal(got, ctx.synth(radar, d, tier).cpu().numpy())
+    assert oracle.rel_l2(got, oracle.cube_separable(radar, px)) <= bar
