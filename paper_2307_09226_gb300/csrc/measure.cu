@@ -1,20 +1,21 @@
-// Measured peaks of the units that bound two kernels, taken on the device the library
+// Measured peaks of the units that two kernels lean on, taken on the device the library
 // runs on (the roofline denominators the benchmarks report beside vendor-library figures).
 //
 // 1. The NUFFT tier's spreading kernel: non-returning
 // 32-bit integer atomic additions to shared memory without bank conflicts.  The
-// spreading kernel adds every tap of a record with such atomics (two words per
-// component, see k_nufft.cu), so this rate, taken on the device the library runs on,
-// is the roofline denominator of that kernel.  The probe has the spreading kernel's
-// occupancy (four blocks of 256 threads per SM) and its access pattern: each atomic
+// spreading kernel adds the taps of every run of points in one cell with such atomics
+// (two words per component, see k_nufft.cu), so this rate, taken on the device the
+// library runs on, is the roofline denominator of that kernel.  The probe has four blocks
+// of 256 threads per SM and the spreading kernel's access pattern: each atomic
 // instruction of a warp touches 32 consecutive words, one per bank, of one of four word
 // arrays.
 //
 // 2. The contraction's tensor-core instruction: tcgen05.mma kind::f16, M = 128, N = 256,
 // K = 16, A from tensor memory and B from shared memory (128-byte-swizzled K-major), FP32
-// accumulation, issued in the contraction's 12-MMA stages by one thread per CTA with at
+// accumulation, issued in 12-MMA stages by one thread per CTA with at
 // most three committed stages in flight, one CTA per SM, on zero operands.  Its flop rate
-// is the ceiling of the contraction's executed flop rate (a cuBLAS GEMM, the measured
+// is the ceiling of the contraction's executed flop rate, also of the kernel on pairs of CTAs,
+// whose M = 256 instruction does the same work per SM and clock (a cuBLAS GEMM, the measured
 // BF16 peak, also spends time outside its MMAs).
 #include <cuda_runtime.h>
 
