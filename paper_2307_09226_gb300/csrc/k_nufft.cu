@@ -29,9 +29,9 @@
 //   nu_bin_fill   (cell, pixel) pairs stored bin by bin (one global reservation per (block,
 //                 bin), ranks within the block from shared memory).  Extra blocks clear the
 //                 grid rows that some bin reaches, and mark them;
-//   nu_sort       a block counting-sorts up to 8192 pixels of a bin by cell (and quarter of a
+//   nu_sort       (frames where it pays) a block counting-sorts up to 8192 pixels of a bin by cell (and quarter of a
 //                 cell along x);
-//   nu_spread     persistent CTAs take (1024 sorted pixels, channel) units in turn; a warp takes
+//   nu_spread     persistent CTAs take (1024 or 512 pixels, channel) units in turn; a warp takes
 //                 one pixel at a time, lane k holding tap k of its w x w taps.  Successive
 //                 pixels of one cell are summed in registers and leave for a shared-memory
 //                 tile with a halo when the cell changes, as fixed-point integers (each term
@@ -67,10 +67,12 @@ constexpr int kNWMin = 4, kNWMax = 8;       // kernel widths in cells (the defau
 constexpr float kNBetaPerW = 2.30f;         // ES shape beta = 2.30 w for an oversampling of 2
 constexpr int kNTile = 32;                  // grid cells per tile side
 constexpr int kNQuad = 128;                 // midpoint nodes for Psi
-constexpr int kSpreadChunk = 1024;          // sorted pixels per spreading work item
+constexpr int kSpreadChunk = 1024;          // pixels per spreading work item, or half as many
 constexpr int kSortChunk = 8192;            // pixels a block sorts (whole spreading items)
 constexpr int kSortThreads = 1024;
-constexpr int kSortFrom = 12288;            // pixels of the frames that are sorted (see launch_nufft)
+constexpr int kSortFrom = 12288;            // frames that are sorted have this many pixels and
+constexpr int64_t kSortWork = 400000;       // this many (channel, pixel) pairs (see nufft_geometry)
+constexpr int64_t kLongWork = 300000;       // pairs from which spreading items are kSpreadChunk long
 constexpr int kSub = 4;                     // sort keys per cell: the quarter along x
 static_assert(kSortChunk % kSpreadChunk == 0 && kSortChunk % kSortThreads == 0, "sorting items");
 constexpr int kBinThreads = 256;            // binning blocks: one group, kBinItems pixels
@@ -221,7 +223,7 @@ struct NuItems {
 // Exclusive scan of n bin counts by one block into `off` and `cursor`, and of their chunk
 // counts into the work-item tables.  The counts were added by other blocks' atomics, so
 // they are read from L2.
-__device__ void scan_bins(const int* __restrict__ count, int n, const NuItems& it) {
+__device__ void scan_bins(const int* __restrict__ count, int n, int chunk, const NuItems& it) {
   __shared__ int wsum[32], wcsum[32], n_sort;
   const int nt = blockDim.x, nw = nt >> 5;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -243,7 +245,7 @@ __device__ void scan_bins(const int* __restrict__ count, int n, const NuItems& i
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
       s += kk[j];
-      c += (kk[j] + kSpreadChunk - 1) / kSpreadChunk;
+      c += (kk[j] + chunk - 1) / chunk;
       if (b == b0) first[j] = kk[j];
     }
   }
@@ -284,7 +286,7 @@ __device__ void scan_bins(const int* __restrict__ count, int n, const NuItems& i
       if (b + j >= b1) break;
       off[b + j] = run;
       cursor[b + j] = run;
-      for (int q = 0; q < kk[j]; q += kSpreadChunk, ++crun) {
+      for (int q = 0; q < kk[j]; q += chunk, ++crun) {
         item_bin[crun] = b + j;
         item_first[crun] = run + q;
       }
@@ -337,7 +339,7 @@ __global__ void __launch_bounds__(kBinThreads) nu_bin_count(const FrameIO* __res
   __syncthreads();
   if (ticket != (int)(gridDim.x * g.groups) - 1) return;
   __threadfence();
-  scan_bins(count, nbins, it);
+  scan_bins(count, nbins, g.chunk, it);
 }
 
 // The first groups x fill_blocks blocks store the pixels; each of the groups x G_x blocks after
@@ -592,7 +594,7 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadBlocksPerSm) nu_spread(
     if (v >= g.V) continue;
     const int ty = (bin % nb) % g.nty, tx = (bin % nb) / g.nty;
     const int r_begin = item_first[item];
-    const int n = min(off[bin + 1] - r_begin, kSpreadChunk);
+    const int n = min(off[bin + 1] - r_begin, g.chunk);
     for (int i = threadIdx.x; i < WORDS; i += blockDim.x)  // 4 arrays of WORDS / 4 16-byte words
       reinterpret_cast<uint4*>(smem_sp)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
@@ -958,7 +960,9 @@ size_t nu_max_items(const NuGeo& g, int chunk) {
 
 NuScratch nufft_layout(const NuGeo& g, const FftPlan& plx, const FftPlan& ply, char* base) {
   const size_t nbins = (size_t)g.groups * g.ntx * g.nty;
-  const size_t max_items = nu_max_items(g, kSpreadChunk), max_sorts = nu_max_items(g, kSortChunk);
+  // for the shorter items: a batch's slots hold the largest frame, and its smaller ones may
+  // have more items
+  const size_t max_items = nu_max_items(g, kSpreadChunk / 2), max_sorts = nu_max_items(g, kSortChunk);
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   NuScratch sc{};
   size_t o = 0;
@@ -1010,10 +1014,18 @@ NuGeo nufft_geometry(const Consts& k, int64_t P) {
   const double cells = fabs(k.k_da) * g.Gx;
   g.gch = cells * (k.V - 1) <= 0.9 ? k.V : std::max(1, (int)(0.9 / cells) + 1);
   g.groups = (k.V + g.gch - 1) / g.gch;
+  // A frame is sorted where its channels repay the sort (a launch and some 5 us), and takes
+  // the longer spreading items where there are units enough for every CTA.  Time of a frame
+  // with 1024 pixels sorted / 1024 / 512 an item (V x pixels): 12 x 262,144 204 / 228 / 240 us,
+  // 12 x 65,536 90 / 90 / 95, 24 x 16,384 66 / 66 / 66, 12 x 28,145 64 / 60 / 62, 4 x 65,536
+  // 70 / 66 / 62, 1 x 65,536 62 / 56 / 50, 2 x 14,619 56 / 50 / 44
+  const int64_t work = (int64_t)k.V * g.P;
+  g.sorted = g.P >= kSortFrom && work >= kSortWork;
+  g.chunk = work >= kLongWork ? kSpreadChunk : kSpreadChunk / 2;
   return g;
 }
 
-int nufft_kernels(int64_t P) { return P >= kSortFrom ? 6 : 5; }
+int nufft_kernels(const Consts& k, int64_t P) { return nufft_geometry(k, P).sorted ? 6 : 5; }
 
 bool nufft_supported(const Consts& k) {
   // FFT lengths up to 4096 in one CTA's shared memory, at least 8 cells per axis, and a
@@ -1053,8 +1065,7 @@ cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int o
   tb.inv_y = sc.inv_y;
   tb.twx = sc.tw_x;
   tb.twy = sc.tw_y;
-  // few pixels share a cell in a small frame: its sort (a launch and some 5 us) gains nothing
-  const bool sorted = g.P >= kSortFrom;
+  const bool sorted = g.sorted;
   const NuItems it{sc.off, sc.cursor, sc.items, sc.item_bin, sc.item_first, sc.sort_bin, sc.sort_first};
   e = launch_dependent(nu_bin_count, dim3(bgrid.x, bgrid.y + 1), dim3(kBinThreads), (size_t)(4 * nb), st, frame, g,
                        sc.count, tb, it);
@@ -1083,7 +1094,7 @@ cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int o
   if (e == cudaSuccess && spread_begin) e = cudaEventRecord(spread_begin, st);
   if (e == cudaSuccess)
     e = launch_dependent(spread,
-                         dim3((unsigned)std::min<size_t>(nu_max_items(g, kSpreadChunk) * g.gch,
+                         dim3((unsigned)std::min<size_t>(nu_max_items(g, g.chunk) * g.gch,
                                                          (size_t)kSpreadBlocksPerSm * num_sms)),
                          dim3(kSpreadThreads), spread_smem, st, frame, g, (const int*)sc.off, (const int*)sc.items,
                          (const int*)sc.item_bin, (const int*)sc.item_first, (const uint32_t*)sc.ord, sc.grid);

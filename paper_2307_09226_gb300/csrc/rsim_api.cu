@@ -322,7 +322,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     // split reduction (1 when the partial buffer is used)
     const bool tensor = tensor_tier(tier);
     if (tier == RSIM_TIER_NUFFT) {
-      for (int f = 0; f < F; ++f) ctx->prof_kernels += nufft_kernels(frames[f].P);
+      for (int f = 0; f < F; ++f) ctx->prof_kernels += nufft_kernels(k, frames[f].P);
     } else {
       ctx->prof_kernels += (tensor ? 1 + (mp > 0 ? 1 : 0) + (F > 1 ? 1 : 0) : 1) + (use_partial ? 1 : 0);
     }
@@ -331,9 +331,11 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
   cudaError_t e = cudaSuccess;
   // the tensor tiers' operand builder computes the fast-time and channel phases
   const bool defer = tensor_tier(tier);
-  // NUFFT batches: every frame's compaction goes to the frame's own stream (below), where its
-  // FP64 work runs beside other frames' spreading
-  const bool per_frame = tier == RSIM_TIER_NUFFT && nufft_slots(F) > 1;
+  // NUFFT batches of large frames: every frame's compaction goes to the frame's own stream
+  // (below), where its FP64 work runs beside other frames' spreading (64 walking frames -5%).
+  // Small frames wait for the host's launches, of which that would be more (20 frames of V = 2
+  // and 65,536 pixels 381 -> 408 us)
+  const bool per_frame = tier == RSIM_TIER_NUFFT && nufft_slots(F) > 1 && nufft_geometry(k, mp).sorted;
   if (!per_frame) {
     NvtxRange r(defer ? "compaction + slow-time phases" : "compaction + FP64 phases");
     int launched = 0;

@@ -128,13 +128,15 @@ struct NuGeo {
   int ntx, nty;   // tiles per axis
   int sx, sy;     // centring shifts Ns / 2, L / 2
   int64_t P;      // pixel bound (items per channel)
+  int chunk;      // sorted pixels per spreading work item
+  bool sorted;    // the bins are sorted by cell
   int W;          // gridding kernel width (cells)
   float beta;     // its shape parameter, 2.30 W
   int gch, groups;  // channels sorted together, and such groups
 };
 // Kernels launch_nufft starts for a frame of P pixels (binning with the tables and the scan,
-// fill, sort in larger frames, spreading, two FFT passes).
-int nufft_kernels(int64_t P);
+// fill, sort in larger frames (see nufft_geometry), spreading, two FFT passes).
+int nufft_kernels(const Consts& k, int64_t P);
 NuGeo nufft_geometry(const Consts& k, int64_t P);
 bool nufft_supported(const Consts& k);
 size_t nufft_scratch_bytes(const Consts& k, int64_t P);

@@ -152,3 +152,25 @@ def test_channel_groups_and_sorting(ctx, d_rx_lambda, groups, n_az, n_el, w):
     assert ctx.sync_status() == _abi.OK
     assert np.array_equal(first, again)
     assert oracle.rel_l2(first, nu.cube_nufft(radar, px, w=w)) <= 5e-6
+
+
+@pytest.mark.parametrize("d_rx_lambda", [0.5, 8.0])
+def test_channel_groups_of_a_large_frame(ctx, d_rx_lambda):
+    """Eight channels of 51,200 pixels: the sorted frames and the longer spreading items."""
+    test_channel_groups_and_sorting(ctx, d_rx_lambda, "", 256, 200, 7)
+
+
+def test_batch_of_every_size_class_bitwise(ctx):
+    """Sorted, unsorted and short-item frames in one batch, the largest last: every frame's bits
+    are its own, whichever slot of scratch it finds."""
+    radar = synth.Radar(M=2, N=4, Ns=64, L=32)
+    sizes = [(64, 64), (193, 194), (193, 195), (256, 200), (30, 20)] * 2 + [(256, 201)]
+    pxs = [device.upload(synth.random_frame(radar, a, e, seed=70 + i, mask_frac=0.2)) for i, (a, e) in enumerate(sizes)]
+    alone = [ctx.synth(radar, px, "nufft").cpu().numpy() for px in pxs]
+    batch = [c.cpu().numpy() for c in ctx.synth_batch(radar, pxs, "nufft")]
+    small = [c.cpu().numpy() for c in ctx.synth_batch(radar, pxs[:3], "nufft")]
+    assert ctx.sync_status() == _abi.OK
+    for a, b in zip(alone, batch):
+        assert np.array_equal(a, b)
+    for a, b in zip(alone, small):
+        assert np.array_equal(a, b)
