@@ -13,8 +13,8 @@
 // clear of is skipped after an FP32 test.
 // Per call, before and after: 600 x 600 pixels, 100 primitives 165 -> 75 us (FP32), 4423 ->
 // 692 us (FP64); 512 x 512, 20 primitives 39 -> 21 us; 256 x 256, 12 primitives 25 -> 20 us
-// (FP32, bound by the host's call), 134 -> 49 us (FP64); the same bits.  The primitives are staged in shared memory in
-// tiles of 64, each thread of a block deriving one primitive's constants (unit normal,
+// (FP32, bound by the host's call), 134 -> 49 us (FP64); the same bits.  The primitives are
+// staged in shared memory in tiles of 64, each thread of a block deriving one primitive's constants (unit normal,
 // the dual basis of a plane, the unit-sphere frame of an ellipsoid, the constant terms
 // of the quadratics) in the compute precision T = float for FP32 buffers, double for
 // FP64 buffers.  A plane's in-plane coordinates use the dual basis b* = (c x n) / |n|^2,
@@ -41,8 +41,11 @@ constexpr int kRcTile = 64;  // primitives per shared-memory tile
 constexpr int kRcThreads = 256;
 constexpr int kRcByValue = 24;  // 3,840 bytes of kernel arguments
 
+// N primitives in the kernel's arguments; more than kRcByValue come from device memory, and
+// their launch carries one (unread) instead of 3,840 bytes.
+template <int N>
 struct RcArgs {
-  rsim_primitive p[kRcByValue];
+  rsim_primitive p[N];
 };
 
 template <typename T>
@@ -276,16 +279,16 @@ __device__ __forceinline__ void sin_cos(T x, T* s, T* c) {
 }
 
 // `prims`: the primitives in device memory, or NULL when they are in `byval`.
-template <typename T>
+template <typename T, int N>
 __global__ void __launch_bounds__(kRcThreads)
-rc_render(const __grid_constant__ RcArgs byval, const rsim_primitive* __restrict__ prims, int n_prims, int n_az,
+rc_render(const __grid_constant__ RcArgs<N> byval, const rsim_primitive* __restrict__ prims, int n_prims, int n_az,
           int n_el, int tw, int tiles_x, double az0, double az1, double el0, double el1, int falloff, T* __restrict__ R,
           T* __restrict__ sre, T* __restrict__ sim, T* __restrict__ az_out, T* __restrict__ el_out,
           T* __restrict__ vel) {
   __shared__ RcPrim<T> tile[kRcTile];
   // the tile's angles, tw columns then th rows, their sines and cosines (tw + th <= 257)
   __shared__ T ang[kRcThreads + 1], sn[kRcThreads + 1], cs[kRcThreads + 1];
-  __shared__ __align__(16) rsim_primitive raw[kRcByValue];
+  __shared__ __align__(16) rsim_primitive raw[N];
   const int th = kRcThreads / tw;
   const int i0 = (int)(blockIdx.x % (unsigned)tiles_x) * tw, j0 = (int)(blockIdx.x / (unsigned)tiles_x) * th;
   const int tid = threadIdx.x, tx = tid % tw, ty = tid / tw;
@@ -299,7 +302,7 @@ rc_render(const __grid_constant__ RcArgs byval, const rsim_primitive* __restrict
     ang[q] = x;
     sin_cos(x, &sn[q], &cs[q]);
   }
-  if (!prims) {
+  if (N > 1 && !prims) {
     const uint32_t* from = reinterpret_cast<const uint32_t*>(&byval);
     uint32_t* to = reinterpret_cast<uint32_t*>(raw);
     for (int w = tid; w < n_prims * (int)(sizeof(rsim_primitive) / 4); w += kRcThreads) to[w] = from[w];
@@ -400,16 +403,16 @@ int rc_tile_width(int n_az) {
   return w;
 }
 
-template <typename T>
+template <typename T, int N>
 cudaError_t launch_raycast(const rsim_primitive* host, const rsim_primitive* dev, int n, const rsim_camera& cam,
                            const rsim_pixel_out& out, cudaStream_t st) {
-  RcArgs byval;
+  RcArgs<N> byval;
   if (!dev)
     for (int i = 0; i < n; ++i) byval.p[i] = host[i];
   const int w = rc_tile_width(cam.n_az), h = kRcThreads / w;
   const int tiles_x = (cam.n_az + w - 1) / w;
   const int64_t blocks = (int64_t)tiles_x * ((cam.n_el + h - 1) / h);
-  return launch_dependent(rc_render<T>, dim3((unsigned)blocks), dim3(kRcThreads), 0, st, byval, dev, n, cam.n_az,
+  return launch_dependent(rc_render<T, N>, dim3((unsigned)blocks), dim3(kRcThreads), 0, st, byval, dev, n, cam.n_az,
                           cam.n_el, w, tiles_x, cam.az_min, cam.az_max, cam.el_min, cam.el_max,
                           (cam.flags & RSIM_RC_NO_FALLOFF) ? 0 : 1, (T*)out.range, (T*)out.sigma_re,
                           (T*)out.sigma_im, (T*)out.az, (T*)out.el, (T*)out.vel);
@@ -451,10 +454,9 @@ extern "C" rsim_status rsim_raycast(rsim_ctx* ctx, const rsim_camera* cam, const
     if (e != cudaSuccess) return cuda_fail(e, "upload of the primitives");
     raw = (const rsim_primitive*)ctx->ws;
   }
-  if (out->dtype == RSIM_F32)
-    e = launch_raycast<float>(prims, raw, n_prims, *cam, *out, st);
-  else
-    e = launch_raycast<double>(prims, raw, n_prims, *cam, *out, st);
+  auto launch = out->dtype == RSIM_F32 ? (raw ? launch_raycast<float, 1> : launch_raycast<float, kRcByValue>)
+                                       : (raw ? launch_raycast<double, 1> : launch_raycast<double, kRcByValue>);
+  e = launch(prims, raw, n_prims, *cam, *out, st);
   if (e != cudaSuccess) return cuda_fail(e, "ray-caster kernels");
   return RSIM_OK;
 }
