@@ -87,13 +87,14 @@ int default_splits(int tier, int V, int Ns, int L, int tile_n, int64_t P, int nu
     return (int)bs;
   }
   // tensor tiers: one persistent CTA (or half a pair) per SM takes equal units in turn; pick
-  // the split count whose unit count fills whole rounds best, with a cost per split for the
-  // partial sums it adds: a hundredth of the contraction (plain BF16, V = 20, N_s = 335,
-  // L = 124, 5643 pixels: 17 splits at 0.003 and 85 us, 8 and 62 us at 0.01 with the longer
-  // rings, which alone give 4 to 10%).  The split tiers keep 0.003: fewer splits would lengthen their accumulation groups,
-  // whose rounding toward zero is most of their error
-  const int slots = std::max(tier == kTierFp32Tensor ? num_sms / 2 : num_sms, 1);
-  const double per_split = split_tier(tier) ? 0.003 : 0.01;
+  // the split count whose unit count fills whole rounds best, with a small cost per split for
+  // the partial sums it adds.  That cost has to stay below the SMs' share of one unit, or a
+  // frame of one tile is not split at all (0.01 against 1 / 152: one CTA works, 8 to 50 times
+  // as long).  On pairs a unit's share is 1 / 76, and 0.01 is the better line there (64 frames
+  // of 12 tiles: 6 splits instead of 19, 10.40 ms against 11.21)
+  const bool on_pairs = tier == kTierFp32Tensor;
+  const int slots = std::max(on_pairs ? num_sms / 2 : num_sms, 1);
+  const double per_split = std::min(on_pairs ? 0.01 : 0.003, 0.75 / slots);
   double best = -1.0;
   int bs = 1;
   for (int s = 1; s <= smax; ++s) {

@@ -135,3 +135,12 @@ def test_odd_column_tiles_take_no_padding(env, tier, bar):
     got = cube.cpu().numpy()
     assert np.array_equal(got, ctx.synth(radar, d, tier).cpu().numpy())
     assert oracle.rel_l2(got, oracle.cube_separable(radar, px)) <= bar
+
+
+@pytest.mark.parametrize("tier", ["fp32", "bf16", "fp16", "split_fp16", "split_bf16"])
+@pytest.mark.parametrize("V,Ns,L", [(1, 64, 16), (1, 128, 128), (2, 96, 40), (3, 128, 64)])
+def test_frames_of_few_tiles_are_split(env, tier, V, Ns, L):
+    """One to three tiles of 65,536 pixels: enough splits to give most SMs a unit."""
+    torch, _abi, device, ctx = env
+    plan = _abi.rsim_get_plan(ctx.h, Radar(M=V, N=1, Ns=Ns, L=L), 65536, _abi.TIERS[tier])
+    assert plan.splits >= 32
