@@ -452,10 +452,11 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
             const bool two = (l + 1 < k.L);
             const int64_t o = d.gr * k.L + l;
             if (out_dtype == RSIM_C128) {
+              // scaled in FP64: the sums of strengths near FP32's largest number pass it
+              const double os = (double)oscale.x * oscale.y;
               double2* cd = reinterpret_cast<double2*>(dfr.cube);
-              cd[o] = make_double2((double)(a0 * oscale.x * oscale.y), (double)(b0 * oscale.x * oscale.y));
-              if (two)
-                cd[o + 1] = make_double2((double)(a1 * oscale.x * oscale.y), (double)(b1 * oscale.x * oscale.y));
+              cd[o] = make_double2(a0 * os, b0 * os);
+              if (two) cd[o + 1] = make_double2(a1 * os, b1 * os);
             } else {
               float2* cf = reinterpret_cast<float2*>(dfr.cube);
               cf[o] = make_float2(a0 * oscale.x * oscale.y, b0 * oscale.x * oscale.y);

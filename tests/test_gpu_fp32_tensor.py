@@ -144,3 +144,22 @@ def test_frames_of_few_tiles_are_split(env, tier, V, Ns, L):
     torch, _abi, device, ctx = env
     plan = _abi.rsim_get_plan(ctx.h, Radar(M=V, N=1, Ns=Ns, L=L), 65536, _abi.TIERS[tier])
     assert plan.splits >= 32
+
+
+@pytest.mark.parametrize("tier", ["split_fp16", "fp16"])
+def test_complex128_cubes_beyond_the_range_of_fp32(env, tier):
+    """Eight pixels of 1.5e38 at one place: their sum passes FP32's largest number, but a
+    complex128 cube holds it when the tile is written directly (one split, one accumulation
+    group)."""
+    torch, _abi, device, ctx = env
+    f = synth.parity_frame(seed=94, M=1, N=2, Ns=64, L=24, n_az=8, n_el=1, mask_frac=0.0)
+    px = f.pixels
+    for a in (px.range, px.az, px.el, px.vel):
+        a[:] = a[0]
+    px.sigma_re[:], px.sigma_im[:] = np.float32(1.5e38), 0.0
+    assert _abi.rsim_get_plan(ctx.h, f.radar, px.P, _abi.TIERS[tier]).splits == 1
+    ref = oracle.cube_separable(f.radar, px)
+    assert np.abs(ref.real).max() > 3.5e38
+    got = ctx.synth(f.radar, device.upload(f), tier, out_dtype="complex128").cpu().numpy()
+    assert ctx.sync_status() == _abi.OK and np.all(np.isfinite(got))
+    assert oracle.rel_l2(got / 1e38, ref / 1e38) <= (2e-5 if tier == "split_fp16" else 1e-2)
