@@ -49,6 +49,16 @@ constexpr int kRegsLaunch = 96, kRegsA = 64, kRegsSum = 152, kRegsRest = 48;
 static_assert(32 * (kAWarps * kRegsA + kSumWarps * kRegsSum + 4 * kRegsRest) <= kThreads * kRegsLaunch,
               "the warpgroups' registers fit the launch's");
 constexpr uint32_t kFineLong = 20000 / kChunkPx;  // chunks of a frame from which groups are long
+// The accumulator rounds toward zero, so a group's sum comes out short by about half a unit in
+// the last place of each addition at its size: by 0.8 x 2^-23 of itself in groups of one chunk
+// (four additions of A_hi B_hi at a quarter to all of the size) and by 2.4 x 2^-23 in groups of
+// two (twelve more).  Measured against the CUDA-core sum, which has the same phasors, over 128 to
+// 262,144 pixels and equal, log-normal and 1/R^2 strengths of one and of random phase: 0.9 to
+// 1.0e-7 and 2.6 to 2.9e-7.  A unit's sums are lengthened by it.  Error with strengths of one
+// phase (rendered scenes; the CUDA-core sum's in brackets) without and with it: 2,048 pixels
+// 2.5 -> 1.9e-7 (2.5e-7), 40,000 4.2 -> 1.8e-7 (1.7e-7), 262,144 4.1 -> 1.7e-7 (1.9e-7); of
+// random phase 3.2 -> 2.6e-7 (4.1e-7), 5.2 -> 3.4e-7 (5.8e-7) and 5.6 -> 3.8e-7 (1.4e-6).
+constexpr float kShort1 = 0.8f * 0x1p-23f, kShort2 = 2.4f * 0x1p-23f;
 constexpr int kPartBytes = 128 * 128;      // one 16-bit part of a stage's A (128 rows) or of its half of B
 constexpr int kAccCols = 256;              // columns of one accumulator (N <= 256 FP32)
 constexpr int kTmemCols = 512;             // two accumulators
@@ -170,7 +180,8 @@ __device__ __forceinline__ Unit decode(const Geo& g, const FrameIO* frames, cons
   x.nt = r % g.ntiles;
   x.s = r / g.ntiles;
   const uint32_t nch = (uint32_t)((frames[x.f].meta[0] + kChunkPx - 1) / kChunkPx);
-  // one chunk a group (error 3.3e-7 to 3.7e-7), two for long sums (5.6e-7)
+  // one chunk a group (error 2.6 to 3.0e-7 with equal strengths), two for long sums (3.0 to
+  // 3.8e-7; in groups of one the frame of 46,000 valid pixels takes 327 us instead of 275)
   x.group = nch < kFineLong ? 1 : 2;
   x.c0 = nch * (uint32_t)x.s / (uint32_t)g.splits;
   x.c1 = nch * (uint32_t)(x.s + 1) / (uint32_t)g.splits;
@@ -406,6 +417,15 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int out
         if (lane == 0) mbar_arrive_at(&sh->acc_empty[gi & 1u], 0);
       }
       if (!alive) break;
+      // 2 (chunks - ngr) of the chunks were summed in groups of two
+      const float lost = kShort1 + (kShort2 - kShort1) * (2.f * (float)(chunks - min(ngr, chunks)) / (float)max(chunks, 1u));
+#pragma unroll
+      for (int b = 0; b < kBlocks; ++b)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          sre[b][i] = fmaf(sre[b][i], lost, sre[b][i]);
+          sim[b][i] = fmaf(sim[b][i], lost, sim[b][i]);
+        }
       const int mt = xs->mt, nt = xs->nt;
       const FrameIO& fr = frames[xs->f];
       const int64_t gr = (int64_t)mt * 128 + r;
