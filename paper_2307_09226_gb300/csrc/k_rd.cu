@@ -37,6 +37,7 @@ namespace {
 constexpr int kRdCols = 8;          // Doppler columns per CTA: a 64-byte run of every row
 constexpr int kRdThreads = 256;     // row kernel, and the column kernel of many frames
 constexpr int kRdThreadsMax = 512;  // column kernel when few frames leave SMs idle
+static_assert(kRdThreadsMax == 2 * kRdThreads, "a helper for every group of the smaller block");
 constexpr int kRdByValue = 64;      // cube pointers passed in the kernel's arguments
 
 // FFT of N = 2^k points, 2 <= N <= 1024: a thread holds PER values and T threads share a
@@ -56,6 +57,9 @@ struct FftShape {
   static constexpr int pitch(int want) { return N + N / 16 + ((want - (N + N / 16)) % 16 + 16) % 16; }
   static constexpr int kRowPitch = pitch(T < 16 ? T : 0);
   static constexpr int kColPitch = pitch(2);
+  // Floats of a column group: its transforms' buffers, or its sums if it has none.
+  static constexpr int kGroupFloats = R2 > 1 ? 16 * kColPitch : 8 * N;
+  static_assert(kGroupFloats >= 8 * N, "the sums fit over the buffers");
   // Index in the transform of the i-th value a thread holds after the last pass.
   __device__ static __forceinline__ int pos(int i, int t) { return t + (i / RL) * T + (i % RL) * (N / RL); }
 };
@@ -175,9 +179,12 @@ fft_rows(const __grid_constant__ CubePtrs byval, const float2* const* __restrict
 
 // Columns: the threads of a CTA form groups of T x 8, each taking every (number of
 // groups)-th channel's 8 columns; a group sums |X|^2 over its channels in registers and the
-// groups' sums are added in group order.  Frames run from the last to the first: the rows
-// written last are the ones still in L2.
-template <int Ns>
+// groups' sums are added in group order.  In the larger block (kPaired) the second half of the
+// groups helps the first: it hands its |X|^2 over in shared memory, and the sums are those of the
+// smaller block, so that a map's bits do not depend on the number of frames (with a run-time
+// switch in one kernel the smaller block lost 1 to 3%).  Frames run from the last to
+// the first: the rows written last are the ones still in L2.
+template <int Ns, bool kPaired>
 __global__ void __launch_bounds__(kRdThreadsMax)
 fft_cols(const float2* __restrict__ tmp, float* __restrict__ power, int F, int V, int L) {
   using S = FftShape<Ns>;
@@ -189,9 +196,12 @@ fft_cols(const float2* __restrict__ tmp, float* __restrict__ power, int F, int V
   __syncthreads();
   const int c = threadIdx.x % kRdCols, t = (threadIdx.x / kRdCols) % S::T;
   const int g = threadIdx.x / kGroup, groups = blockDim.x / kGroup;
+  const int mains = kPaired ? groups / 2 : groups;
   float2* bufs = rd_smem + S::kTw2 + S::kTw3;
   float2* x = bufs + (g * kRdCols + c) * S::kColPitch;
   float* red = reinterpret_cast<float*>(bufs);  // [group][PER][T x 8], over the transform buffers
+  // the helpers' values of this round and of the next, [2][group][PER][T x 8], behind the buffers
+  [[maybe_unused]] float* handed = red + groups * S::kGroupFloats + (g % mains) * S::PER * kGroup + threadIdx.x % kGroup;
   auto sync = [g] {
     if (kGroup <= 32)
       __syncwarp();
@@ -203,6 +213,7 @@ fft_cols(const float2* __restrict__ tmp, float* __restrict__ power, int F, int V
     float pw[S::PER];
 #pragma unroll
     for (int i = 0; i < S::PER; ++i) pw[i] = 0.f;
+    [[maybe_unused]] int at = 0;  // the round's half of the values handed over
     // every group runs the same number of rounds: for short transforms groups share a warp
     for (int v0 = 0; v0 < V; v0 += groups) {
       const int v = v0 + g;
@@ -214,16 +225,30 @@ fft_cols(const float2* __restrict__ tmp, float* __restrict__ power, int F, int V
         a[j] = live ? src[(int64_t)(t + j * S::T) * L] : make_float2(0.f, 0.f);
       rd_fft<Ns>(a, x, t, tw, sync);
 #pragma unroll
-      for (int i = 0; i < S::PER; ++i) pw[i] += a[i].x * a[i].x + a[i].y * a[i].y;
+      for (int i = 0; i < S::PER; ++i) pw[i] += fmaf(a[i].x, a[i].x, a[i].y * a[i].y);
+      if constexpr (kPaired) {
+        if (g >= mains) {
+#pragma unroll
+          for (int i = 0; i < S::PER; ++i) handed[at + i * kGroup] = pw[i], pw[i] = 0.f;
+        }
+        __syncthreads();  // also between a round's reads and the stores of the next but one
+        if (g < mains) {
+#pragma unroll
+          for (int i = 0; i < S::PER; ++i) pw[i] += handed[at + i * kGroup];
+        }
+        at = mains * S::PER * kGroup - at;
+      }
     }
     __syncthreads();
+    if (!kPaired || g < mains) {
 #pragma unroll
-    for (int i = 0; i < S::PER; ++i) red[(g * S::PER + i) * kGroup + threadIdx.x % kGroup] = pw[i];
+      for (int i = 0; i < S::PER; ++i) red[(g * S::PER + i) * kGroup + threadIdx.x % kGroup] = pw[i];
+    }
     __syncthreads();
     // the block size is a multiple of 8, so an output's column is this thread's own
     for (int o = threadIdx.x; o < S::PER * kGroup; o += blockDim.x) {
       float sum = red[o];
-      for (int h = 1; h < groups; ++h) sum += red[h * S::PER * kGroup + o];
+      for (int h = 1; h < mains; ++h) sum += red[h * S::PER * kGroup + o];
       const int i = o / kGroup, to = (o % kGroup) / kRdCols;
       if (d < L) power[((int64_t)f * Ns + S::pos(i, to)) * L + d] = sum;
     }
@@ -309,9 +334,9 @@ struct RowKernel {
   int rows, smem;  // rows per pass of a block
 };
 struct ColKernel {
-  ColFn fn;
-  int group, fixed, per_group;  // threads of a group; shared memory: twiddles, then per group
-};
+  ColFn fn, paired;
+  int group, fixed, per_group, handed;  // threads of a group; shared memory: twiddles, then per
+};                                      // group, and what a helper hands over in a round
 
 template <int N>
 RowKernel row_kernel() {
@@ -322,8 +347,8 @@ RowKernel row_kernel() {
 template <int N>
 ColKernel col_kernel() {
   using S = FftShape<N>;
-  const int buf = S::R2 > 1 ? 8 * kRdCols * S::kColPitch : 0, sums = 4 * S::PER * S::T * kRdCols;
-  return {fft_cols<N>, S::T * kRdCols, 8 * (S::kTw2 + S::kTw3), std::max(buf, sums)};
+  static_assert(kRdCols == 8, "kGroupFloats");
+  return {fft_cols<N, false>, fft_cols<N, (S::T * kRdCols < kRdThreadsMax)>, S::T * kRdCols, 8 * (S::kTw2 + S::kTw3), 4 * S::kGroupFloats, 4 * kRdCols * N};
 }
 
 template <class R, template <int> class Pick>
@@ -375,10 +400,13 @@ cudaError_t launch_range_doppler(const float2* const* cubes, const float2* const
   // of a frame at a time)
   const int cx = (L + kRdCols - 1) / kRdCols;
   const int threads = std::max(ck.group, (int64_t)cx * F >= 2ll * num_sms ? kRdThreads : kRdThreadsMax);
-  const int smem = ck.fixed + (threads / ck.group) * ck.per_group;
-  e = cudaFuncSetAttribute(ck.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // a helper for every second group, two rounds of values each
+  const bool paired = threads > kRdThreads && ck.group < kRdThreadsMax;
+  const int smem = ck.fixed + (threads / ck.group) * (ck.per_group + (paired ? ck.handed : 0));
+  const ColFn cols = paired ? ck.paired : ck.fn;
+  e = cudaFuncSetAttribute(cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  e = launch_dependent(ck.fn, dim3(cx, fy), dim3(threads), (size_t)smem, st, (const float2*)tmp, power, F, V, L);
+  e = launch_dependent(cols, dim3(cx, fy), dim3(threads), (size_t)smem, st, (const float2*)tmp, power, F, V, L);
   if (e != cudaSuccess) return e;
   return launch_dependent(rd_argmax, dim3(F), dim3(kArgThreads), 0, st, (const float*)power, Ns, L, skip_static,
                           v_per_bin, v_est, peak);

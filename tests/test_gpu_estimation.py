@@ -128,3 +128,18 @@ def test_every_transform_length(env, Ns, L, V, F):
             m[:, :, 0] = -1.0
         first = m.reshape(F, -1).argmax(1)
         assert np.array_equal(peak.cpu().numpy(), np.stack([first // L, first % L], axis=1))
+
+
+@pytest.mark.parametrize("Ns,L,V", [(2, 4, 70), (16, 64, 67), (32, 64, 40), (128, 64, 13), (256, 128, 12), (512, 32, 5),
+                                    (1024, 16, 3)])
+def test_a_map_does_not_depend_on_the_other_cubes(env, Ns, L, V):
+    """The map of a cube alone and among as many as fill the GPU: the same bits."""
+    torch, _abi, device, ctx = env
+    radar = Radar(M=V, N=1, Ns=Ns, L=L)
+    g = torch.Generator(device="cpu").manual_seed(Ns + L + V)
+    cubes = [torch.randn((V, Ns, L), dtype=torch.complex64, generator=g).cuda() for _ in range(3)]
+    F = max(3, 320 * 8 // L + 1)  # two blocks of 8 columns an SM and more
+    many, _, _ = _rd(env, radar, [cubes[i % 3] for i in range(F)])
+    for i in range(3):
+        alone, _, _ = _rd(env, radar, [cubes[i]])
+        assert np.array_equal(alone[0], many[i]) and np.array_equal(alone[0], many[F - 3 + (i - (F - 3)) % 3])
