@@ -297,7 +297,7 @@ rc_render(const __grid_constant__ RcArgs<N> byval, const rsim_primitive* __restr
   for (int q = (tid + kRcThreads - 32) % kRcThreads; q < tw + th; q += kRcThreads) {
     const bool is_az = q < tw;
     const double lo = is_az ? az0 : el0, hi = is_az ? az1 : el1;
-    const int at = is_az ? i0 + q : j0 + q - tw, n = is_az ? n_az : n_el;
+    const int at = is_az ? i0 + q : j0 + (q - tw), n = is_az ? n_az : n_el;
     const T x = (T)__dadd_rn(lo, __ddiv_rn(__dmul_rn((double)at + 0.5, __dsub_rn(hi, lo)), (double)n));
     ang[q] = x;
     sin_cos(x, &sn[q], &cs[q]);
@@ -403,19 +403,26 @@ int rc_tile_width(int n_az) {
   return w;
 }
 
+// Tiles along the columns, and in all: 64-bit, a side may be as long as an int holds.
+int64_t rc_tiles_x(const rsim_camera& cam) {
+  const int64_t w = rc_tile_width(cam.n_az);
+  return (cam.n_az + w - 1) / w;
+}
+int64_t rc_tiles(const rsim_camera& cam) {
+  const int64_t h = kRcThreads / rc_tile_width(cam.n_az);
+  return rc_tiles_x(cam) * ((cam.n_el + h - 1) / h);
+}
+
 template <typename T, int N>
 cudaError_t launch_raycast(const rsim_primitive* host, const rsim_primitive* dev, int n, const rsim_camera& cam,
                            const rsim_pixel_out& out, cudaStream_t st) {
   RcArgs<N> byval;
   if (!dev)
     for (int i = 0; i < n; ++i) byval.p[i] = host[i];
-  const int w = rc_tile_width(cam.n_az), h = kRcThreads / w;
-  const int tiles_x = (cam.n_az + w - 1) / w;
-  const int64_t blocks = (int64_t)tiles_x * ((cam.n_el + h - 1) / h);
-  return launch_dependent(rc_render<T, N>, dim3((unsigned)blocks), dim3(kRcThreads), 0, st, byval, dev, n, cam.n_az,
-                          cam.n_el, w, tiles_x, cam.az_min, cam.az_max, cam.el_min, cam.el_max,
-                          (cam.flags & RSIM_RC_NO_FALLOFF) ? 0 : 1, (T*)out.range, (T*)out.sigma_re,
-                          (T*)out.sigma_im, (T*)out.az, (T*)out.el, (T*)out.vel);
+  return launch_dependent(rc_render<T, N>, dim3((unsigned)rc_tiles(cam)), dim3(kRcThreads), 0, st, byval, dev, n,
+                          cam.n_az, cam.n_el, rc_tile_width(cam.n_az), (int)rc_tiles_x(cam), cam.az_min, cam.az_max,
+                          cam.el_min, cam.el_max, (cam.flags & RSIM_RC_NO_FALLOFF) ? 0 : 1, (T*)out.range,
+                          (T*)out.sigma_re, (T*)out.sigma_im, (T*)out.az, (T*)out.el, (T*)out.vel);
 }
 
 }  // namespace
@@ -436,8 +443,7 @@ extern "C" rsim_status rsim_raycast(rsim_ctx* ctx, const rsim_camera* cam, const
   if (out->dtype != RSIM_F32 && out->dtype != RSIM_F64) return fail(RSIM_ERR_INVALID_ARG, "unknown dtype");
   if (!out->range || !out->sigma_re || !out->sigma_im || !out->az || !out->el || !out->vel)
     return fail(RSIM_ERR_INVALID_ARG, "NULL output array");
-  const int64_t tw = rc_tile_width(cam->n_az), th = kRcThreads / tw;
-  if ((cam->n_az + tw - 1) / tw * ((cam->n_el + th - 1) / th) > 0x7fffffffll) return fail(RSIM_ERR_OVERFLOW, "too many pixels");
+  if (rc_tiles(*cam) > 0x7fffffffll) return fail(RSIM_ERR_OVERFLOW, "too many pixels");
   for (int k = 0; k < n_prims; ++k) {
     const std::string why = check_prim(prims[k]);
     if (!why.empty()) return fail(RSIM_ERR_INVALID_ARG, "primitive " + std::to_string(k) + ": " + why);

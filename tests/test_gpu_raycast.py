@@ -124,3 +124,29 @@ def test_image_tiles_and_primitives_by_value(ctx, n_az, n_el, n_prims):
     np.testing.assert_array_equal(got["az"], want["az"])
     np.testing.assert_array_equal(got["el"], want["el"])
     _compare(scene, got, want, 1e-11, 1e-9, 1e-9, max_ambiguous=0.03)
+
+
+@pytest.mark.parametrize("wide", [True, False])
+def test_sides_as_long_as_an_int_holds(ctx, wide):
+    """One row, or one column, of 2^31 - 1 pixels (52 GB of buffers): the number of tiles along
+    a side is not an int's arithmetic.  Every pixel is written, and the angles at both ends and
+    between are those of the grid formula."""
+    n = 2 ** 31 - 1
+    if torch.cuda.mem_get_info()[0] < 64 << 30:
+        pytest.skip("needs 64 GB of free device memory")
+    out = {k: torch.full((n,), float("nan"), dtype=torch.float32, device="cuda") for k in device.FIELDS}
+    ctx.raycast([], n if wide else 1, 1 if wide else n, FOV, out=out)
+    torch.cuda.synchronize()
+    assert bool((out["range"] == float("inf")).all())
+    for k in ("sigma_re", "sigma_im", "vel"):
+        assert bool((out[k] == 0).all())
+    (az0, az1), (el0, el1) = FOV
+    at = np.array([0, 1, 255, 256, n // 3, n - 257, n - 32, n - 1])
+    for k, lo, hi, side in (("az", az0, az1, n if wide else 1), ("el", el0, el1, 1 if wide else n)):
+        i = at if side == n else 0 * at
+        want = (lo + ((i + 0.5) * (hi - lo)) / side).astype(np.float32)
+        got = out[k][torch.from_numpy(at).cuda()].cpu().numpy()
+        np.testing.assert_array_equal(got, want)
+        assert not bool(torch.isnan(out[k]).any())
+    del out
+    torch.cuda.empty_cache()
