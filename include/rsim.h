@@ -411,14 +411,17 @@ rsim_status rsim_profile_read(rsim_ctx* ctx, rsim_profile* out);
 typedef struct {
   int32_t splits;        /* pixel splits of the contraction (K-split), 1..64 */
   int32_t chunk_px;      /* pixels per pipeline stage (always 32; reported) */
-  int32_t grid;          /* CTAs of the persistent tensor-core contraction, 0 = one per SM */
+  int32_t grid;          /* CTAs of the persistent tensor-core contraction, 0 = one per SM.  FP32
+                            tier: 0 in plans of the CUDA-core sum; a CTA count (the SM count or
+                            more: one per SM) in plans of the tensor-core form */
   int32_t variant;       /* reserved: must be 0 */
   int32_t tuned;         /* 1 if chosen by timing, 0 if by the default rule or pinned */
   int32_t tile_n;        /* tile shape.  Tensor-core tiers: l values per column tile, NT,
                             a multiple of 8 in 8..128 and at most L rounded up to 8 (the
                             MMA's N is 2 NT; default min(128, L rounded up to 8)).  FP32
-                            tier: n values per CTA tile, 64 or 128 (default 128); the CTA
-                            tile of the CUDA-core sum is tile_n x 64 (l).  NUFFT tier: ignored.  0 = default */
+                            tier, 64 or 128 (default 128): the n values of a CTA tile of the
+                            CUDA-core sum, tile_n x 64 (l); the l values of a column tile of
+                            the tensor-core form, at most.  NUFFT tier: ignored.  0 = default */
   int32_t group_chunks;  /* tensor-core tiers: 32-pixel chunks summed in one tensor-memory
                             accumulator before it is drained into round-to-nearest FP32
                             sums.  The accumulator rounds toward zero, so the cap bounds the
@@ -439,15 +442,17 @@ rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* params, int64_
                           rsim_tier tier, rsim_plan* chosen, rsim_stream stream);
 
 /* Pin `plan` for the bucket of (params, P, tier) in the context's cache (replaces a tuned
- * or default plan).  For RSIM_TIER_FP32 the plan is one of the CUDA-core sum, which then
- * runs the bucket.  splits in 1..64; grid 0 (one CTA per SM) or a positive CTA count
+ * or default plan).  For RSIM_TIER_FP32 a plan with grid 0 is one of the CUDA-core sum, which
+ * then runs the bucket, and one with a CTA count one of the tensor-core form, as rsim_get_plan
+ * and rsim_autotune return them (a plan read and set again changes nothing).  splits in 1..64; grid 0 (one CTA per SM) or a positive CTA count
  * (more than the SM count runs as one per SM); variant 0; tile_n and group_chunks 0 or in
  * the ranges stated in rsim_plan.  Host only.  Errors: INVALID_ARG. */
 rsim_status rsim_set_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_t P,
                           rsim_tier tier, const rsim_plan* plan);
 
 /* The plan rsim_synth would use now for (params, P, tier), with tile_n and group_chunks
- * resolved (never 0 for the tiers that use them).  Host only. */
+ * resolved (never 0 for the tiers that use them; group_chunks of the FP32 tier is 0: the
+ * library's own).  Host only. */
 rsim_status rsim_get_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_t P,
                           rsim_tier tier, rsim_plan* plan);
 

@@ -147,9 +147,12 @@ rsim_plan choose_plan(rsim_ctx* ctx, int tier, const Consts& k, int64_t P) {
 // bucket, and one frame's workspace fits tensor_bytes_cap(budget).
 size_t tensor_bytes_cap(size_t budget) { return budget ? std::min(budget, kFp32TensorBytes) : kFp32TensorBytes; }
 
+static bool tensor_form_possible(const rsim_ctx* ctx, int64_t P) {
+  return ctx->cc_major == 10 && ctx->cc_minor == 3 && fp32_on_tensor_cores(P);
+}
+
 int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budget) {
-  if (tier != RSIM_TIER_FP32 || !(ctx->cc_major == 10 && ctx->cc_minor == 3) || !fp32_on_tensor_cores(P))
-    return tier;
+  if (tier != RSIM_TIER_FP32 || !tensor_form_possible(ctx, P)) return tier;
   {
     std::lock_guard<std::mutex> g(ctx->plan_mu);
     auto it = ctx->plans.find(plan_key(tier, k, P));
@@ -159,15 +162,27 @@ int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budg
   return batch_bytes(k, &P, 1, plan, kTierFp32Tensor) > tensor_bytes_cap(budget) ? tier : kTierFp32Tensor;
 }
 
-// A plan as its caller sees it: the tensor-core engine of the FP32 tier shows its splits and
-// grid, and the tier's n tile (128 rows, which it uses too).
-rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int engine) {
+// Plans of the FP32 tier as callers see and set them (rsim_plan): a CTA count marks those of the
+// tensor-core form, whose column tile is the default one (shown as 128) or 64.  The two functions
+// undo each other, so that a plan that was read and is set again changes nothing.
+rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int engine, int num_sms) {
   if (engine == tier) return plan;
   rsim_plan p{};
   resolve_tile(tier, k, &p);
   p.splits = plan.splits;
-  p.grid = plan.grid;
+  p.grid = plan.grid > 0 && plan.grid < num_sms ? plan.grid : num_sms;
+  p.tile_n = plan.tile_n < tile_nt(k.L) ? 64 : 128;
   p.tuned = plan.tuned;
+  return p;
+}
+
+static rsim_plan tensor_form_plan(const Consts& k, const rsim_plan& plan, int num_sms) {
+  rsim_plan p{};
+  p.splits = plan.splits;
+  p.grid = plan.grid < num_sms ? plan.grid : 0;
+  p.tile_n = plan.tile_n == 64 ? std::min(64, tile_nt(k.L)) : 0;
+  p.tuned = plan.tuned;
+  resolve_tile(kTierFp32Tensor, k, &p);
   return p;
 }
 
@@ -827,7 +842,12 @@ rsim_status rsim_set_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_
   rsim_plan p = *plan;
   resolve_tile(tier, k, &p);
   std::lock_guard<std::mutex> g(ctx->plan_mu);
-  ctx->plans[plan_key(tier, k, P)] = p;
+  if (tier == RSIM_TIER_FP32 && p.grid > 0 && tensor_form_possible(ctx, P)) {
+    ctx->plans.erase(plan_key(tier, k, P));
+    ctx->plans[plan_key(kTierFp32Tensor, k, P)] = tensor_form_plan(k, p, ctx->num_sms);
+  } else {
+    ctx->plans[plan_key(tier, k, P)] = p;
+  }
   return RSIM_OK;
 }
 
@@ -839,7 +859,7 @@ rsim_status rsim_get_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_
   rsim_status s = check_params(params, &k);
   if (s != RSIM_OK) return s;
   const int engine = engine_tier(ctx, tier, k, P, ctx->budget);
-  *plan = reported_plan(tier, k, choose_plan(ctx, engine, k, P), engine);
+  *plan = reported_plan(tier, k, choose_plan(ctx, engine, k, P), engine, ctx->num_sms);
   return RSIM_OK;
 }
 

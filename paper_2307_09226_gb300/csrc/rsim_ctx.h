@@ -49,7 +49,7 @@ rsim_status check_pixels(const rsim_pixels* px);
 bool tier_ok(int tier);
 std::string plan_key(int tier, const Consts& k, int64_t P);
 rsim_plan choose_plan(rsim_ctx* ctx, int tier, const Consts& k, int64_t P);
-rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int engine);
+rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int engine, int num_sms);
 int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budget);
 size_t batch_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& plan, int tier);
 rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st);

@@ -264,6 +264,6 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
     ctx->plans[plan_key(tier, k, P)] = best;
     save_plan_cache(ctx);
   }
-  *chosen = reported_plan(asked, k, best, tier);
+  *chosen = reported_plan(asked, k, best, tier, ctx->num_sms);
   return RSIM_OK;
 }

@@ -1,0 +1,83 @@
+"""The FP32 tier's two forms, the tensor-core form and the CUDA-core sum: which one a call
+takes (plans, saved plans, workspace bounds, captures) and the CUDA-core sum's own results."""
+import json
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_09226_gb300 import synth
+from paper_2307_09226_gb300.synth import Radar
+
+pytestmark = pytest.mark.gpu
+FP32_BAR = 1e-6    # the tensor-core form (derived in test_gpu_fp32_tensor.py)
+DIRECT_BAR = 2e-5  # the tier
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2307_09226_gb300 import _abi, device
+    ctx = device.Context(0)
+    yield torch, _abi, device, ctx
+    ctx.close()
+
+
+def sizes(env, radar, P):
+    """Workspace of the tensor-core form and of the CUDA-core sum under their default plans."""
+    torch, _abi, device, ctx = env
+    tensor = _abi.rsim_workspace_size(ctx.h, radar, P, _abi.TIER_FP32)
+    small = device.Context(0, hbm_budget_bytes=tensor - 256)
+    direct = _abi.rsim_workspace_size(small.h, radar, P, _abi.TIER_FP32)
+    small.close()
+    assert direct < tensor
+    return tensor, direct
+
+
+def split(plan):
+    d = plan.as_dict()
+    d.pop("tuned")
+    return d
+
+
+@pytest.mark.parametrize("Ns,L,n_az,n_el", [(128, 64, 64, 64), (96, 40, 60, 50), (64, 256, 90, 40), (64, 32, 10, 9)])
+@pytest.mark.parametrize("tune", [False, True])
+def test_a_plan_read_and_set_again_changes_nothing(env, Ns, L, n_az, n_el, tune):
+    """What rsim_get_plan or rsim_autotune returns, pinned in a new context: the same form
+    (its workspace), the same plan, the same bits."""
+    torch, _abi, device, _ = env
+    f = synth.parity_frame(seed=Ns + L, M=2, N=3, Ns=Ns, L=L, n_az=n_az, n_el=n_el)
+    d, P = device.upload(f), f.pixels.P
+    a, b = device.Context(0), device.Context(0)
+    plan = _abi.rsim_autotune(a.h, f.radar, P, _abi.TIER_FP32) if tune else _abi.rsim_get_plan(a.h, f.radar, P, _abi.TIER_FP32)
+    _abi.rsim_set_plan(b.h, f.radar, P, _abi.TIER_FP32, **split(plan))
+    assert split(_abi.rsim_get_plan(b.h, f.radar, P, _abi.TIER_FP32)) == split(plan)
+    assert _abi.rsim_workspace_size(a.h, f.radar, P, _abi.TIER_FP32) == _abi.rsim_workspace_size(b.h, f.radar, P, _abi.TIER_FP32)
+    want, got = (c.synth(f.radar, d, "fp32").cpu().numpy() for c in (a, b))
+    assert a.sync_status() == _abi.OK and b.sync_status() == _abi.OK
+    assert np.array_equal(want, got)
+    assert oracle.rel_l2(got, oracle.cube_separable(f.radar, f.pixels)) <= FP32_BAR
+    a.close(), b.close()
+
+
+def test_a_plan_of_the_cuda_core_sum_and_back(env):
+    """grid 0 pins the CUDA-core sum, a CTA count the tensor-core form again; a plan read while
+    the CUDA-core sum runs pins the CUDA-core sum."""
+    torch, _abi, device, _ = env
+    radar, P = Radar(M=2, N=4, Ns=64, L=64), 4800
+    tensor, direct = sizes(env, radar, P)
+    c = device.Context(0)
+    _abi.rsim_set_plan(c.h, radar, P, _abi.TIER_FP32, splits=2)
+    pinned = _abi.rsim_workspace_size(c.h, radar, P, _abi.TIER_FP32)
+    plan = _abi.rsim_get_plan(c.h, radar, P, _abi.TIER_FP32)
+    assert plan.grid == 0 and plan.splits == 2
+    _abi.rsim_set_plan(c.h, radar, P, _abi.TIER_FP32, **split(plan))
+    assert _abi.rsim_workspace_size(c.h, radar, P, _abi.TIER_FP32) == pinned < tensor
+    free = device.Context(0)
+    _abi.rsim_set_plan(c.h, radar, P, _abi.TIER_FP32, **split(_abi.rsim_get_plan(free.h, radar, P, _abi.TIER_FP32)))
+    assert _abi.rsim_workspace_size(c.h, radar, P, _abi.TIER_FP32) == tensor
+    free.close(), c.close()
