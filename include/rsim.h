@@ -75,8 +75,8 @@ typedef enum {
   RSIM_TIER_FP32 = 0,       /* FP32 accuracy (relative error below 1e-6 where measured).  From 128
                                pixels on, tcgen05 with FP16 hi+lo operands (3 products) and FP32 sums
                                of at most two 32-pixel chunks each; else, and wherever a plan of its
-                               own is pinned or tuned for the shape or the workspace bound holds no
-                               more, the FP32 direct sum on CUDA cores */
+                               own is pinned for the shape or the workspace bound holds no more, the
+                               FP32 direct sum on CUDA cores */
   RSIM_TIER_BF16 = 1,       /* tcgen05 tensor cores, BF16 operands, FP32 accumulate */
   RSIM_TIER_SPLIT_BF16 = 2, /* tcgen05, BF16 hi+lo operands (3 products), FP32 accumulate */
   RSIM_TIER_SPLIT_FP16 = 3, /* tcgen05, FP16 hi+lo operands (3 products), FP32 accumulate */

@@ -1,5 +1,5 @@
 // FP32 direct sum of Eq. 2 on CUDA cores: the FP32 tier's form for frames of fewer than
-// kFp32TensorPixels pixels, for buckets with a plan of their own and where the operand images
+// kFp32TensorPixels pixels, for buckets with a pinned plan of its own and where the operand images
 // do not fit (see fp32_on_tensor_cores); other FP32 frames run on the tensor cores.
 //
 // The phase of Eq. 2 separates into a fast-time/channel part a_{p,v} n + c_{p,v} and a

@@ -143,8 +143,9 @@ rsim_plan choose_plan(rsim_ctx* ctx, int tier, const Consts& k, int64_t P) {
 
 // The arithmetic that runs a call of `tier` over F frames of at most P pixels: `tier` itself,
 // or, for the FP32 tier, the tensor cores where the pixel count says so
-// (fp32_on_tensor_cores), no plan for the CUDA-core kernel is pinned or tuned for the shape's
-// bucket, and one frame's workspace fits tensor_bytes_cap(budget).
+// (fp32_on_tensor_cores), no plan of the CUDA-core sum is pinned for the shape's bucket, and one
+// frame's workspace fits tensor_bytes_cap(budget).  (A tuned plan of the CUDA-core sum, from this
+// context or a tuning file, is for the calls that it runs and chooses nothing.)
 size_t tensor_bytes_cap(size_t budget) { return budget ? std::min(budget, kFp32TensorBytes) : kFp32TensorBytes; }
 
 static bool tensor_form_possible(const rsim_ctx* ctx, int64_t P) {
@@ -155,8 +156,7 @@ int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budg
   if (tier != RSIM_TIER_FP32 || !tensor_form_possible(ctx, P)) return tier;
   {
     std::lock_guard<std::mutex> g(ctx->plan_mu);
-    auto it = ctx->plans.find(plan_key(tier, k, P));
-    if (it != ctx->plans.end() && plan_problem(tier, k, it->second).empty()) return tier;
+    if (ctx->pinned_direct.count(plan_key(tier, k, P))) return tier;
   }
   const rsim_plan plan = choose_plan(ctx, kTierFp32Tensor, k, P);
   return batch_bytes(k, &P, 1, plan, kTierFp32Tensor) > tensor_bytes_cap(budget) ? tier : kTierFp32Tensor;
@@ -844,9 +844,11 @@ rsim_status rsim_set_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_
   std::lock_guard<std::mutex> g(ctx->plan_mu);
   if (tier == RSIM_TIER_FP32 && p.grid > 0 && tensor_form_possible(ctx, P)) {
     ctx->plans.erase(plan_key(tier, k, P));
+    ctx->pinned_direct.erase(plan_key(tier, k, P));
     ctx->plans[plan_key(kTierFp32Tensor, k, P)] = tensor_form_plan(k, p, ctx->num_sms);
   } else {
     ctx->plans[plan_key(tier, k, P)] = p;
+    if (tier == RSIM_TIER_FP32) ctx->pinned_direct.insert(plan_key(tier, k, P));
   }
   return RSIM_OK;
 }

@@ -4,6 +4,7 @@
 
 #include <map>
 #include <mutex>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -34,6 +35,7 @@ struct rsim_ctx {
   bool nu_ready = false;                   // all of nu_st and nu_ev exist
   std::mutex plan_mu;
   std::map<std::string, rsim_plan> plans;
+  std::set<std::string> pinned_direct;  // FP32 buckets for which rsim_set_plan chose the CUDA-core sum
   // stage profiling (rsim_profile_enable / rsim_profile_read)
   bool prof = false;
   std::vector<cudaEvent_t> ev_pool;  // kProfEvents events per recorded call

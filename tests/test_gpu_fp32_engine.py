@@ -81,3 +81,25 @@ def test_a_plan_of_the_cuda_core_sum_and_back(env):
     _abi.rsim_set_plan(c.h, radar, P, _abi.TIER_FP32, **split(_abi.rsim_get_plan(free.h, radar, P, _abi.TIER_FP32)))
     assert _abi.rsim_workspace_size(c.h, radar, P, _abi.TIER_FP32) == tensor
     free.close(), c.close()
+
+
+def test_a_tuned_entry_of_the_cuda_core_sum_does_not_choose_the_form(env, tmp_path, monkeypatch):
+    """A tuning file may hold an entry of the CUDA-core sum for a shape (tuned where the
+    workspace bound left nothing else, or by a version of the library that had nothing else):
+    it is the plan of that sum, not a choice of it, and tuning again times the form that runs."""
+    torch, _abi, device, _ = env
+    radar, P = Radar(M=2, N=4, Ns=128, L=64), 4000
+    tensor, direct = sizes(env, radar, P)
+    cache = tmp_path / "tune.json"
+    cache.write_text(json.dumps({"t0_V8_Ns128_L64_b12": [2, 0, 64, 0]}))
+    monkeypatch.setenv("RSIM_TUNE_CACHE", str(cache))
+    c = device.Context(0)
+    assert not _abi.rsim_get_plan(c.h, radar, P, _abi.TIER_FP32).tuned
+    assert _abi.rsim_workspace_size(c.h, radar, P, _abi.TIER_FP32) == tensor
+    small = device.Context(0, hbm_budget_bytes=tensor - 256)
+    plan = _abi.rsim_get_plan(small.h, radar, P, _abi.TIER_FP32)
+    assert plan.tuned == 1 and plan.splits == 2 and plan.tile_n == 64
+    assert _abi.rsim_autotune(c.h, radar, P, _abi.TIER_FP32).tuned == 1
+    assert any(key.startswith("t6_V8_Ns128_L64") for key in json.loads(cache.read_text()))
+    assert _abi.rsim_get_plan(c.h, radar, P, _abi.TIER_FP32).grid > 0  # the tensor-core form
+    small.close(), c.close()
