@@ -53,6 +53,7 @@ std::string plan_key(int tier, const Consts& k, int64_t P);
 rsim_plan choose_plan(rsim_ctx* ctx, int tier, const Consts& k, int64_t P);
 rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int engine, int num_sms);
 int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budget);
+size_t tensor_bytes_cap(size_t budget);
 size_t batch_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& plan, int tier);
 rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st);
 rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k,

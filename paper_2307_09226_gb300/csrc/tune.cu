@@ -166,7 +166,11 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
   auto time_plan = [&](const rsim_plan& p) -> float {
     if (err != RSIM_OK || !plan_problem(tier, k, p).empty()) return 1e30f;
     int64_t PP = P;
-    rsim_status s2 = ensure_workspace(ctx, batch_bytes(k, &PP, 1, p, tier), st);
+    const size_t need = batch_bytes(k, &PP, 1, p, tier);
+    // candidates with more splits that pass the bound of the FP32 tier's tensor-core form, which
+    // the default plan keeps
+    if (tier == kTierFp32Tensor && need > tensor_bytes_cap(ctx->budget)) return 1e30f;
+    rsim_status s2 = ensure_workspace(ctx, need, st);
     if (s2 != RSIM_OK) {
       err = s2;
       return 1e30f;
@@ -250,6 +254,7 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
       }
     }
   }
+  if (tb >= 1e30f && err == RSIM_OK) best = choose_plan(ctx, tier, k, P);  // no candidate fits: the plan in use
   best.tuned = 1;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

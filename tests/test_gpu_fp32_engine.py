@@ -103,3 +103,16 @@ def test_a_tuned_entry_of_the_cuda_core_sum_does_not_choose_the_form(env, tmp_pa
     assert any(key.startswith("t6_V8_Ns128_L64") for key in json.loads(cache.read_text()))
     assert _abi.rsim_get_plan(c.h, radar, P, _abi.TIER_FP32).grid > 0  # the tensor-core form
     small.close(), c.close()
+
+
+def test_tuning_within_a_bound(env):
+    """A budget that holds the default plan of the tensor-core form, but not the candidates with
+    more splits: tuning takes the candidates that fit."""
+    torch, _abi, device, _ = env
+    radar, P = Radar(M=2, N=4, Ns=128, L=64), 4000
+    tensor, direct = sizes(env, radar, P)
+    c = device.Context(0, hbm_budget_bytes=tensor + 4096)
+    plan = _abi.rsim_autotune(c.h, radar, P, _abi.TIER_FP32)
+    assert plan.tuned == 1 and plan.as_dict() == _abi.rsim_get_plan(c.h, radar, P, _abi.TIER_FP32).as_dict()
+    assert direct < _abi.rsim_workspace_size(c.h, radar, P, _abi.TIER_FP32) <= tensor + 4096
+    c.close()
