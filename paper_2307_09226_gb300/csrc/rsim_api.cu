@@ -239,6 +239,16 @@ rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st) {
   return RSIM_OK;
 }
 
+// Whether `st` is being captured (the workspace cannot grow meanwhile).
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap != cudaStreamCaptureStatusNone;
+}
+
 // Fill FrameIO entries for F frames in workspace `ws`.  A batch's table is uploaded
 // here; a single frame's entry goes to the first kernel by value (launch_prep), and the
 // meta words and the unit counter are cleared by that kernel too.
@@ -670,27 +680,36 @@ rsim_status rsim_synth_batch(rsim_ctx* ctx, const rsim_radar_params* params,
   if (engine != tier) {
     // the FP32 tier on the tensor cores needs more workspace than its CUDA-core kernel (2 KB
     // a pixel and column tile): a batch beyond the cap runs a few frames at a time (the same
-    // bits), and where the memory cannot be had at all the CUDA-core kernel takes the call
-    // below
+    // bits), and where the memory cannot be had at all, or not during a capture in a workspace
+    // that holds the CUDA-core kernel's, that kernel takes the call below
     const size_t cap = tensor_bytes_cap(ctx->budget);
-    const rsim_plan plan = choose_plan(ctx, engine, k, maxp);
-    int done = 0;
-    while (done < F) {
-      int n = F - done;
-      while (n > 1 && batch_bytes(k, Ps.data() + done, n, plan, engine) > cap) n = (n + 1) / 2;
-      s = ensure_workspace(ctx, batch_bytes(k, Ps.data() + done, n, plan, engine), st);
-      if (s == RSIM_ERR_OOM && done == 0) break;
-      if (s == RSIM_OK)
-        s = run_frames(ctx, (char*)ctx->ws, ctx->ws_bytes, k, frames + done, n, cubes + done, engine, out_dtype, plan,
-                       ctx->status_dev, st);
-      if (s != RSIM_OK) return s;
-      done += n;
+    const rsim_plan tplan = choose_plan(ctx, engine, k, maxp);
+    std::vector<int> parts;
+    size_t most = 0;
+    for (int at = 0; at < F; at += parts.back()) {
+      int n = F - at;
+      while (n > 1 && batch_bytes(k, Ps.data() + at, n, tplan, engine) > cap) n = (n + 1) / 2;
+      parts.push_back(n);
+      most = std::max(most, batch_bytes(k, Ps.data() + at, n, tplan, engine));
     }
-    if (done == F) return RSIM_OK;
+    const bool instead = ctx->ws_bytes < most && capturing(st) &&
+                         batch_bytes(k, Ps.data(), F, choose_plan(ctx, tier, k, maxp), tier) <= ctx->ws_bytes;
+    if (!instead) {
+      int done = 0;
+      for (int n : parts) {
+        s = ensure_workspace(ctx, batch_bytes(k, Ps.data() + done, n, tplan, engine), st);
+        if (s == RSIM_ERR_OOM && done == 0) break;
+        if (s == RSIM_OK)
+          s = run_frames(ctx, (char*)ctx->ws, ctx->ws_bytes, k, frames + done, n, cubes + done, engine, out_dtype,
+                         tplan, ctx->status_dev, st);
+        if (s != RSIM_OK) return s;
+        done += n;
+      }
+      if (done == F) return RSIM_OK;
+    }
   }
-  rsim_plan plan = choose_plan(ctx, tier, k, maxp);
-  const size_t need = batch_bytes(k, Ps.data(), F, plan, tier);
-  s = ensure_workspace(ctx, need, st);
+  const rsim_plan plan = choose_plan(ctx, tier, k, maxp);
+  s = ensure_workspace(ctx, batch_bytes(k, Ps.data(), F, plan, tier), st);
   if (s != RSIM_OK) return s;
   return run_frames(ctx, (char*)ctx->ws, ctx->ws_bytes, k, frames, F, cubes, tier, out_dtype, plan,
                     ctx->status_dev, st);

@@ -116,3 +116,33 @@ def test_tuning_within_a_bound(env):
     assert plan.tuned == 1 and plan.as_dict() == _abi.rsim_get_plan(c.h, radar, P, _abi.TIER_FP32).as_dict()
     assert direct < _abi.rsim_workspace_size(c.h, radar, P, _abi.TIER_FP32) <= tensor + 4096
     c.close()
+
+
+def test_capture_in_a_workspace_of_the_cuda_core_sum(env):
+    """A call captured in a workspace that holds the CUDA-core sum but not the tensor-core form:
+    it cannot grow during the capture, and the call takes the CUDA-core sum."""
+    torch, _abi, device, ctx = env
+    radar = Radar(M=1, N=1, Ns=64, L=64)
+    px = synth.random_frame(radar, 100, 96, seed=21, mask_frac=0.2)
+    tensor, direct = sizes(env, radar, px.P)
+    d, cube = device.upload(px), torch.zeros((1, 64, 64), dtype=torch.complex64, device="cuda")
+    ctx.synth(radar, device.upload(synth.random_frame(radar, 10, 10, seed=22)), "fp32")  # loads the kernels
+    c = device.Context(0)
+    # 2 MiB of row transforms: a workspace of 3 MiB
+    big = Radar(M=1, N=1, Ns=512, L=512)
+    assert direct < 2 << 20 and tensor > 4 << 20
+    _abi.rsim_range_doppler(c.h, big, [torch.zeros((1, 512, 512), dtype=torch.complex64, device="cuda")],
+                            torch.empty((1, 512, 512), device="cuda"), torch.empty(1, device="cuda"))
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        c.synth(radar, d, "fp32", cube=cube, stream=s)
+    g.replay()
+    torch.cuda.synchronize()
+    assert c.sync_status() == _abi.OK
+    assert oracle.rel_l2(cube.cpu().numpy(), oracle.cube_separable(radar, px)) <= DIRECT_BAR
+    # outside a capture the workspace grows and the tensor-core form runs
+    got = c.synth(radar, d, "fp32").cpu().numpy()
+    assert np.array_equal(got, ctx.synth(radar, d, "fp32").cpu().numpy())
+    c.close()
