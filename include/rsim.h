@@ -182,7 +182,8 @@ rsim_status rsim_synth(rsim_ctx* ctx, const rsim_radar_params* params, const rsi
  * and unchanged until the stream has passed the call's work (e.g. rsim_sync_status); with
  * pageable memory and no direct access the copies block the calling thread.  The staging buffer grows when
  * needed (cudaMalloc after one stream synchronisation) and counts against the context's
- * budget with the workspace.
+ * budget with the workspace (which is given back first, if an FP32-tier call on the tensor
+ * cores had grown it beyond what other calls need).
  * Errors: as rsim_synth. */
 rsim_status rsim_synth_host(rsim_ctx* ctx, const rsim_radar_params* params, const rsim_pixels* pixels,
                             rsim_tier tier, void* cube, int32_t out_dtype, rsim_stream stream);

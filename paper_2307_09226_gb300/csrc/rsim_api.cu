@@ -217,7 +217,15 @@ size_t batch_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& pl
   return o;
 }
 
-rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st) {
+// The size a workspace that has to hold `bytes` is given: an eighth more where the budget allows.
+static size_t grown(const rsim_ctx* ctx, size_t bytes) {
+  const size_t want = align_up(bytes + bytes / 8, 1 << 20);
+  return ctx->budget && want > ctx->budget ? bytes : want;
+}
+
+rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st, size_t base) {
+  base = std::min(base, bytes);
+  if (base > ctx->ws_base && !(ctx->budget && base > ctx->budget)) ctx->ws_base = grown(ctx, base);
   if (ctx->ws_bytes >= bytes) return RSIM_OK;
   if (ctx->budget && bytes > ctx->budget)
     return fail(RSIM_ERR_BUDGET, "workspace of " + std::to_string(bytes) +
@@ -228,8 +236,7 @@ rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st) {
   if (ctx->ws) cudaFree(ctx->ws);
   ctx->ws = nullptr;
   ctx->ws_bytes = 0;
-  size_t want = align_up(bytes + bytes / 8, 1 << 20);
-  if (ctx->budget && want > ctx->budget) want = bytes;
+  const size_t want = grown(ctx, bytes);
   e = cudaMalloc(&ctx->ws, want);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -592,10 +599,17 @@ rsim_status rsim_synth_host(rsim_ctx* ctx, const rsim_radar_params* params, cons
   for (int i = 0; i < 6 && direct; ++i) direct = (view[i] = device_view(ctx, src[i])) != nullptr;
   if (direct) need = cube_bytes;
   if (ctx->stage_bytes < need) {
-    if (ctx->budget && ctx->ws_bytes + need > ctx->budget)
+    const bool give_back = ctx->budget && ctx->ws_bytes + need > ctx->budget;
+    if (give_back && (ctx->ws_base >= ctx->ws_bytes || ctx->ws_base + need > ctx->budget))
       return fail(RSIM_ERR_BUDGET, "staging of " + std::to_string(need) + " bytes exceeds the context budget");
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    if (give_back) {
+      // the FP32 tier's tensor-core form had grown the workspace beyond what other calls need
+      cudaFree(ctx->ws);
+      ctx->ws = nullptr;
+      ctx->ws_bytes = 0;
+    }
     if (ctx->stage) cudaFree(ctx->stage);
     ctx->stage = nullptr;
     ctx->stage_bytes = 0;
@@ -697,7 +711,10 @@ rsim_status rsim_synth_batch(rsim_ctx* ctx, const rsim_radar_params* params,
     if (!instead) {
       int done = 0;
       for (int n : parts) {
-        s = ensure_workspace(ctx, batch_bytes(k, Ps.data() + done, n, tplan, engine), st);
+        const size_t bytes = batch_bytes(k, Ps.data() + done, n, tplan, engine);
+        // (the CUDA-core sum's need is worked out only where the workspace grows)
+        s = ensure_workspace(ctx, bytes, st, ctx->ws_bytes >= bytes ? 0 :
+                             batch_bytes(k, Ps.data(), F, choose_plan(ctx, tier, k, maxp), tier));
         if (s == RSIM_ERR_OOM && done == 0) break;
         if (s == RSIM_OK)
           s = run_frames(ctx, (char*)ctx->ws, ctx->ws_bytes, k, frames + done, n, cubes + done, engine, out_dtype,

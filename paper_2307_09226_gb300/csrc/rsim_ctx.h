@@ -20,6 +20,7 @@ struct rsim_ctx {
   size_t budget = 0;
   void* ws = nullptr;
   size_t ws_bytes = 0;
+  size_t ws_base = 0;  // what it would be without the FP32 tier's tensor-core form
   // 256 bytes: word 0 is the status word of the context's own calls (rsim_sync_status);
   // word 32 is the shared-atomic probe's sink and word 33 the tensor-core probe's wait
   // failures (measure.cu); the rest is unused
@@ -55,7 +56,8 @@ rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int en
 int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budget);
 size_t tensor_bytes_cap(size_t budget);
 size_t batch_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& plan, int tier);
-rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st);
+// `base`: the bytes without the FP32 tier's tensor-core form, where that is what takes `bytes`.
+rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st, size_t base = SIZE_MAX);
 rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k,
                        const rsim_pixels* frames, int F, void* const* cubes, int tier,
                        int out_dtype, const rsim_plan& plan, unsigned* status, cudaStream_t st);

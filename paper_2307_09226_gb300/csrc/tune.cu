@@ -170,7 +170,7 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
     // candidates with more splits that pass the bound of the FP32 tier's tensor-core form, which
     // the default plan keeps
     if (tier == kTierFp32Tensor && need > tensor_bytes_cap(ctx->budget)) return 1e30f;
-    rsim_status s2 = ensure_workspace(ctx, need, st);
+    rsim_status s2 = ensure_workspace(ctx, need, st, tier == kTierFp32Tensor ? 0 : need);
     if (s2 != RSIM_OK) {
       err = s2;
       return 1e30f;

@@ -146,3 +146,41 @@ def test_capture_in_a_workspace_of_the_cuda_core_sum(env):
     got = c.synth(radar, d, "fp32").cpu().numpy()
     assert np.array_equal(got, ctx.synth(radar, d, "fp32").cpu().numpy())
     c.close()
+
+
+def test_host_call_after_the_tensor_core_form_filled_the_budget(env):
+    """The staging buffer of rsim_synth_host counts against the budget with the workspace.  A
+    workspace that an FP32 call on the tensor cores grew beyond the CUDA-core sum's is given
+    back where the staging would otherwise be refused."""
+    torch, _abi, device, ctx = env
+    radar = Radar(M=2, N=4, Ns=64, L=64)
+    px = synth.random_frame(radar, 80, 60, seed=31, mask_frac=0.3)
+    tensor, direct = sizes(env, radar, px.P)
+    cube_bytes = 8 * 64 * 64 * 8
+    assert direct + direct // 8 + (1 << 20) + cube_bytes < tensor
+    c = device.Context(0, hbm_budget_bytes=tensor + 4096)
+    d = device.upload(px)
+    want = c.synth(radar, d, "fp32").cpu().numpy()
+    host = {k: torch.from_numpy(np.ascontiguousarray(a)).pin_memory() for k, a in zip(device.FIELDS, px.arrays())}
+    for tier, bar in (("nufft", 2e-5), ("fp32", FP32_BAR)):
+        got = c.synth_host(radar, host, tier)
+        assert c.sync_status() == _abi.OK
+        assert oracle.rel_l2(got.numpy(), oracle.cube_separable(radar, px)) <= bar
+    assert np.array_equal(got.numpy(), want)
+    c.close()
+
+
+def test_staging_beyond_the_budget_stays_refused(env):
+    """A staging buffer that does not fit beside the workspace other calls need is refused."""
+    torch, _abi, device, ctx = env
+    radar = Radar(M=2, N=4, Ns=64, L=64)
+    px = synth.random_frame(radar, 80, 60, seed=32, mask_frac=0.3)
+    need = _abi.rsim_workspace_size(ctx.h, radar, px.P, _abi.TIER_SPLIT_FP16)
+    c = device.Context(0, hbm_budget_bytes=need + 4096)
+    c.synth(radar, device.upload(px), "split_fp16")
+    c.synth(radar, device.upload(px), "fp32")
+    host = {k: torch.from_numpy(np.ascontiguousarray(a)).pin_memory() for k, a in zip(device.FIELDS, px.arrays())}
+    with pytest.raises(_abi.RsimError) as e:
+        c.synth_host(radar, host, "split_fp16")
+    assert e.value.status == _abi.ERR_BUDGET
+    c.close()
