@@ -357,6 +357,12 @@ rsim_status rsim_sync_status(rsim_ctx* ctx, rsim_stream stream);
  * Errors: INVALID_ARG (NULL ctx, limit out of range), CUDA. */
 rsim_status rsim_selftest_wait_timeout(rsim_ctx* ctx, uint64_t limit_ns, rsim_stream stream);
 
+/* The same for device memory that cannot be had (no counterpart in the paper): workspace
+ * allocations of more than `bytes`, the context's and those of servers on it, fail from now
+ * on as they do when the device's memory is exhausted.  0 ends the test.  Host only.
+ * Errors: INVALID_ARG (NULL ctx). */
+rsim_status rsim_selftest_alloc_limit(rsim_ctx* ctx, size_t bytes);
+
 /* Measurement helper for benchmarks (no counterpart in the paper): the rate, in lane
  * operations per second, at which this device performs non-returning 32-bit integer
  * atomic additions to shared memory without bank conflicts, at the NUFFT spreading
@@ -478,7 +484,9 @@ rsim_status rsim_get_plan(rsim_ctx* ctx, const rsim_radar_params* params, int64_
  * slots (rsim_server_opts.express_slots), beyond the general ones, take short requests
  * only, so a short request does not wait in the queue while long requests hold every
  * general slot; a short request also goes to a free express slot first.  Results do not
- * depend on the policy or the priority.  Completion is detected by a host function after
+ * depend on the policy or the priority.  An FP32-tier request takes the tensor-core form where
+ * its workspace fits the server's budget, as rsim_synth does with the context's; where that much
+ * cannot be allocated it runs as the CUDA-core sum.  Completion is detected by a host function after
  * the request's work; latency is measured from submit() to completion.
  * ---------------------------------------------------------------------------------- */
 typedef struct rsim_server rsim_server;

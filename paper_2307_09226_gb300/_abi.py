@@ -139,6 +139,7 @@ SIGNATURES = {
                                    c_void_p, c_void_p, c_void_p, c_int32, c_void_p]),
     "rsim_sync_status": (c_int, [c_void_p, c_void_p]),
     "rsim_selftest_wait_timeout": (c_int, [c_void_p, c_uint64, c_void_p]),
+    "rsim_selftest_alloc_limit": (c_int, [c_void_p, c_size_t]),
     "rsim_measure_smem_atomics": (c_int, [c_void_p, POINTER(c_double), c_void_p]),
     "rsim_measure_mma_rate": (c_int, [c_void_p, POINTER(c_double), c_void_p]),
     "rsim_autotune": (c_int, [c_void_p, POINTER(rsim_radar_params), c_int64, c_int,
@@ -362,6 +363,10 @@ def rsim_raycast(ctx, scene, n_az, n_el, fov, out, falloff=True, stream=None):
     arr = primitives_array(scene)
     ptr = arr.ctypes.data_as(POINTER(rsim_primitive)) if arr.size else None
     check(load().rsim_raycast(ctx, ctypes.byref(cam), ptr, int(arr.size), ctypes.byref(po), _stream(stream)))
+
+
+def rsim_selftest_alloc_limit(ctx, nbytes: int) -> None:
+    check(load().rsim_selftest_alloc_limit(ctx, int(nbytes)))
 
 
 def rsim_profile_enable(ctx, on: bool):

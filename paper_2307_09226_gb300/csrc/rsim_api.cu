@@ -217,6 +217,17 @@ size_t batch_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& pl
   return o;
 }
 
+static bool beyond_limit(const rsim_ctx* ctx, size_t bytes) {
+  const size_t limit = ctx->alloc_limit;
+  return limit && bytes > limit;
+}
+cudaError_t workspace_malloc(const rsim_ctx* ctx, void** p, size_t bytes) {
+  return beyond_limit(ctx, bytes) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+}
+cudaError_t workspace_malloc_async(const rsim_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
+  return beyond_limit(ctx, bytes) ? cudaErrorMemoryAllocation : cudaMallocAsync(p, bytes, st);
+}
+
 // The size a workspace that has to hold `bytes` is given: an eighth more where the budget allows.
 static size_t grown(const rsim_ctx* ctx, size_t bytes) {
   const size_t want = align_up(bytes + bytes / 8, 1 << 20);
@@ -237,7 +248,7 @@ rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st, size_
   ctx->ws = nullptr;
   ctx->ws_bytes = 0;
   const size_t want = grown(ctx, bytes);
-  e = cudaMalloc(&ctx->ws, want);
+  e = workspace_malloc(ctx, &ctx->ws, want);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(RSIM_ERR_OOM, "cudaMalloc of the workspace (" + std::to_string(want) + " bytes) failed");
@@ -825,6 +836,12 @@ rsim_status rsim_selftest_wait_timeout(rsim_ctx* ctx, uint64_t limit_ns, rsim_st
   cudaSetDevice(ctx->device);
   const cudaError_t e = launch_wait_selftest(ctx->status_dev, limit_ns, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "self-test kernel");
+  return RSIM_OK;
+}
+
+rsim_status rsim_selftest_alloc_limit(rsim_ctx* ctx, size_t bytes) {
+  if (!ctx) return fail(RSIM_ERR_INVALID_ARG, "ctx is NULL");
+  ctx->alloc_limit = bytes;
   return RSIM_OK;
 }
 

@@ -2,6 +2,7 @@
 // the API, the autotuner and the server sources.
 #pragma once
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <set>
@@ -21,6 +22,7 @@ struct rsim_ctx {
   void* ws = nullptr;
   size_t ws_bytes = 0;
   size_t ws_base = 0;  // what it would be without the FP32 tier's tensor-core form
+  std::atomic<size_t> alloc_limit{0};  // rsim_selftest_alloc_limit (0: none)
   // 256 bytes: word 0 is the status word of the context's own calls (rsim_sync_status);
   // word 32 is the shared-atomic probe's sink and word 33 the tensor-core probe's wait
   // failures (measure.cu); the rest is unused
@@ -56,6 +58,9 @@ rsim_plan reported_plan(int tier, const Consts& k, const rsim_plan& plan, int en
 int engine_tier(rsim_ctx* ctx, int tier, const Consts& k, int64_t P, size_t budget);
 size_t tensor_bytes_cap(size_t budget);
 size_t batch_bytes(const Consts& k, const int64_t* P, int F, const rsim_plan& plan, int tier);
+// cudaMalloc of a workspace, or on a stream cudaMallocAsync.
+cudaError_t workspace_malloc(const rsim_ctx* ctx, void** p, size_t bytes);
+cudaError_t workspace_malloc_async(const rsim_ctx* ctx, void** p, size_t bytes, cudaStream_t st);
 // `base`: the bytes without the FP32 tier's tensor-core form, where that is what takes `bytes`.
 rsim_status ensure_workspace(rsim_ctx* ctx, size_t bytes, cudaStream_t st, size_t base = SIZE_MAX);
 rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k,

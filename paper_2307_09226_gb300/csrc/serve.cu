@@ -225,7 +225,21 @@ bool admit_one(rsim_server* s) {
   r.t_admit = now;
   Slot& sl = s->slots[free_slot];
   cudaStream_t rs = sl.st[r.prio];
-  cudaError_t e = cudaMallocAsync(&r.ws, r.bytes, rs);
+  cudaError_t e = workspace_malloc_async(s->ctx, &r.ws, r.bytes, rs);
+  if (e != cudaSuccess && r.engine == kTierFp32Tensor) {
+    // no memory for the operand images: the FP32 tier's CUDA-core sum, if there is room for that
+    cudaGetLastError();
+    const int64_t P = r.r.pixels.P;
+    const rsim_plan plan = choose_plan(s->ctx, RSIM_TIER_FP32, r.k, P);
+    const size_t bytes = batch_bytes(r.k, &P, 1, plan, RSIM_TIER_FP32);
+    const size_t budget = s->opts.hbm_budget_bytes;
+    if (!budget || s->reserved + bytes <= budget) e = workspace_malloc_async(s->ctx, &r.ws, bytes, rs);
+    if (e == cudaSuccess) {
+      r.engine = RSIM_TIER_FP32;
+      r.plan = plan;
+      r.bytes = bytes;
+    }
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     r.result = RSIM_ERR_OOM;

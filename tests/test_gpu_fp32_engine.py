@@ -184,3 +184,32 @@ def test_staging_beyond_the_budget_stays_refused(env):
         c.synth_host(radar, host, "split_fp16")
     assert e.value.status == _abi.ERR_BUDGET
     c.close()
+
+
+def test_served_requests_without_memory_for_the_operand_images(env):
+    """A request whose operand images cannot be allocated runs as the CUDA-core sum; one of a
+    tier that has nothing else fails with OOM, and the server goes on."""
+    torch, _abi, device, _ = env
+    radar = Radar(M=2, N=4, Ns=64, L=64)
+    px = synth.random_frame(radar, 80, 60, seed=71, mask_frac=0.3)
+    tensor, direct = sizes(env, radar, px.P)
+    d = device.upload(px)
+    cubes = [torch.zeros((8, 64, 64), dtype=torch.complex64, device="cuda") for _ in range(3)]
+    c = device.Context(0)
+    srv = _abi.rsim_server_create(c.h, slots=2, hbm_budget_bytes=2 * tensor)
+    _abi.rsim_selftest_alloc_limit(c.h, tensor - 256)
+    tickets = [_abi.rsim_server_submit(srv, _abi.make_request(radar, d, tier, cube))
+               for tier, cube in zip((_abi.TIER_FP32, _abi.TIER_SPLIT_FP16, _abi.TIER_FP32), cubes)]
+    status = [_abi.rsim_server_wait(srv, t, -1) for t in tickets]
+    stats = _abi.rsim_server_stats_get(srv)
+    _abi.rsim_server_destroy(srv)
+    split = _abi.rsim_workspace_size(c.h, radar, px.P, _abi.TIER_SPLIT_FP16)
+    assert status == [_abi.OK, _abi.ERR_OOM if split > tensor - 256 else _abi.OK, _abi.OK]
+    assert stats.failed == (1 if split > tensor - 256 else 0)
+    assert stats.peak_reserved_bytes < 2 * tensor
+    ref = oracle.cube_separable(radar, px)
+    for cube in (cubes[0], cubes[2]):
+        assert oracle.rel_l2(cube.cpu().numpy(), ref) <= DIRECT_BAR
+    small = device.Context(0, hbm_budget_bytes=tensor - 256)
+    assert np.array_equal(cubes[0].cpu().numpy(), small.synth(radar, d, "fp32").cpu().numpy())
+    small.close(), c.close()
