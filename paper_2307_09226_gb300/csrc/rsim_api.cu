@@ -720,20 +720,21 @@ rsim_status rsim_synth_batch(rsim_ctx* ctx, const rsim_radar_params* params,
     const bool instead = ctx->ws_bytes < most && capturing(st) &&
                          batch_bytes(k, Ps.data(), F, choose_plan(ctx, tier, k, maxp), tier) <= ctx->ws_bytes;
     if (!instead) {
-      int done = 0;
-      for (int n : parts) {
-        const size_t bytes = batch_bytes(k, Ps.data() + done, n, tplan, engine);
-        // (the CUDA-core sum's need is worked out only where the workspace grows)
-        s = ensure_workspace(ctx, bytes, st, ctx->ws_bytes >= bytes ? 0 :
-                             batch_bytes(k, Ps.data(), F, choose_plan(ctx, tier, k, maxp), tier));
-        if (s == RSIM_ERR_OOM && done == 0) break;
-        if (s == RSIM_OK)
-          s = run_frames(ctx, (char*)ctx->ws, ctx->ws_bytes, k, frames + done, n, cubes + done, engine, out_dtype,
-                         tplan, ctx->status_dev, st);
-        if (s != RSIM_OK) return s;
-        done += n;
+      // room for the largest part before the first runs, so that the call cannot end half done
+      // (the CUDA-core sum's need is worked out only where the workspace grows)
+      s = ensure_workspace(ctx, most, st, ctx->ws_bytes >= most ? 0 :
+                           batch_bytes(k, Ps.data(), F, choose_plan(ctx, tier, k, maxp), tier));
+      if (s == RSIM_OK) {
+        int at = 0;
+        for (int n : parts) {
+          s = run_frames(ctx, (char*)ctx->ws, ctx->ws_bytes, k, frames + at, n, cubes + at, engine, out_dtype, tplan,
+                         ctx->status_dev, st);
+          if (s != RSIM_OK) return s;
+          at += n;
+        }
+        return RSIM_OK;
       }
-      if (done == F) return RSIM_OK;
+      if (s != RSIM_ERR_OOM) return s;
     }
   }
   const rsim_plan plan = choose_plan(ctx, tier, k, maxp);

@@ -213,3 +213,27 @@ def test_served_requests_without_memory_for_the_operand_images(env):
     small = device.Context(0, hbm_budget_bytes=tensor - 256)
     assert np.array_equal(cubes[0].cpu().numpy(), small.synth(radar, d, "fp32").cpu().numpy())
     small.close(), c.close()
+
+
+def test_a_batch_in_parts_without_memory_for_the_largest(env):
+    """A batch that goes in parts, the second of which cannot have its workspace: the whole batch
+    runs as the CUDA-core sum, instead of failing after the first part."""
+    torch, _abi, device, _ = env
+    radar = Radar(M=2, N=4, Ns=64, L=64)
+    frames = [synth.random_frame(radar, a, e, seed=81 + a, mask_frac=0.2) for a, e in ((25, 20), (80, 60))]
+    tensor, direct = sizes(env, radar, 4800)
+    c = device.Context(0, hbm_budget_bytes=tensor + 4096)
+    _abi.rsim_selftest_alloc_limit(c.h, tensor - 256)
+    pxs = [device.upload(f) for f in frames]
+    cubes = c.synth_batch(radar, pxs, "fp32")
+    assert c.sync_status() == _abi.OK
+    for f, cube in zip(frames, cubes):
+        assert oracle.rel_l2(cube.cpu().numpy(), oracle.cube_separable(radar, f)) <= DIRECT_BAR
+    _abi.rsim_selftest_alloc_limit(c.h, 0)
+    for f, px, cube in zip(frames, pxs, c.synth_batch(radar, pxs, "fp32")):
+        assert oracle.rel_l2(cube.cpu().numpy(), oracle.cube_separable(radar, f)) <= FP32_BAR
+    _abi.rsim_selftest_alloc_limit(c.h, 1)
+    with pytest.raises(_abi.RsimError) as e:  # a batch that nothing holds
+        c.synth_batch(radar, [device.upload(synth.random_frame(radar, 80, 60, seed=s)) for s in range(9)], "split_fp16")
+    assert e.value.status in (_abi.ERR_OOM, _abi.ERR_BUDGET)
+    c.close()
