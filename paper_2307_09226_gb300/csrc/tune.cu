@@ -139,9 +139,15 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
   Consts k;
   rsim_status s = check_params(params, &k);
   if (s != RSIM_OK) return s;
-  const int tier = engine_tier(ctx, asked, k, P, ctx->budget);  // the arithmetic that runs the shape
+  int tier = engine_tier(ctx, asked, k, P, ctx->budget);  // the arithmetic that runs the shape
   cudaSetDevice(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
+  bool short_of_memory = false;
+  if (tier == kTierFp32Tensor &&
+      ensure_workspace(ctx, batch_bytes(k, &P, 1, choose_plan(ctx, tier, k, P), tier), st, 0) == RSIM_ERR_OOM) {
+    tier = RSIM_TIER_FP32;  // what rsim_synth would run without that memory
+    short_of_memory = true;
+  }
 
   // synthetic pixels and an output buffer
   float* px = nullptr;
@@ -167,10 +173,14 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
     if (err != RSIM_OK || !plan_problem(tier, k, p).empty()) return 1e30f;
     int64_t PP = P;
     const size_t need = batch_bytes(k, &PP, 1, p, tier);
-    // candidates with more splits that pass the bound of the FP32 tier's tensor-core form, which
-    // the default plan keeps
+    // candidates with more splits that pass the bound of the FP32 tier's tensor-core form, or
+    // what memory there is, both of which the plan in use keeps
     if (tier == kTierFp32Tensor && need > tensor_bytes_cap(ctx->budget)) return 1e30f;
     rsim_status s2 = ensure_workspace(ctx, need, st, tier == kTierFp32Tensor ? 0 : need);
+    if (s2 == RSIM_ERR_OOM && (tier != asked || short_of_memory)) {
+      short_of_memory = true;
+      return 1e30f;
+    }
     if (s2 != RSIM_OK) {
       err = s2;
       return 1e30f;
@@ -254,6 +264,7 @@ extern "C" rsim_status rsim_autotune(rsim_ctx* ctx, const rsim_radar_params* par
       }
     }
   }
+  if (tb >= 1e30f && err == RSIM_OK && short_of_memory) err = RSIM_ERR_OOM;
   if (tb >= 1e30f && err == RSIM_OK) best = choose_plan(ctx, tier, k, P);  // no candidate fits: the plan in use
   best.tuned = 1;
   cudaEventDestroy(e0);

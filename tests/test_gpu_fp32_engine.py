@@ -237,3 +237,21 @@ def test_a_batch_in_parts_without_memory_for_the_largest(env):
         c.synth_batch(radar, [device.upload(synth.random_frame(radar, 80, 60, seed=s)) for s in range(9)], "split_fp16")
     assert e.value.status in (_abi.ERR_OOM, _abi.ERR_BUDGET)
     c.close()
+
+
+def test_tuning_without_memory_for_the_operand_images(env):
+    """Where the tensor-core form's workspace cannot be had, tuning tunes the CUDA-core sum that
+    calls then run; where only the larger candidates' cannot, it passes them over."""
+    torch, _abi, device, _ = env
+    radar, P = Radar(M=2, N=4, Ns=128, L=64), 4000
+    tensor, direct = sizes(env, radar, P)
+    for limit, form in ((tensor - 256, "direct"), (tensor + tensor // 8 + (1 << 20), "tensor")):
+        c = device.Context(0)
+        _abi.rsim_selftest_alloc_limit(c.h, limit)
+        plan = _abi.rsim_autotune(c.h, radar, P, _abi.TIER_FP32)
+        assert plan.tuned == 1 and (plan.grid > 0) == (form == "tensor")
+        px = synth.random_frame(radar, 80, 50, seed=91, mask_frac=0.2)
+        got = c.synth(radar, device.upload(px), "fp32").cpu().numpy()
+        assert c.sync_status() == _abi.OK
+        assert oracle.rel_l2(got, oracle.cube_separable(radar, px)) <= (FP32_BAR if form == "tensor" else DIRECT_BAR)
+        c.close()
