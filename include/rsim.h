@@ -391,7 +391,8 @@ rsim_status rsim_measure_mma_rate(rsim_ctx* ctx, double* flops_per_s, rsim_strea
  * of the contraction stage: the tensor-core contraction (after the operand builder),
  * the FP32 direct sum, or the NUFFT tier's spreading kernel (first frame of a batch).  The events
  * stand between the stages' kernels, so profiled calls do not overlap one stage's
- * launch with the previous stage's end.  rsim_profile_read waits for the recorded
+ * launch with the previous stage's end, and a profiled NUFFT batch compacts all its frames
+ * before the first is gridded (otherwise large frames are compacted on their own streams).  rsim_profile_read waits for the recorded
  * events, returns the summed stage times and launch counts since profiling was
  * switched on, and starts a new tally. */
 typedef struct {

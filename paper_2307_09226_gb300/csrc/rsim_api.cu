@@ -377,8 +377,9 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
   // NUFFT batches of large frames: every frame's compaction goes to the frame's own stream
   // (below), where its FP64 work runs beside other frames' spreading (64 walking frames -5%).
   // Small frames wait for the host's launches, of which that would be more (20 frames of V = 2
-  // and 65,536 pixels 381 -> 408 us)
-  const bool per_frame = tier == RSIM_TIER_NUFFT && nufft_slots(F) > 1 && nufft_geometry(k, mp).sorted;
+  // and 65,536 pixels 381 -> 408 us).  A profiled call compacts all frames first, so that the
+  // stage events stand between the stages
+  const bool per_frame = tier == RSIM_TIER_NUFFT && nufft_slots(F) > 1 && !prof && nufft_geometry(k, mp).sorted;
   if (!per_frame) {
     NvtxRange r(defer ? "compaction + slow-time phases" : "compaction + FP64 phases");
     int launched = 0;
@@ -428,10 +429,8 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
       cudaStream_t fs = S > 1 ? ctx->nu_st[f % S] : st;
       if (per_frame) {
         // the two-kernel form: a cooperative grid would wait for room beside the other streams
-        int launched = 0;
         le = launch_prep(k, table + f, nullptr, 1, frames[f].P, frames[f].dtype, false, false, status, nullptr, fs,
-                         false, &launched);
-        if (prof) ctx->prof_kernels += launched;
+                         false);
         if (le != cudaSuccess) break;
       }
       le = launch_nufft(k, table + f, frames[f].P, out_dtype, scratch + (size_t)(f % S) * slot, status, fs,

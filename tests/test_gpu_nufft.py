@@ -174,3 +174,29 @@ def test_batch_of_every_size_class_bitwise(ctx):
         assert np.array_equal(a, b)
     for a, b in zip(alone, small):
         assert np.array_equal(a, b)
+
+
+def test_stage_times_of_a_batch(ctx):
+    """The compaction of a batch of frames that are sorted counts as compaction: about as long
+    as that of its frames one by one, not nothing."""
+    radar = synth.Radar(M=2, N=4, Ns=64, L=32)
+    pxs = [device.upload(synth.random_frame(radar, 256, 210, seed=80 + i, mask_frac=0.2)) for i in range(6)]
+
+    def stages(call):
+        call()
+        _abi.rsim_profile_enable(ctx.h, True)
+        for _ in range(3):
+            call()
+        p = _abi.rsim_profile_read(ctx.h)
+        _abi.rsim_profile_enable(ctx.h, False)
+        return p
+
+    one = stages(lambda: ctx.synth(radar, pxs[0], "nufft"))
+    many = stages(lambda: ctx.synth_batch(radar, pxs, "nufft"))
+    # six frames' compaction in one launch: more than half of one frame's
+    assert many.prep_ms > 0.5 * one.prep_ms > 0
+    alone = [ctx.synth(radar, px, "nufft").cpu().numpy() for px in pxs]
+    _abi.rsim_profile_enable(ctx.h, True)
+    for a, b in zip(alone, ctx.synth_batch(radar, pxs, "nufft")):
+        assert np.array_equal(a, b.cpu().numpy())
+    _abi.rsim_profile_enable(ctx.h, False)
