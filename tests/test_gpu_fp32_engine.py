@@ -255,3 +255,50 @@ def test_tuning_without_memory_for_the_operand_images(env):
         assert c.sync_status() == _abi.OK
         assert oracle.rel_l2(got, oracle.cube_separable(radar, px)) <= (FP32_BAR if form == "tensor" else DIRECT_BAR)
         c.close()
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("V,Ns,L,n_az,n_el,splits,tile_n", [
+    (1, 128, 64, 256, 256, 8, 128),   # 65,536 pixels, whole tiles
+    (3, 70, 33, 251, 130, 4, 128),    # ragged rows, columns and pixels
+    (2, 200, 96, 120, 100, 7, 64),    # the narrower tile
+    (1, 64, 64, 90, 60, 1, 0),        # one split: written directly
+])
+def test_the_cuda_core_sum(env, dtype, V, Ns, L, n_az, n_el, splits, tile_n):
+    """The CUDA-core sum, pinned, at sizes that the tensor cores take by default: alone, written
+    as complex128, and as a batch of uneven valid counts with the same bits."""
+    torch, _abi, device, _ = env
+    radar = Radar(M=V, N=1, Ns=Ns, L=L)
+    frames = [synth.random_frame(radar, n_az, n_el, seed=41 + i, mask_frac=m, dtype=dtype) for i, m in enumerate((0.3, 0.0))]
+    c = device.Context(0)
+    _abi.rsim_set_plan(c.h, radar, frames[0].P, _abi.TIER_FP32, splits=splits, tile_n=tile_n)
+    pxs = [device.upload(f) for f in frames]
+    refs = [oracle.cube_separable(radar, f) for f in frames]
+    alone = [c.synth(radar, px, "fp32").cpu().numpy() for px in pxs]
+    for got, ref in zip(alone, refs):
+        assert oracle.rel_l2(got, ref) <= DIRECT_BAR
+    wide = c.synth(radar, pxs[0], "fp32", out_dtype="complex128").cpu().numpy()
+    assert np.array_equal(wide.astype(np.complex64), alone[0])
+    for got, want in zip(c.synth_batch(radar, pxs, "fp32"), alone):
+        assert np.array_equal(got.cpu().numpy(), want)
+    assert c.sync_status() == _abi.OK
+    c.close()
+
+
+def test_static_entry_falls_back_to_the_cuda_core_sum(env):
+    """80,000 pixels and 64 columns: 82 MB of operand images pass the static workspace, the
+    CUDA-core sum's scratch does not.  The result is that of a context whose budget leaves the
+    same sum, bit for bit."""
+    torch, _abi, device, _ = env
+    radar = Radar(M=1, N=1, Ns=64, L=64)
+    px = synth.random_frame(radar, 400, 200, seed=51, mask_frac=0.1)
+    tensor, direct = sizes(env, radar, px.P)
+    assert direct < 64 << 20 < tensor
+    d = device.upload(px)
+    cube = torch.empty((1, 64, 64), dtype=torch.complex64, device="cuda")
+    assert _abi.rsim_synth_static(radar, d, _abi.TIER_FP32, cube) == _abi.OK, _abi.last_error()
+    torch.cuda.synchronize()
+    small = device.Context(0, hbm_budget_bytes=tensor - 256)
+    assert np.array_equal(cube.cpu().numpy(), small.synth(radar, d, "fp32").cpu().numpy())
+    assert oracle.rel_l2(cube.cpu().numpy(), oracle.cube_separable(radar, px)) <= DIRECT_BAR
+    small.close()
