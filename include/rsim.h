@@ -194,8 +194,11 @@ rsim_status rsim_synth_host(rsim_ctx* ctx, const rsim_radar_params* params, cons
  * device counter, in the FP32 tier by a fixed stride).  An FP32-tier
  * batch whose operand images would pass 16 GiB or the context's budget goes in
  * sub-batches.  frames: HOST array of F descriptors; cubes: HOST array
- * of F device pointers, each laid out as in rsim_synth.  Each frame's result is
- * bit-identical to rsim_synth of that frame alone with the same tier.  The NUFFT tier
+ * of F device pointers, each laid out as in rsim_synth.  A batch takes the plan of its
+ * largest frame.  A frame's result is bit-identical to rsim_synth of that frame alone
+ * where that takes the same plan: frames of the largest one's pixel count do, and in the
+ * NUFFT tier all.  A smaller frame may alone take other splits and, below 128 pixels in
+ * the FP32 tier, the CUDA-core sum: the same sum in other roundings.  The NUFFT tier
  * runs the frames on up to eight streams of the context (each with its own grid
  * scratch), which wait for `stream` first; `stream` then waits for all of them, so the
  * call stays ordered on `stream` like every other.

@@ -302,3 +302,19 @@ def test_static_entry_falls_back_to_the_cuda_core_sum(env):
     assert np.array_equal(cube.cpu().numpy(), small.synth(radar, d, "fp32").cpu().numpy())
     assert oracle.rel_l2(cube.cpu().numpy(), oracle.cube_separable(radar, px)) <= DIRECT_BAR
     small.close()
+
+
+def test_uneven_batch_across_the_pixel_limit(env):
+    """A batch takes the form and the plan of its largest frame: frames of fewer than 128 pixels
+    run on the tensor cores there, on the CUDA cores alone.  Each within the tier's bar, and the
+    largest with the bits it has alone."""
+    torch, _abi, device, ctx = env
+    radar = Radar(M=2, N=2, Ns=64, L=24)
+    frames = [synth.random_frame(radar, a, e, seed=60 + i, mask_frac=0.0)
+              for i, (a, e) in enumerate([(5, 3), (16, 8), (1, 1), (127, 1), (60, 50), (43, 3)])]
+    pxs = [device.upload(f) for f in frames]
+    cubes = [x.cpu().numpy() for x in ctx.synth_batch(radar, pxs, "fp32")]
+    assert ctx.sync_status() == _abi.OK
+    for f, got in zip(frames, cubes):
+        assert oracle.rel_l2(got, oracle.cube_separable(radar, f)) <= DIRECT_BAR
+    assert np.array_equal(cubes[4], ctx.synth(radar, pxs[4], "fp32").cpu().numpy())
