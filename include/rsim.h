@@ -73,8 +73,9 @@ typedef enum {
 /* Arithmetic tier of the contraction over pixels. */
 typedef enum {
   RSIM_TIER_FP32 = 0,       /* FP32 accuracy (relative error below 1e-6 where measured).  From 128
-                               pixels on, tcgen05 with FP16 hi+lo operands (3 products) and FP32 sums
-                               of at most two 32-pixel chunks each; else, and wherever a plan of its
+                               pixels on, tcgen05 with FP16 hi+lo operands (3 products; 22 bits
+                               of strengths down to 2^-16 of the frame's strongest, 2^-40 of that
+                               below) and FP32 sums of at most two 32-pixel chunks each; else, and wherever a plan of its
                                own is pinned for the shape or the workspace bound holds no more, the
                                FP32 direct sum on CUDA cores */
   RSIM_TIER_BF16 = 1,       /* tcgen05 tensor cores, BF16 operands, FP32 accumulate */

@@ -398,7 +398,7 @@ umma_contract(const FrameIO* __restrict__ frames, Consts k, Geo g, int scaled, i
   fence_before();
   __syncthreads();
   fence_after();
-  wait_prior_grid();  // the set-up above overlaps the operand builder's last blocks
+  wait_prior_grid();  // the operand builder's writes are visible
   const uint32_t tmem = sh->tmem_base;
   const int64_t rows_total = (int64_t)k.V * k.Ns;
 

@@ -281,7 +281,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int out
   __syncthreads();
   cluster_sync();  // the peer's barriers exist
   fence_after();
-  wait_prior_grid();  // the set-up above overlaps the operand builder's last blocks
+  wait_prior_grid();  // the operand builder's writes are visible
   const uint32_t tmem = sh->tmem_base;
   const int64_t rows_total = (int64_t)k.V * k.Ns;
 

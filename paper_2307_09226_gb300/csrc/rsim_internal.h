@@ -111,8 +111,10 @@ constexpr size_t kFp32TensorBytes = size_t(16) << 30;
 // Tiers of hi + lo operands on one CTA per tile.
 inline bool split_tier(int tier) { return tier == RSIM_TIER_SPLIT_BF16 || tier == RSIM_TIER_SPLIT_FP16; }
 // Sigma scaling of the tiers with FP16 operands, 0 for none: max(|re|, |im|) is put into
-// [2^(n-2), 2^(n-1)).  The FP32 tier takes 16: every component stays below FP16's largest number
-// and pixels down to 2^-29 of the strongest keep all their bits.  The 16-bit tiers take 1: their
+// [2^(n-2), 2^(n-1)).  The FP32 tier takes 16: every component stays below FP16's largest number,
+// and components down to 2^-16 of the strongest keep the 22 bits of a hi + lo pair (1.2e-7);
+// weaker ones have an error of at most 2^-40 of the strongest, which FP32 sums at its size (2^-24)
+// do not resolve either.  The 16-bit tiers take 1: their
 // bars ask for no more, and the low parts' fewer set bits draw less power (split FP16 on 256 x
 // 256 pixels, V = 12, N_s = 256, L = 128: 230 us a contraction against 238 with 16).
 inline __host__ __device__ constexpr int sigma_scaling(int tier) {
@@ -147,9 +149,10 @@ cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int o
                          unsigned* status, cudaStream_t st, cudaEvent_t spread_begin = nullptr,
                          cudaEvent_t spread_end = nullptr);
 
-// Programmatic dependent launch: a kernel launched with launch_dependent may be
-// scheduled while the previous kernel in the stream drains its last blocks, hiding the
-// launch latency between the stages of one call.  Such a kernel executes
+// Programmatic dependent launch: a kernel launched with launch_dependent may start as soon as
+// every block of the previous kernel in the stream has exited, before that kernel's memory
+// flush, which hides the launch latency between the stages of one call (no kernel lets its
+// dependent start earlier: none executes griddepcontrol.launch_dependents).  Such a kernel executes
 // wait_prior_grid() before it touches anything the previous kernel writes; the wait
 // returns once that kernel has completed and its writes are visible (it is a no-op for
 // a kernel launched without the attribute).
