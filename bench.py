@@ -394,10 +394,11 @@ def run_gpu(args):
 
     if rank == 0:
         peaks, kind = _peaks()
-        # the FP32 tier runs three products on the tensor cores, like the split tiers
-        roof = _roofline("split_fp16" if tier == "fp32" else tier, prof.contract_ms - prof.operand_ms, prof.calls,
+        # the FP32 tier's tensor-core form runs three products, like the split tiers
+        pairs = tier == "fp32" and on_tensor_cores(ctx, radar, frame.pixels.P)
+        roof = _roofline("split_fp16" if pairs else tier, prof.contract_ms - prof.operand_ms, prof.calls,
                          samples, peaks, kind)
-        traffic = _load_traffic(tier)
+        traffic = _load_traffic(tier) if pairs or tier != "fp32" else None
         if traffic is not None:
             roof["traffic"] = traffic
         if roof.get("kernel") == "umma_contract":
@@ -407,10 +408,15 @@ def run_gpu(args):
             mma = _abi.rsim_measure_mma_rate(ctx.h) / 1e12
             roof["mma_rate_tflops"] = round(mma, 1)
             roof["executed_frac_of_mma_rate"] = round(roof["executed_tflops"] / mma, 4)
+            if pairs:
+                roof["kernel"] = "umma_contract_pairs"
         one_v, one_sample, _ = _cpu_one_core(frame)
         batch = run_batch(ctx, tier, steps=max(3, min(args.steps, 10)), warmup=3) if not args.no_extras else None
         serving = run_serving(ctx) if not args.no_extras else None
         raycast = run_raycast(ctx, tier) if not args.no_extras else None
+        direct = run_direct(local, frame, px, ref, args.steps, args.warmup) if not args.no_extras else None
+        if direct is not None:
+            direct["headline_tier_speedup"] = round(direct["ms_per_step"] / (step_ms / args.steps), 3)
         nufft = run_nufft(ctx, frame, px, ref, args.steps, args.warmup) if not args.no_extras else None
         if nufft is not None:
             nufft["speedup_vs_headline_tier"] = round(step_ms / args.steps / nufft["ms_per_step"], 3)
@@ -421,8 +427,8 @@ def run_gpu(args):
             "metric": "cube synth Gpath-samples/s at rel err<=2e-5 vs FP64",
             "value": value, "unit": "Gpath-samples/s", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": step_ms / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "f32" if tier == "fp32" else
-            ("fp16x2+f32acc" if tier == "split_fp16" else "bf16x2+f32acc"),
+            "scaling": "weak", "vs_baseline": None, "dtype": {"split_fp16": "fp16x2+f32acc", "split_bf16": "bf16x2+f32acc", "bf16": "bf16+f32acc",
+                      "fp16": "fp16+f32acc", "fp32": "fp16x2+f32acc" if pairs else "f32"}[tier],
             "data": "synthetic",
             "config": {"workload": frame.meta["workload"], "tier": tier, "P": radar and frame.pixels.P,
                        "plan": _abi.rsim_get_plan(ctx.h, radar, frame.pixels.P, _abi.TIERS[tier]).as_dict(),
@@ -448,6 +454,7 @@ def run_gpu(args):
             "batch": batch,
             "serving": serving,
             "raycast": raycast,
+            "fp32_direct": direct,
             "nufft": nufft,
         }
         print(json.dumps(line))
@@ -498,6 +505,49 @@ def ensure_tuned(ctx, radar, P, tier):
     from paper_2307_09226_gb300 import _abi
     if not _abi.rsim_get_plan(ctx.h, radar, P, _abi.TIERS[tier]).tuned:
         _abi.rsim_autotune(ctx.h, radar, P, _abi.TIERS[tier])
+
+
+def on_tensor_cores(ctx, radar, P):
+    """Whether the FP32 tier runs the shape on the tensor cores (its plan has a CTA count) or as
+    the CUDA-core direct sum."""
+    from paper_2307_09226_gb300 import _abi
+    return _abi.rsim_get_plan(ctx.h, radar, P, _abi.TIER_FP32).grid > 0
+
+
+def run_direct(device_index, frame, px, ref, steps, warmup):
+    """Config 2: the same frame through the plain FP32 direct sum on the CUDA cores (its plan
+    pinned, then tuned, in a context of its own), with its error and the FMA-pipe roofline."""
+    import torch
+    from paper_2307_09226_gb300 import _abi, device
+    radar, P = frame.radar, frame.pixels.P
+    samples = _valid_count(frame.pixels) * radar.V * radar.Ns * radar.L
+    ctx = device.Context(device_index)
+    _abi.rsim_set_plan(ctx.h, radar, P, _abi.TIER_FP32, splits=(P + 8191) // 8192)
+    _abi.rsim_autotune(ctx.h, radar, P, _abi.TIER_FP32)
+    cube = device.cube_tensor(radar)
+    flush = torch.empty(2 * L2_BYTES // 4, dtype=torch.float32, device="cuda")
+    ms = []
+    for i in range(warmup + steps):
+        flush.fill_(float(i))
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        ctx.synth(radar, px, "fp32", cube=cube)
+        b.record()
+        torch.cuda.synchronize()
+        ms.append(a.elapsed_time(b))
+    t = statistics.median(ms[warmup:])
+    _abi.rsim_profile_enable(ctx.h, True)
+    for _ in range(3):
+        ctx.synth(radar, px, "fp32", cube=cube)
+    prof = _abi.rsim_profile_read(ctx.h)
+    peaks, kind = _peaks()
+    plan = _abi.rsim_get_plan(ctx.h, radar, P, _abi.TIER_FP32).as_dict()
+    out = {"workload": frame.meta["workload"], "tier": "fp32, CUDA cores", "dtype": "f32", "plan": plan,
+           "ms_per_step": round(t, 4), "value": samples / (t * 1e-3) / 1e9, "unit": "Gpath-samples/s",
+           "rel_err": _rel_l2(cube.cpu().numpy(), ref), "steps": steps,
+           "roofline": _roofline("fp32", prof.main_ms, prof.calls, samples, peaks, kind)}
+    ctx.close()
+    return out
 
 
 def run_batch(ctx, tier, steps, warmup):
