@@ -417,15 +417,9 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int out
         if (lane == 0) mbar_arrive_at(&sh->acc_empty[gi & 1u], 0);
       }
       if (!alive) break;
-      // 2 (chunks - ngr) of the chunks were summed in groups of two
-      const float lost = kShort1 + (kShort2 - kShort1) * (2.f * (float)(chunks - min(ngr, chunks)) / (float)max(chunks, 1u));
-#pragma unroll
-      for (int b = 0; b < kBlocks; ++b)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          sre[b][i] = fmaf(sre[b][i], lost, sre[b][i]);
-          sim[b][i] = fmaf(sim[b][i], lost, sim[b][i]);
-        }
+      // (a group of one at the end of a unit of two-chunk groups: at most 2e-8 of its sums)
+      const float lost = xs->group > 1 ? kShort2 : kShort1;
+      auto whole = [lost](float x) { return fmaf(x, lost, x); };
       const int mt = xs->mt, nt = xs->nt;
       const FrameIO& fr = frames[xs->f];
       const int64_t gr = (int64_t)mt * 128 + r;
@@ -442,7 +436,7 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int out
             const int l = nt * g.NT + jb + i;
             if (l < k.L) {
               const int64_t o = gr * k.L + l;
-              const float re = sre[b][i] * oscale.x * oscale.y, im = sim[b][i] * oscale.x * oscale.y;
+              const float re = whole(sre[b][i]) * oscale.x * oscale.y, im = whole(sim[b][i]) * oscale.x * oscale.y;
               if (out_dtype == RSIM_C128)
                 reinterpret_cast<double2*>(fr.cube)[o] = make_double2((double)re, (double)im);
               else
@@ -463,7 +457,8 @@ umma_contract_pairs(const FrameIO* __restrict__ frames, Consts k, Geo g, int out
 #pragma unroll
           for (int i = 0; i < 8; i += 2)
             st_hint_v4(t4 + ((jb + i) >> 1) * 128,
-                       make_float4(sre[b][i], sim[b][i], sre[b][i + 1], sim[b][i + 1]), pol_p);
+                       make_float4(whole(sre[b][i]), whole(sim[b][i]), whole(sre[b][i + 1]), whole(sim[b][i + 1])),
+                       pol_p);
         }
       }
       __syncwarp();

@@ -13,10 +13,11 @@ namespace {
 // FP16 operands, three products, at most kFp32Group chunks in an accumulator, FP32 sums of
 // those.  At every shape measured it is closer to FP64 than the FP32 sum on the CUDA cores
 // and faster (relative error and time, tensor / CUDA cores):
-//   512 x 512 pixels, V = 8,  N_s = 512, L = 256   6.7e-7 / 1.77e-6   2583 / 29370 us
-//   256 x 256,        V = 12, N_s = 256, L = 128   5.6e-7 / 1.27e-6    277 / 2806 us
-//   128 x 128,        V = 8,  N_s = 256, L = 128   3.5e-7 / 6.6e-7      81 / 489 us
-//   32 x 32,          V = 8,  N_s = 64,  L = 32    3.3e-7 / 4.7e-7      31 / 57 us
+//   512 x 512 pixels, V = 8,  N_s = 512, L = 256   5.4e-7 / 1.79e-6   2517 / 29280 us
+//   256 x 256,        V = 12, N_s = 256, L = 128   4.1e-7 / 1.29e-6    272 / 2816 us
+//   128 x 128,        V = 8,  N_s = 256, L = 128   3.1e-7 / 6.8e-7      81 / 492 us
+//   32 x 32,          V = 8,  N_s = 64,  L = 32    2.8e-7 / 4.8e-7      39 / 73 us
+//   16 x 8,           V = 2,  N_s = 64,  L = 16    2.8e-7 / 3.6e-7      31 / 42 us
 // Frames of a few chunks take as long either way (5 x 3 pixels: 25-29 / 26 us).
 constexpr int kFp32Group = 2;
 constexpr int64_t kFp32TensorPixels = 128;
