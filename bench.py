@@ -216,6 +216,16 @@ def _roofline(tier, prof_contract_ms, launches, samples, peaks, peak_kind):
             "peak_source": f"bf16 dense burst ({peak_kind})"}
 
 
+def _issue_roofline(warp_insts, kernel_ms, clk_mhz):
+    """Roofline of a kernel bound by instruction issue: its warp instructions over its time
+    against one per scheduler (four an SM, 152 SMs) and clock."""
+    achieved = warp_insts / (kernel_ms * 1e-3) / 1e12
+    peak = 152 * 4 * clk_mhz * 1e6 / 1e12
+    return {"bound": "issue", "kernel": "nu_spread", "achieved": round(achieved, 4), "peak": round(peak, 4),
+            "unit": "T warp-inst/s", "frac": round(achieved / peak, 4), "kernel_ms": round(kernel_ms, 5),
+            "peak_source": f"152 SM x 4 schedulers x {clk_mhz:.0f} MHz"}
+
+
 def _cpu_sample(frame, target_s=12.0):
     """Time the CPU oracle on a bounded sample of the frame: whole channels of the full
     pixel set, as many as fit in ~target_s seconds."""
@@ -635,26 +645,15 @@ def run_nufft(ctx, frame, px, ref, steps, warmup):
     _abi.rsim_profile_enable(ctx.h, False)
     samples = pv * radar.V * radar.Ns * radar.L
     t = sum(ms) / len(ms)
-    # spreading (the dominant kernel): 49 taps x (re, im) x two words = 196 shared atomic
-    # lane-operations per (channel, point) record (the kernel issues fewer: it sums the taps
-    # of successive points of one cell in registers first), against the rate this device performs
-    # such atomics (measured by the library's probe on the same GPU), with the derived
-    # one-wavefront-per-clock figure beside it
+    # spreading (the dominant kernel) is bound by the issue of its instructions: 56.6 warp
+    # instructions per (channel, point) record, counted by ncu on this frame
+    # (profiles/nufft_frame256x256.md), against one per scheduler and clock; beside it the rate
+    # of this device's shared-memory atomics, which the kernel uses for every run of points in
+    # one cell (measured by the library's probe on the same GPU)
     spread_ms = prof.main_ms / prof.calls
-    lane_ops = 196.0 * radar.V * pv
     peaks, _ = _peaks()
-    clk = peaks.get("sm_max_mhz", 2070.0)
-    derived = 152 * 32 * clk * 1e6 / 1e12
-    measured = _abi.rsim_measure_smem_atomics(ctx.h) / 1e12
-    achieved = lane_ops / (spread_ms * 1e-3) / 1e12
-    roof = {"bound": "smem", "kernel": "nu_spread", "achieved": round(achieved, 3), "peak": round(measured, 3),
-            "unit": "T lane-op/s", "frac": round(achieved / measured, 4), "kernel_ms": round(spread_ms, 5),
-            "peak_source": "measured: non-returning conflict-free 32-bit shared atomics at the spreading "
-                           "kernel's occupancy (rsim_measure_smem_atomics, this GPU)",
-            "derived_peak": round(derived, 3), "frac_of_derived": round(achieved / derived, 4),
-            "derived_source": f"one 32-lane wavefront per clock: 152 SM x 32 lanes x {clk:.0f} MHz",
-            "algorithmic": "196 shared atomic lane-operations per (channel, point) record, before runs of "
-                           "points in one cell are summed in registers"}
+    roof = _issue_roofline(56.6 * radar.V * pv, spread_ms, peaks.get("sm_max_mhz", 2070.0))
+    roof["smem_atomic_rate_t_lane_ops"] = round(_abi.rsim_measure_smem_atomics(ctx.h) / 1e12, 3)
     # the accuracy each gridding kernel width buys, and its time (the same frame)
     from dataclasses import replace as _replace
     widths = {}

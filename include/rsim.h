@@ -369,10 +369,11 @@ rsim_status rsim_selftest_alloc_limit(rsim_ctx* ctx, size_t bytes);
 
 /* Measurement helper for benchmarks (no counterpart in the paper): the rate, in lane
  * operations per second, at which this device performs non-returning 32-bit integer
- * atomic additions to shared memory without bank conflicts, at the NUFFT spreading
- * kernel's occupancy and access pattern.  The spreading kernel puts its taps into shared
- * memory with such atomics, so the rate is its roofline denominator.  Runs a probe kernel six times on `stream` (the first
- * as a warm-up) and returns the best; synchronous.  Allocates nothing.
+ * atomic additions to shared memory without bank conflicts, in the access pattern of the
+ * NUFFT spreading kernel, which puts every run of points in one cell into shared memory with
+ * such atomics (its own bound is the issue of its instructions).  Runs a probe kernel six
+ * times on `stream` (the first as a warm-up) and returns the best; synchronous.  Allocates
+ * nothing.
  * Errors: INVALID_ARG, CUDA. */
 rsim_status rsim_measure_smem_atomics(rsim_ctx* ctx, double* lane_ops_per_s, rsim_stream stream);
 

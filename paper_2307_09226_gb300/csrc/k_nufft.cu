@@ -49,8 +49,8 @@
 // channels: a frame of 256 x 256 pixels 99.3 -> 93.6 us, 64 walking frames 2956 -> 2487 us, the
 // same bits.  Before, every (channel, pixel) was binned as a 16-byte record (21 us of the
 // frame's time, now 18 with the sort), each tap went to the tile by atomics of its own, and the
-// whole grid was cleared.  The spreading (45 us, 68% of the issue slots) is bound by its
-// instructions, 57 a pixel and channel.  Not kept: 64-bit register sums by wide multiply-adds
+// whole grid was cleared.  The spreading (45-47 us, 70% of the issue slots while active, the
+// shared-memory pipe at 36%) is bound by its instructions, 56.6 a pixel and channel.  Not kept: 64-bit register sums by wide multiply-adds
 // (56 us), three blocks of 40 registers per SM (59 us), items of 2048 or 4096 pixels (frame
 // +7 and +15 us, the 64 frames -4 and -7%).
 #include <math.h>

@@ -1,12 +1,12 @@
 // Measured peaks of the units that two kernels lean on, taken on the device the library
-// runs on (the roofline denominators the benchmarks report beside vendor-library figures).
+// runs on (the benchmarks report them beside vendor-library figures).
 //
 // 1. The NUFFT tier's spreading kernel: non-returning
 // 32-bit integer atomic additions to shared memory without bank conflicts.  The
 // spreading kernel adds the taps of every run of points in one cell with such atomics
-// (two words per component, see k_nufft.cu), so this rate, taken on the device the
-// library runs on, is the roofline denominator of that kernel.  The probe has four blocks
-// of 256 threads per SM and the spreading kernel's access pattern: each atomic
+// (two words per component, see k_nufft.cu); it is bound by the issue of its instructions
+// (profiles/nufft_frame256x256.md), this rate says how far the atomics are from that.  The
+// probe has four blocks of 256 threads per SM and the spreading kernel's access pattern: each atomic
 // instruction of a warp touches 32 consecutive words, one per bank, of one of four word
 // arrays.
 //

@@ -60,3 +60,11 @@ def test_traffic_lookup_follows_the_kernel_source(tmp_path, monkeypatch):
     assert bench._load_traffic("split_fp16") is None
     os.remove(tmp_path / "profiles" / "traffic.txt")
     assert bench._load_traffic("split_fp16") is None
+
+
+def test_roofline_of_the_spreading_counts_issued_instructions():
+    """31.2 M warp instructions in 0.0471 ms are 0.6626 T/s, of 152 x 4 x 2.07 GHz = 1.2586 T/s."""
+    r = bench._issue_roofline(31.21e6, 0.0471, 2070.0)
+    assert r["bound"] == "issue" and r["kernel"] == "nu_spread"
+    assert r["achieved"] == pytest.approx(0.6626, abs=1e-4) and r["peak"] == pytest.approx(1.2586, abs=1e-4)
+    assert r["frac"] == pytest.approx(0.6626 / 1.2586, abs=1e-4)
