@@ -150,3 +150,14 @@ def test_sides_as_long_as_an_int_holds(ctx, wide):
         assert not bool(torch.isnan(out[k]).any())
     del out
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n_az,n_el", [(65, 70), (40, 33), (9, 33), (161, 31), (37, 1)])
+def test_widths_that_pad_their_tiles(ctx, n_az, n_el):
+    """Widths whose last tile would be mostly padding take narrower and higher tiles: as above."""
+    scene = synth.random_scene(seed=17, n_prims=12)
+    got = _host(ctx.raycast(scene, n_az, n_el, FOV, dtype=torch.float64))
+    want = rc.raycast(scene, n_az, n_el, *FOV)
+    np.testing.assert_array_equal(got["az"], want["az"])
+    np.testing.assert_array_equal(got["el"], want["el"])
+    _compare(scene, got, want, 1e-11, 1e-9, 1e-9, max_ambiguous=0.03)
