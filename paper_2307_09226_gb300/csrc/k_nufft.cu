@@ -365,13 +365,13 @@ __global__ void __launch_bounds__(kBinThreads) nu_bin_fill(const FrameIO* __rest
       if (((gx - tx * g.Tx + halo) & (g.Gx - 1)) < min(g.Gx, g.Tx + 2 * halo)) hit |= count[grp * nb + e] != 0;
     }
     hit = __syncthreads_or(hit);
-    for (int v = grp * g.gch; v < min(g.V, (grp + 1) * g.gch); ++v) {
-      const int64_t row = (int64_t)v * g.Gx + gx;
-      if (threadIdx.x == 0) row_used[row] = hit;
-      if (hit)
-        for (int y = threadIdx.x; y < g.Gy; y += blockDim.x)
-          reinterpret_cast<ulonglong2*>(grid)[row * g.Gy + y] = make_ulonglong2(0ull, 0ull);
-    }
+    // the group's channels side by side: rows shorter than the block share it
+    const int v0 = grp * g.gch, nv = min(g.V - v0, g.gch);
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) row_used[(int64_t)(v0 + i) * g.Gx + gx] = hit;
+    if (hit)
+      for (int e = threadIdx.x; e < nv * g.Gy; e += blockDim.x)
+        reinterpret_cast<ulonglong2*>(grid)[((int64_t)(v0 + e / g.Gy) * g.Gx + gx) * g.Gy + e % g.Gy] =
+            make_ulonglong2(0ull, 0ull);
     return;
   }
   const int grp = block / fill_blocks, v = grp * g.gch;

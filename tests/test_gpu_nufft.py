@@ -200,3 +200,17 @@ def test_stage_times_of_a_batch(ctx):
     for a, b in zip(alone, ctx.synth_batch(radar, pxs, "nufft")):
         assert np.array_equal(a, b.cpu().numpy())
     _abi.rsim_profile_enable(ctx.h, False)
+
+
+@pytest.mark.parametrize("Ns,L,V", [(1024, 8, 24), (512, 12, 40), (64, 4, 12)])
+def test_short_grid_rows_share_a_block(ctx, Ns, L, V):
+    """Grid rows of 16 and 32 cells, of which a block clears several channels' side by side, in
+    one channel group and in several; a frame of another scene leaves its cells in the scratch
+    before.  Against the CPU reference (bar as above, 5e-6)."""
+    radar = synth.Radar(M=V, N=1, Ns=Ns, L=L)
+    px = synth.random_frame(radar, 30, 20, seed=Ns, mask_frac=0.1, r_lo=0.5, r_hi=8.0)
+    other = synth.random_frame(radar, 60, 50, seed=Ns + 1, r_lo=3.0, r_hi=40.0)
+    ctx.synth(radar, device.upload(other), "nufft")
+    got = ctx.synth(radar, device.upload(px), "nufft").cpu().numpy()
+    assert ctx.sync_status() == _abi.OK
+    assert oracle.rel_l2(got, nu.cube_nufft(radar, px, w=7)) <= 5e-6
