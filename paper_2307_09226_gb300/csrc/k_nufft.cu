@@ -70,9 +70,12 @@ constexpr int kNQuad = 128;                 // midpoint nodes for Psi
 constexpr int kSpreadChunk = 1024;          // pixels per spreading work item, or half as many
 constexpr int kSortChunk = 8192;            // pixels a block sorts (whole spreading items)
 constexpr int kSortThreads = 1024;
-constexpr int kSortFrom = 12288;            // frames that are sorted have this many pixels and
-constexpr int64_t kSortWork = 400000;       // this many (channel, pixel) pairs (see nufft_geometry)
-constexpr int64_t kLongWork = 300000;       // pairs from which spreading items are kSpreadChunk long
+// Frames that are sorted have kSortFrom pixels and kSortWork (pixel, channel of a group) pairs,
+// in batches of fewer than kSortBatch frames kSortWorkFew; items are kSpreadChunk long from
+// kLongWork pairs on, in any batch from kLongWorkBatch (see nufft_geometry).
+constexpr int kSortFrom = 12288, kSortBatch = 8;
+constexpr int64_t kSortWork = 400000, kSortWorkFew = 700000;
+constexpr int64_t kLongWork = 300000, kLongWorkBatch = 200000;
 constexpr int kSub = 4;                     // sort keys per cell: the quarter along x
 static_assert(kSortChunk % kSpreadChunk == 0 && kSortChunk % kSortThreads == 0, "sorting items");
 constexpr int kBinThreads = 256;            // binning blocks: one group, kBinItems pixels
@@ -994,7 +997,7 @@ NuScratch nufft_layout(const NuGeo& g, const FftPlan& plx, const FftPlan& ply, c
 
 }  // namespace
 
-NuGeo nufft_geometry(const Consts& k, int64_t P) {
+NuGeo nufft_geometry(const Consts& k, int64_t P, int F) {
   NuGeo g{};
   g.V = k.V;
   g.Ns = k.Ns;
@@ -1014,18 +1017,27 @@ NuGeo nufft_geometry(const Consts& k, int64_t P) {
   const double cells = fabs(k.k_da) * g.Gx;
   g.gch = cells * (k.V - 1) <= 0.9 ? k.V : std::max(1, (int)(0.9 / cells) + 1);
   g.groups = (k.V + g.gch - 1) / g.gch;
-  // A frame is sorted where its channels repay the sort (a launch and some 5 us), and takes
-  // the longer spreading items where there are units enough for every CTA.  Time of a frame
-  // with 1024 pixels sorted / 1024 / 512 an item (V x pixels): 12 x 262,144 204 / 228 / 240 us,
-  // 12 x 65,536 90 / 90 / 95, 24 x 16,384 66 / 66 / 66, 12 x 28,145 64 / 60 / 62, 4 x 65,536
-  // 70 / 66 / 62, 1 x 65,536 62 / 56 / 50, 2 x 14,619 56 / 50 / 44
-  const int64_t work = (int64_t)k.V * g.P;
-  g.sorted = g.P >= kSortFrom && work >= kSortWork;
-  g.chunk = work >= kLongWork ? kSpreadChunk : kSpreadChunk / 2;
+  // A frame is sorted where the channels that share the order repay it (a launch and some 5 us),
+  // and takes the longer spreading items where there are units enough for every CTA; beside other
+  // frames of a batch the SMs are full, so items are longer earlier, and the sort pays in batches
+  // of kSortBatch frames and more.  Microseconds with 512-pixel items unsorted / 1024 unsorted /
+  // 1024 sorted (V x pixels, of which 30% are background; N_s 256, L 128):
+  //   one frame: 12 x 19,881 64 / 62 / 66, 12 x 40,000 86 / 82 / 83, 12 x 65,536 103 / 105 / 102,
+  //   12 x 99,856 132 / 126 / 120, 4 x 94,864 77 / 74 / 77, 4 x 119,716 86 / 89 / 90, 4 x 199,809
+  //   113 / 107 / 108, 24 x 26,896 106 / 99 / 100 (between 300 and 700 thousand pairs which is
+  //   best follows how the units fill the CTAs, within 8%);
+  //   frames of a batch: 40 of 4 x 65,536 1256 / 1185 / 1142, 40 of 12 x 26,896 1513 / 1436 / 1500,
+  //   4 of 12 x 52,900 277 / 256 / 272, 12 of 12 x 57,840 801 / 748 / 741, 40 of 12 x 57,840
+  //   2552 / 2367 / 2300.
+  // Channels far apart (gch below V) share less: 12 x 65,536 at 400 wavelengths, w = 4, 103 / 101
+  // / 115
+  const int64_t work = (int64_t)g.gch * g.P;
+  g.sorted = g.P >= kSortFrom && work >= (F > 1 && F < kSortBatch ? kSortWorkFew : kSortWork);
+  g.chunk = work >= (F > 1 ? kLongWorkBatch : kLongWork) ? kSpreadChunk : kSpreadChunk / 2;
   return g;
 }
 
-int nufft_kernels(const Consts& k, int64_t P) { return nufft_geometry(k, P).sorted ? 6 : 5; }
+int nufft_kernels(const Consts& k, int64_t P, int F) { return nufft_geometry(k, P, F).sorted ? 6 : 5; }
 
 bool nufft_supported(const Consts& k) {
   // FFT lengths up to 4096 in one CTA's shared memory, at least 8 cells per axis, and a
@@ -1035,13 +1047,13 @@ bool nufft_supported(const Consts& k) {
 }
 
 size_t nufft_scratch_bytes(const Consts& k, int64_t P) {
-  const NuGeo g = nufft_geometry(k, P);
+  const NuGeo g = nufft_geometry(k, P, 1);
   return nufft_layout(g, fft_plan(g.Gx), fft_plan(g.Gy), nullptr).total;
 }
 
-cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int out_dtype, char* scratch,
+cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int F, int out_dtype, char* scratch,
                          unsigned* status, cudaStream_t st, cudaEvent_t spread_begin, cudaEvent_t spread_end) {
-  const NuGeo g = nufft_geometry(k, P);
+  const NuGeo g = nufft_geometry(k, P, F);
   const int nb = g.ntx * g.nty;
   const int nbins = g.groups * nb;
   const FftPlan plx = fft_plan(g.Gx), ply = fft_plan(g.Gy);

@@ -19,7 +19,10 @@ namespace {
 //   128 x 128,        V = 8,  N_s = 256, L = 128   3.1e-7 / 6.8e-7      81 / 492 us
 //   32 x 32,          V = 8,  N_s = 64,  L = 32    2.8e-7 / 4.8e-7      39 / 73 us
 //   16 x 8,           V = 2,  N_s = 64,  L = 16    2.8e-7 / 3.6e-7      31 / 42 us
-// Frames of a few chunks take as long either way (5 x 3 pixels: 25-29 / 26 us).
+// Frames of a few chunks take as long either way (5 x 3 pixels: 25-29 / 26 us).  With 0 to 30%
+// of background every one of 118 frames from 128 pixels on was as fast or faster (0.99 to 2.3
+// times); with 90% the CUDA-core sum's fewer launches win below some 10,000 pixels (25 / 35 us),
+// but the valid count is not known when the form is chosen.
 constexpr int kFp32Group = 2;
 constexpr int64_t kFp32TensorPixels = 128;
 }  // namespace

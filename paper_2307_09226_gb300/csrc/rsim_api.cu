@@ -365,7 +365,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
     // split reduction (1 when the partial buffer is used)
     const bool tensor = tensor_tier(tier);
     if (tier == RSIM_TIER_NUFFT) {
-      for (int f = 0; f < F; ++f) ctx->prof_kernels += nufft_kernels(k, frames[f].P);
+      for (int f = 0; f < F; ++f) ctx->prof_kernels += nufft_kernels(k, frames[f].P, F);
     } else {
       ctx->prof_kernels += (tensor ? 1 + (mp > 0 ? 1 : 0) + (F > 1 ? 1 : 0) : 1) + (use_partial ? 1 : 0);
     }
@@ -379,7 +379,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
   // Small frames wait for the host's launches, of which that would be more (20 frames of V = 2
   // and 65,536 pixels 381 -> 408 us).  A profiled call compacts all frames first, so that the
   // stage events stand between the stages
-  const bool per_frame = tier == RSIM_TIER_NUFFT && nufft_slots(F) > 1 && !prof && nufft_geometry(k, mp).sorted;
+  const bool per_frame = tier == RSIM_TIER_NUFFT && nufft_slots(F) > 1 && !prof && nufft_geometry(k, mp, F).sorted;
   if (!per_frame) {
     NvtxRange r(defer ? "compaction + slow-time phases" : "compaction + FP64 phases");
     int launched = 0;
@@ -433,7 +433,7 @@ rsim_status run_frames(rsim_ctx* ctx, char* ws, size_t ws_bytes, const Consts& k
                          false);
         if (le != cudaSuccess) break;
       }
-      le = launch_nufft(k, table + f, frames[f].P, out_dtype, scratch + (size_t)(f % S) * slot, status, fs,
+      le = launch_nufft(k, table + f, frames[f].P, F, out_dtype, scratch + (size_t)(f % S) * slot, status, fs,
                         prof && f == 0 ? ev[4] : nullptr, prof && f == 0 ? ev[5] : nullptr);
     }
     // the join also follows a failed launch, so that nothing of this call runs on after it

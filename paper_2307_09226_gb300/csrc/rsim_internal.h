@@ -136,16 +136,17 @@ struct NuGeo {
   float beta;     // its shape parameter, 2.30 W
   int gch, groups;  // channels sorted together, and such groups
 };
-// Kernels launch_nufft starts for a frame of P pixels (binning with the tables and the scan,
-// fill, sort in larger frames (see nufft_geometry), spreading, two FFT passes).
-int nufft_kernels(const Consts& k, int64_t P);
-NuGeo nufft_geometry(const Consts& k, int64_t P);
+// Kernels launch_nufft starts for a frame of P pixels, one of a call of F frames (binning with
+// the tables and the scan, fill, sort in larger frames (see nufft_geometry), spreading, two FFT
+// passes).
+int nufft_kernels(const Consts& k, int64_t P, int F);
+NuGeo nufft_geometry(const Consts& k, int64_t P, int F);
 bool nufft_supported(const Consts& k);
 size_t nufft_scratch_bytes(const Consts& k, int64_t P);
-// One frame (`frame`: device pointer to its table entry, P: its pixel count), using
+// One frame of a call of F (`frame`: device pointer to its table entry, P: its pixel count), using
 // nufft_scratch_bytes(k, P) bytes of scratch; a copy that times out sets kStatusTimeout in
 // `status`.  Non-null events are recorded just before and after the spreading kernel.
-cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int out_dtype, char* scratch,
+cudaError_t launch_nufft(const Consts& k, const FrameIO* frame, int64_t P, int F, int out_dtype, char* scratch,
                          unsigned* status, cudaStream_t st, cudaEvent_t spread_begin = nullptr,
                          cudaEvent_t spread_end = nullptr);
 

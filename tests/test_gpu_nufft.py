@@ -214,3 +214,22 @@ def test_short_grid_rows_share_a_block(ctx, Ns, L, V):
     got = ctx.synth(radar, device.upload(px), "nufft").cpu().numpy()
     assert ctx.sync_status() == _abi.OK
     assert oracle.rel_l2(got, nu.cube_nufft(radar, px, w=7)) <= 5e-6
+
+
+def test_frames_at_the_size_rules_bitwise(ctx):
+    """Eight channels of pixel counts around the sizes from which a frame takes longer items (37,500
+    alone, 25,000 in a batch) and is sorted (50,000 alone and in larger batches, 87,500 in batches
+    of few frames): every frame's bits are the same alone and in batches of either kind, also with
+    channels too far apart to share an order."""
+    for d_rx in (0.5, 400.0):
+        radar = synth.Radar(M=2, N=4, Ns=64, L=32, d_rx=d_rx * 3.9e-3)
+        sizes = [(350, 250), (350, 249), (200, 125), (200, 124), (250, 150), (250, 199), (250, 200), (250, 149), (128, 96), (128, 95)]
+        pxs = [device.upload(synth.random_frame(radar, a, e, seed=90 + i, mask_frac=0.2)) for i, (a, e) in enumerate(sizes)]
+        alone = [ctx.synth(radar, px, "nufft").cpu().numpy() for px in pxs]
+        many = [c.cpu().numpy() for c in ctx.synth_batch(radar, pxs, "nufft")]
+        few = [c.cpu().numpy() for i in (0, 5) for c in ctx.synth_batch(radar, pxs[i:i + 5], "nufft")]
+        assert ctx.sync_status() == _abi.OK
+        for a, b, c in zip(alone, many, few):
+            assert np.array_equal(a, b) and np.array_equal(a, c)
+    got = alone[5]
+    assert oracle.rel_l2(got, oracle.cube_separable(radar, synth.random_frame(radar, 250, 199, seed=95, mask_frac=0.2))) <= 2e-5
