@@ -403,7 +403,7 @@ int rc_tile_width(int n_az) {
   int w = 1;
   while (w < 32 && w < n_az) w *= 2;
   auto padded = [n_az](int64_t x) { return (n_az + x - 1) / x * x; };
-  while (w > 8 && padded(w) > n_az + n_az / 8 && padded(w / 2) < padded(w)) w /= 2;
+  while (w > 8 && padded(w) > (int64_t)n_az + n_az / 8 && padded(w / 2) < padded(w)) w /= 2;
   return w;
 }
 
